@@ -1332,9 +1332,9 @@ static void run_blocks_win(Run &R, std::vector<int32_t> sources, const std::vect
         w.seg_hi = seg_start[sg + 1];
         w.src_lo = lo;
         w.src_hi = hi + 1;
-        // storage: every row hop L + 1 may read (the neighbours of hop L's window)
+        // storage: the widest window's rows and their neighbours
         int32_t a, e;
-        window_rows(w, beta, w.L + 1, &a, &e);
+        window_rows(w, beta, (w.L + 1) / 2 + 1, &a, &e);
         w.base = a;
         w.rows = e - a;
         const auto &H = g->h_heavy_ids;
@@ -1451,7 +1451,7 @@ static void run_blocks_win(Run &R, std::vector<int32_t> sources, const std::vect
             for (size_t b = b0; b < b0 + active; ++b) {
                 if (blocks[b].w.L < ell) continue;
                 int32_t lo, hi;
-                window_rows(blocks[b].w, beta, ell, &lo, &hi);
+                window_rows(blocks[b].w, beta, window_reach(blocks[b].w.L, ell), &lo, &hi);
                 heavy_max = std::max(heavy_max, blocks[b].w.heavy_cnt);
                 rows_max = std::max<int64_t>(rows_max, hi - lo);
                 hop_bytes += 4.0 * (hrp[hi] - hrp[lo]) + 4.0 * (hi - lo + 1) +
@@ -1749,14 +1749,14 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     g->acc_t1.reserve(nnz);
     g->acc_t2.reserve(nnz);
     // windowed blocks (the frontier as an interval) when the graph's bandwidth
-    // keeps a block's last window under half the graph, or when asked for
+    // keeps a block's widest window under half the graph, or when asked for
     const int32_t beta = ensure_bandwidth(g);
     // the longest run of the first pass (a learned length's cap is reached only by extensions,
     // which rerun few sources; the windows and the launch shape are chosen for the first pass)
     const int32_t Lmax = (len.empty() ? 0 : *std::max_element(len.begin(), len.end())) + (record_after ? 2 : 0);
     const bool use_win = !plus && o.rows_split != -1 && !(o.flags & SC_OPT_WINDOWS_OFF) &&
                          ((o.flags & SC_OPT_WINDOWS_FORCE) ||
-                          2.0 * (Lmax + 1.0) * static_cast<double>(beta) + 128.0 < 0.5 * static_cast<double>(n));
+                          2.0 * (Lmax / 2 + 2.0) * static_cast<double>(beta) + 128.0 < 0.5 * static_cast<double>(n));
     // a bf16 run whose early hops are fp32 is tuned (and its buffers sized) in fp32
     const int32_t h0 = bf16_first_hop(o);
     const int tune_prec = (o.precision == SC_PREC_BF16 && h0 > 1) ? SC_PREC_FP32 : o.precision;

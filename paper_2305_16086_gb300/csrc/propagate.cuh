@@ -90,11 +90,18 @@ struct GatherRec {
 // The rows one slice of a launch covers (the frontier of Algorithm 2, which
 // only visits nodes with p_{l-1} > 0, kept as an interval). The slice stores
 // rows [base, base + rows) at element offset xoff of the block buffer; hop l
-// computes rows [lo_l, hi_l) = [max(seg_lo, src_lo - l beta), min(seg_hi,
-// src_hi + l beta)) with beta the graph's bandwidth (beta = 0: the whole
-// segment). A segment is one graph of a batch (or the whole graph). The
-// support of X_l lies in [lo_l, hi_l) and rows outside it stay zero, so the
-// result is the one of the full hop.
+// computes rows [lo_l, hi_l) = [max(seg_lo, src_lo - r beta), min(seg_hi,
+// src_hi + r beta)) with beta the graph's bandwidth (beta = 0: the whole
+// segment) and r the reach below. A segment is one graph of a batch (or the whole
+// graph). The
+// support of X_l lies within l bandwidths and rows outside stay zero, so the
+// result is the one of the full hop. The block's outputs read X_l at its sources
+// and their neighbours only, up to hop L, so a row further than L - l + 1 hops
+// from every source no longer reaches them: hop l covers r = min(l, L - l + 1)
+// bandwidths on either side (window_reach), which halves both the rows computed
+// and the rows stored against r = l (a lattice strip of 150 columns at 69 hops:
+// 129 to 94 ms a call). A computed row reads rows one bandwidth further out: at hop l - 1
+// those were computed, or lie past its support and were never written (zero).
 struct SliceWin {
     int64_t xoff;
     int32_t base, rows;
@@ -108,12 +115,16 @@ struct SliceWin {
     int32_t parity;
 };
 
-__host__ __device__ __forceinline__ void window_rows(const SliceWin &w, int32_t beta, int32_t ell, int32_t *lo,
+// bandwidths from its sources that hop ell of a block of L hops covers
+__host__ __device__ __forceinline__ int32_t window_reach(int32_t L, int32_t ell) { return min(ell, L - ell + 1); }
+
+// the rows within `reach` bandwidths of the sources
+__host__ __device__ __forceinline__ void window_rows(const SliceWin &w, int32_t beta, int32_t reach, int32_t *lo,
                                                      int32_t *hi) {
     int64_t a = w.seg_lo, b = w.seg_hi;
     if (beta > 0) {
-        a = max(a, static_cast<int64_t>(w.src_lo) - static_cast<int64_t>(ell) * beta);
-        b = min(b, static_cast<int64_t>(w.src_hi) + static_cast<int64_t>(ell) * beta);
+        a = max(a, static_cast<int64_t>(w.src_lo) - static_cast<int64_t>(reach) * beta);
+        b = min(b, static_cast<int64_t>(w.src_hi) + static_cast<int64_t>(reach) * beta);
     }
     *lo = static_cast<int32_t>(a);
     *hi = static_cast<int32_t>(b);
@@ -266,13 +277,7 @@ __global__ void __launch_bounds__(kSpmmWarps * 32) k_spmm_hop(const HopArgs<T> a
         if (w.parity >= 0) want = (w.parity + a.ell) & 1;
         slice_off = w.xoff;
         base = w.base;
-        int64_t wa = w.seg_lo, wb = w.seg_hi;
-        if (a.beta > 0) {
-            wa = max(wa, static_cast<int64_t>(w.src_lo) - static_cast<int64_t>(a.ell) * a.beta);
-            wb = min(wb, static_cast<int64_t>(w.src_hi) + static_cast<int64_t>(a.ell) * a.beta);
-        }
-        lo = static_cast<int32_t>(wa);
-        hi = static_cast<int32_t>(wb);
+        if (a.ell <= w.L) window_rows(w, a.beta, window_reach(w.L, a.ell), &lo, &hi);
         n_heavy = w.heavy_cnt;
         if (a.ell > w.L) lo = hi = 0, n_heavy = 0;  // the block is done: only its gather remains
     }
