@@ -309,10 +309,16 @@ sc_status sc_series_meet(sc_graph *g, const int32_t *tau, double *s_out);
 #define SC_OPT_TIME_KERNELS 4u  /* bracket every propagation launch with CUDA events (report.hop_ms) */
 /* Windowed blocks: Algorithm 2 visits only nodes with p_{l-1} > 0; a block of
    consecutive sources on a graph of bandwidth beta = max |i - j| reaches at
-   hop l only rows within l * beta of its sources, so each block stores and
-   computes that interval alone. Chosen automatically when a block's last
-   window is under half the graph (grid-like numbering); the values are the
-   same either way. Not with TGT+ or the TMA-gather kernel. */
+   hop l only rows within l * beta of its sources, and past the middle hop only
+   rows from which a source's neighbours are still in reach matter, so each
+   block stores and computes that interval alone. Chosen automatically when a
+   block's widest window is under half the graph (grid-like numbering); the
+   values are the same either way. Not with TGT+ or the TMA-gather kernel.
+   Without either flag, a block width, a split or a slice count of its own, a TGT
+   request on a graph of degree at most 8 runs resident instead: the nodes a few
+   neighbouring sources reach (by hops, not by ids) are kept in shared memory and
+   one kernel runs all their hops; sources whose ball does not fit run windowed.
+   The values are the same again. */
 #define SC_OPT_WINDOWS_OFF 8u
 #define SC_OPT_WINDOWS_FORCE 16u
 /* Unwindowed TGT blocks compute hop 3 from the non-zero values of X_2 only,
@@ -329,7 +335,7 @@ sc_status sc_series_meet(sc_graph *g, const int32_t *tau, double *s_out);
 #define SC_OPT_FULL_TOPGAMMA_SCAN 64u
 
 /* kernel classes of the per-class timing in sc_report (SC_OPT_TIME_KERNELS) */
-#define SC_KC_DENSE_HOP 0   /* full hops (k_spmm_hop, or the TMA-gather hop) */
+#define SC_KC_DENSE_HOP 0   /* full hops (k_spmm_hop, or the TMA-gather hop), or a resident traversal */
 #define SC_KC_MASK_HOP 1    /* hops 1-2 from the sources' neighbour bits (k_mask_scatter + k_hop2_mask) */
 #define SC_KC_SPARSE_HOP 2  /* hop 3 from the non-zero values of X_2 (k_hop_sparse) */
 #define SC_KC_BALL_HOP 3    /* hop L-1 on the two-hop balls (k_hop_ball) */
@@ -404,7 +410,7 @@ typedef struct sc_report {
     double walk_ms;            /* TGT+: wall time drawing walks (planning, kernels) */
     int64_t source_hops;       /* sum over sources of hops traversed (the traversal's work) */
     int32_t extension_rounds;  /* learned policy: rerun rounds for edges that failed their bound */
-    int32_t windowed;          /* 1 if the blocks ran windowed (SC_OPT_WINDOWS_*) */
+    int32_t windowed;          /* 1 if the blocks ran windowed or resident (SC_OPT_WINDOWS_*) */
     int64_t walk_steps;        /* TGT+: walk steps taken (both walks of every pair) */
     double walk_device_ms;     /* TGT+: device time of the walk launches (events) */
     /* with SC_OPT_TIME_KERNELS, per kernel class SC_KC_*: summed duration (events around

@@ -207,6 +207,14 @@ struct sc_graph {
     sc::DevBuf<double> tp_srcstat;  // per column: rho_hat, min and max of p over N(s)
     sc::DevBuf<long long> tp_src_rhs;  // per column: Eq. 14's right side (per-source switch)
     sc::DevBuf<int32_t> tp_cap_list;   // the sources that switch at a test (per-source switch)
+    // resident traversal (resident.cu): neighbour ids in rows of res_width, the
+    // groups of sources per kind of segment (0: bipartite, 1: not), work lists
+    sc::DevBuf<int32_t> res_ell, res_len, res_list, res_over, res_count, res_single, res_order_dev[2];
+    std::vector<int32_t> res_order[2];
+    int res_order_width[2] = {0, 0};
+    int res_width = 0;
+    bool res_ready = false;
+    sc::DevBuf<unsigned char> res_scratch;
     std::vector<cudaEvent_t> hop_events;  // pairs bracketing timed propagation launches
     ~sc_graph() {
         for (cudaEvent_t e : hop_events) cudaEventDestroy(e);

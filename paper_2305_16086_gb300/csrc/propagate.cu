@@ -13,6 +13,7 @@
 
 #include "hop2_mask.cuh"
 #include "hop_tma.cuh"
+#include "resident.cuh"
 #include "sparse_hops.cuh"
 #include "tgtplus.cuh"
 #include "propagate.cuh"
@@ -1496,6 +1497,47 @@ static void run_blocks_win(Run &R, std::vector<int32_t> sources, const std::vect
     }
 }
 
+// a request whose sources may run resident: TGT, no launch shape, window or hop form
+// asked for (the per-graph condition is the largest degree)
+static bool resident_allowed(const sc_options &o) {
+    return o.mode == SC_MODE_TGT && o.rows_split == 0 && o.block_width == 0 && o.max_slices == 0 &&
+           !(o.flags & (SC_OPT_WINDOWS_OFF | SC_OPT_WINDOWS_FORCE | SC_OPT_SPARSE_HOPS));
+}
+
+// the launch shape of the sources a resident run leaves over (balls past shared memory):
+// one row per warp in the widest block, without timing candidates for a few blocks
+static TuneResult leftover_shape(int prec) { return TuneResult{prec == SC_PREC_FP64 ? 64 : 128, 1, 0.0}; }
+
+// the resident traversal of `sources`; returns those left for the block kernels
+static std::vector<int32_t> resident_blocks(Run &R, const std::vector<int32_t> &sources,
+                                            const std::vector<int32_t> &len, const std::vector<int32_t> &seg_start,
+                                            const std::vector<char> &seg_take, const std::vector<char> &seg_bip) {
+    sc_graph *g = R.g;
+    // what a launch cannot do without: the graph, once
+    const double bytes = 4.0 * g->nnz + 4.0 * (g->n + 1) + (R.prec == SC_PREC_FP64 ? 8.0 : 4.0) * g->n;
+    ResidentRun rr{g, R.s, R.prec, R.h0, R.extra, R.rec, [&](const std::function<void()> &launch) {
+                       const int64_t t = timer_open(R, R.s);
+                       launch();
+                       timer_close(R, t, SC_KC_DENSE_HOP, bytes, R.s);
+                       ++R.hop_launches;
+                       R.alg_bytes += bytes;
+                   }};
+    ResidentStats st;
+    std::vector<int32_t> left = run_resident(rr, sources, len, seg_start, seg_take, seg_bip, &st);
+    R.launches += st.launches;
+    R.hops += st.hops;
+    size_t q = 0;  // both lists are in id order
+    for (int32_t v : sources) {
+        while (q < left.size() && left[q] < v) ++q;
+        if (q < left.size() && left[q] == v) continue;
+        const int32_t l = len[v] + R.extra;
+        R.source_hops += l;
+        R.ell_min_src = std::min(R.ell_min_src, l);
+        R.ell_max_src = std::max(R.ell_max_src, l);
+    }
+    return left;
+}
+
 // ---------------------------------------------------------------------------
 // sc_all_edges
 // ---------------------------------------------------------------------------
@@ -1757,12 +1799,17 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     const bool use_win = !plus && o.rows_split != -1 && !(o.flags & SC_OPT_WINDOWS_OFF) &&
                          ((o.flags & SC_OPT_WINDOWS_FORCE) ||
                           2.0 * (Lmax / 2 + 2.0) * static_cast<double>(beta) + 128.0 < 0.5 * static_cast<double>(n));
+    // graphs of small degree run resident (each source's ball in shared memory) as far as it
+    // fits: a 150 x 613 strip at 67 hops takes 9.0 ms a call, windowed 94 ms
+    const bool use_res = resident_allowed(o) && resident_degree_ok(g->max_degree) && Lmax > 0;
+    g->res_width = g->max_degree <= 4 ? 4 : 8;
     // a bf16 run whose early hops are fp32 is tuned (and its buffers sized) in fp32
     const int32_t h0 = bf16_first_hop(o);
     const int tune_prec = (o.precision == SC_PREC_BF16 && h0 > 1) ? SC_PREC_FP32 : o.precision;
     std::vector<TuneResult> per_b;
-    const TuneResult tr = autotune(g, tune_prec, o.block_width, fixV, o.max_slices, Lmax,
-                                   GatherRec{rec.mode, nullptr, 0}, !use_win, s, &per_b);
+    const TuneResult tr = use_res ? leftover_shape(tune_prec)
+                                  : autotune(g, tune_prec, o.block_width, fixV, o.max_slices, Lmax,
+                                             GatherRec{rec.mode, nullptr, 0}, !use_win, s, &per_b);
     Run R;
     R.g = g;
     R.o = &o;
@@ -1804,8 +1851,10 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     }
     const int64_t nblocks_total = (static_cast<int64_t>(n) + R.B - 1) / R.B;
 
-    g->xa.reserve(R.slices * R.slice_bytes);
-    g->xb.reserve(R.slices * R.slice_bytes);
+    if (!use_res) {
+        g->xa.reserve(R.slices * R.slice_bytes);
+        g->xb.reserve(R.slices * R.slice_bytes);
+    }
     k_reset_rows<<<ceil_div(n, 8), 256, 0, s>>>(g->row_ptr.get(), nullptr, n, g->tau_entry.get(), R.rec.mode,
                                                 g->acc_g.get(), g->acc_t1.get(), g->acc_t2.get(), rec_all, rec_stride);
     SC_LAUNCH_CHECK();
@@ -1836,9 +1885,16 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
         std::iota(all.begin(), all.end(), 0);
     }
     const std::vector<int32_t> seg_whole{0, n};
+    const std::vector<char> seg_bip{static_cast<char>(g->bipartite ? 1 : 0)};
     auto run = [&](const std::vector<int32_t> &src, const std::vector<int32_t> &l) {
-        if (use_win) run_blocks_win(R, src, l, seg_whole, beta, std::vector<char>{static_cast<char>(g->bipartite ? 1 : 0)});
-        else run_blocks(R, src, l);
+        if (use_res) {
+            const std::vector<int32_t> left = resident_blocks(R, src, l, seg_whole, std::vector<char>{1}, seg_bip);
+            if (!left.empty()) run_blocks_win(R, left, l, seg_whole, beta, seg_bip);
+        } else if (use_win) {
+            run_blocks_win(R, src, l, seg_whole, beta, seg_bip);
+        } else {
+            run_blocks(R, src, l);
+        }
     };
     DevBuf<int32_t> tau_saved;
     if (learned_plus) {
@@ -2058,7 +2114,7 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
         rep->walks = R.walks;
         rep->edges_extended = static_cast<int32_t>(extended);
         rep->extension_rounds = rounds;
-        rep->windowed = use_win ? 1 : 0;
+        rep->windowed = use_win || use_res ? 1 : 0;
         rep->uncertified = est_learned ? 1 : 0;
         rep->tt_min = plus ? (R.tt_min == INT32_MAX ? 0 : R.tt_min) : 0;
         rep->tt_max = plus ? R.tt_max : 0;
@@ -2374,8 +2430,19 @@ static void batch_impl(sc_graph *const *graphs, int32_t count, const sc_options 
     const int fixV = o.rows_split == 0 ? -1 : o.rows_split;
     const int32_t h0 = bf16_first_hop(o);
     const int tune_prec = (o.precision == SC_PREC_BF16 && h0 > 1) ? SC_PREC_FP32 : o.precision;
-    const TuneResult tr = autotune(gb, tune_prec, o.block_width, fixV, o.max_slices, ell[big] + extra,
-                                   GatherRec{0, nullptr, 0}, false, gb->stream);
+    // graphs of small degree run resident; the block kernels take the others
+    std::vector<char> seg_take(count, 0);
+    int32_t res_deg = 0;
+    bool all_res = true;
+    for (int32_t i = 0; i < count; ++i) {
+        seg_take[i] = resident_allowed(o) && resident_degree_ok(graphs[i]->max_degree) ? 1 : 0;
+        if (seg_take[i]) res_deg = std::max(res_deg, graphs[i]->max_degree);
+        else all_res = false;
+    }
+    U->res_width = res_deg <= 4 ? 4 : 8;
+    const TuneResult tr = all_res ? leftover_shape(tune_prec)
+                                  : autotune(gb, tune_prec, o.block_width, fixV, o.max_slices, ell[big] + extra,
+                                             GatherRec{0, nullptr, 0}, false, gb->stream);
     SC_CUDA(cudaStreamSynchronize(gb->stream));
 
     Run R;
@@ -2430,8 +2497,21 @@ static void batch_impl(sc_graph *const *graphs, int32_t count, const sc_options 
     SC_CUDA(cudaEventRecord(ev1, s));
     std::vector<char> seg_bip(count);
     for (int32_t i = 0; i < count; ++i) seg_bip[i] = graphs[i]->bipartite ? 1 : 0;
-    run_blocks_win(R, all, len, seg_start, beta, seg_bip);
-    book(all);
+    auto run = [&](const std::vector<int32_t> &src) {
+        std::vector<int32_t> res, rest;  // src is in id order
+        int32_t i = 0;
+        for (int32_t v : src) {
+            while (v >= n_off[i + 1]) ++i;
+            (seg_take[i] ? res : rest).push_back(v);
+        }
+        if (!res.empty()) {
+            const std::vector<int32_t> left = resident_blocks(R, res, len, seg_start, seg_take, seg_bip);
+            rest.insert(rest.end(), left.begin(), left.end());
+        }
+        run_blocks_win(R, rest, len, seg_start, beta, seg_bip);
+        book(src);
+    };
+    run(all);
 
     // ---- combine (and for the learned lengths the check / extension loop), Foster sums, outputs
     DevBuf<double> d_s, seg_sum;
@@ -2504,8 +2584,7 @@ static void batch_impl(sc_graph *const *graphs, int32_t count, const sc_options 
                 U->acc_g.get(), U->acc_t1.get(), U->acc_t2.get(), R.rec.all, R.rec.stride);
             SC_LAUNCH_CHECK();
             R.launches += 2;
-            run_blocks_win(R, redo, len, seg_start, beta, seg_bip);
-            book(redo);
+            run(redo);
             combine();
         }
     }

@@ -1,0 +1,648 @@
+// Resident traversal: a few sources' whole traversal (Algorithm 2, every hop
+// and every gather of Eq. 9) by one CTA, the probabilities in shared memory.
+//
+// On graphs of small degree whose balls grow slowly (lattices, road networks,
+// paths) a source's walk reaches few nodes: within l hops of it the support of
+// p_l, and since the outputs read p_l at the source and its neighbours only,
+// hop l of L needs the rows within min(l, L - l + 1) hops (a row further out
+// no longer reaches them). A ball of radius (L + 1) / 2 holds all of it: 2,450
+// nodes of a square lattice at L = 69, against the 150 * 69 rows and more of a
+// block's id interval. So each CTA takes C sources next to each other, walks
+// the ball around them breadth first into a list of nodes in level order
+// (shared-memory hash table), turns their adjacency into 16-bit local ids, and
+// runs all hops on the ball: the rows of hop l are a prefix of the list. No
+// launch per hop, no block in global memory.
+//
+// Every value is bit for bit the block kernels': a row's neighbours are summed
+// in CSR order (degrees up to 8, one chunk), scaled once by 1/d and rounded to
+// the storage type where the block would store it; rows outside the ball are
+// exact zeros or are never read.
+//
+// On a bipartite graph the sources of a CTA have one colour, hop l touches the
+// levels of its own parity only, and one buffer serves both X_{l-1} and X_l
+// (they lie on different levels); otherwise two buffers alternate.
+//
+// What bounds it: shared-memory bandwidth in the hops. 32 rows of 4 neighbours
+// and a 16-byte vector of columns move 23 wavefronts of 128 bytes (4 neighbour
+// vectors, the result, the ids, 1/d): 5.6 values a clock per SM at best, against
+// 2.3 measured for the windowed block kernel, which streams its rows through
+// HBM. Small balls are bound by the latency of a level (one dependent global
+// load and a table insert, then a barrier) and of a hop (one barrier), which is
+// why several CTAs share an SM when the ball is small. Whole calls, windowed
+// blocks against this: 150 x 613 strip at 67 + 2 hops 94 -> 9.0 ms, 400 x 400
+// lattice at learned lengths (37 to 353 hops) 625 -> 31 ms, 24 mixed graphs with
+// lattices of 1,000 to 5,000 nodes at 1,003 hops 223 -> 85 ms.
+#include <algorithm>
+#include <numeric>
+
+#include "resident.cuh"
+
+namespace sc {
+
+constexpr int kResDegMax = 8;       // largest degree taken (neighbour ids kept per row)
+constexpr int kResClasses = 4;      // shared-memory sizes tried in turn; the last keeps the adjacency in global memory
+constexpr int kResSample = 128;     // groups whose ball is measured to choose the first class
+
+struct ResArgs {
+    const int32_t *row_ptr;
+    const int32_t *ell;      // n x W neighbour ids in CSR order, -1 past the degree
+    const void *inv_deg;
+    int32_t n;
+    const int32_t *order;    // groups of C sources (-1: empty slot)
+    const int32_t *groups;   // the launch's groups (nullable: all of 0 .. ngroups)
+    int32_t ngroups;
+    const int32_t *len;      // per node: hops its traversal takes (<= 0: not run)
+    int32_t cap;             // nodes a list holds
+    int32_t levels;          // level bounds held
+    int32_t hash;            // slots of the hash table
+    int32_t h0;              // first hop whose values are rounded to bf16
+    const int32_t *tau;
+    double *g, *t1, *t2;
+    GatherRec rec;
+    int32_t *over;           // [0]: groups that did not fit, [1 ..]: their ids
+    int32_t *count;          // nullable: measure only; [0] = largest list, [1] = groups that did not fit
+    unsigned char *scratch;  // global-adjacency class: per CTA adjacency, 1/d, nodes, local id per node
+    size_t scratch_cta;
+};
+
+template <typename Acc, int C>
+struct alignas(C * sizeof(Acc)) ResVec {
+    Acc v[C];
+};
+
+template <int W>
+struct alignas(2 * W) ResAdj {
+    uint16_t v[W];
+};
+
+// the last CTA-wide layout: adjacency, 1/d, level bounds, then X, which the build's tables overlay
+template <typename Acc, int C, int W, bool BIP, bool GADJ>
+struct ResLayout {
+    static constexpr int NBUF = BIP ? 1 : 2;
+    static constexpr size_t row_bytes = (GADJ ? 0 : 2 * W + sizeof(Acc)) + static_cast<size_t>(NBUF) * C * sizeof(Acc);
+    static __host__ __device__ size_t up(size_t x) { return (x + 15) / 16 * 16; }
+    static __host__ __device__ size_t adj_bytes(int N) { return up(static_cast<size_t>(N) * 2 * W); }
+    static __host__ __device__ size_t inv_bytes(int N) { return up(static_cast<size_t>(N) * sizeof(Acc)); }
+    static __host__ __device__ size_t x_bytes(int N) { return up(static_cast<size_t>(NBUF) * (N + 1) * C * sizeof(Acc)); }
+};
+
+template <typename Acc, int C, int W, bool BIP, bool GADJ>
+__global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
+    using L = ResLayout<Acc, C, W, BIP, GADJ>;
+    using Vec = ResVec<Acc, C>;
+    using Adj = ResAdj<W>;
+    extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ int32_t cnt[2];
+    __shared__ int32_t overflow;
+    const int T = blockDim.x, tid = threadIdx.x;
+    const int cap = a.cap, N = (BIP ? 2 : 1) * cap;  // local ids; id N: a cell that stays zero
+    int32_t *lvl = reinterpret_cast<int32_t *>(sm);  // lvl[k]: nodes of its list up to level k
+    unsigned char *p = sm + L::up(static_cast<size_t>(a.levels) * sizeof(int32_t));
+    Adj *adj;
+    Acc *inv;
+    int32_t *nodes;
+    uint32_t *hkey = nullptr;
+    uint16_t *hval;  // shared: value of a hash slot; global-adjacency class: local id per node of the graph
+    if constexpr (GADJ) {
+        unsigned char *q = a.scratch + blockIdx.x * a.scratch_cta;
+        adj = reinterpret_cast<Adj *>(q);
+        inv = reinterpret_cast<Acc *>(q + L::adj_bytes(N));
+        nodes = reinterpret_cast<int32_t *>(q + L::adj_bytes(N) + L::inv_bytes(N));
+        hval = reinterpret_cast<uint16_t *>(q + L::adj_bytes(N) + L::inv_bytes(N) + L::up(static_cast<size_t>(N) * 4));
+    } else {
+        adj = reinterpret_cast<Adj *>(p);
+        inv = reinterpret_cast<Acc *>(p + L::adj_bytes(N));
+        p += L::adj_bytes(N) + L::inv_bytes(N);
+        nodes = reinterpret_cast<int32_t *>(p);
+        hkey = reinterpret_cast<uint32_t *>(p + L::up(static_cast<size_t>(N) * 4));
+        hval = reinterpret_cast<uint16_t *>(hkey + a.hash);
+    }
+    Vec *X = reinterpret_cast<Vec *>(p);  // NBUF x (N + 1)
+    const Acc *inv_deg = static_cast<const Acc *>(a.inv_deg);
+
+    for (int32_t gi = blockIdx.x; gi < a.ngroups; gi += gridDim.x) {
+        const int32_t gid = a.groups ? a.groups[gi] : gi;
+        const int32_t *src = a.order + static_cast<int64_t>(gid) * C;
+        int32_t Lg = 0;
+#pragma unroll
+        for (int q = 0; q < C; ++q) Lg = max(Lg, src[q] >= 0 ? a.len[src[q]] : 0);
+        if (Lg <= 0) continue;  // CTA-uniform
+        const int32_t R = (Lg + 1) / 2;
+
+        // ---- the ball: nodes in level order, sources first ----
+        if constexpr (!GADJ)
+            for (int t = tid; t < a.hash; t += T) hkey[t] = 0u;
+        if (tid == 0) {
+            cnt[0] = C;
+            cnt[1] = 0;
+            overflow = 0;
+            lvl[0] = C;
+        }
+        __syncthreads();
+        volatile int32_t *ovf = &overflow;
+        // claims node v for `list` unless it is known
+        auto visit = [&](int32_t v, int list) {
+            if constexpr (GADJ) {
+                unsigned short *m = reinterpret_cast<unsigned short *>(hval) + v;
+                if (*reinterpret_cast<volatile unsigned short *>(m) != 0xffffu) return;
+                if (atomicCAS(m, static_cast<unsigned short>(0xffffu), static_cast<unsigned short>(0xfffeu)) != 0xffffu) return;
+                const int32_t at = atomicAdd(&cnt[list], 1);
+                if (at >= cap) {
+                    *m = 0xffffu;
+                    *ovf = 1;
+                    return;
+                }
+                *m = static_cast<unsigned short>(list * cap + at);
+                nodes[list * cap + at] = v;
+            } else {
+                const uint32_t key = static_cast<uint32_t>(v) + 1u;
+                uint32_t slot = __umulhi(key * 2654435761u, static_cast<uint32_t>(a.hash));
+                for (int probe = 0; probe < a.hash; ++probe) {
+                    const uint32_t old = atomicCAS(&hkey[slot], 0u, key);
+                    if (old == key) return;
+                    if (old == 0u) {
+                        const int32_t at = atomicAdd(&cnt[list], 1);
+                        if (at >= cap) {
+                            *ovf = 1;
+                            return;
+                        }
+                        hval[slot] = static_cast<uint16_t>(list * cap + at);
+                        nodes[list * cap + at] = v;
+                        return;
+                    }
+                    slot = slot + 1 == static_cast<uint32_t>(a.hash) ? 0 : slot + 1;
+                }
+                *ovf = 1;
+            }
+        };
+        if (tid == 0) {
+            for (int q = 0; q < C; ++q) {
+                const int32_t s = src[q];
+                const bool on = s >= 0 && a.len[s] > 0;
+                nodes[q] = on ? s : -1;
+                if (!on) continue;
+                if constexpr (GADJ) {
+                    hval[s] = static_cast<uint16_t>(q);
+                } else {
+                    const uint32_t key = static_cast<uint32_t>(s) + 1u;
+                    uint32_t slot = __umulhi(key * 2654435761u, static_cast<uint32_t>(a.hash));
+                    while (hkey[slot]) slot = slot + 1 == static_cast<uint32_t>(a.hash) ? 0 : slot + 1;  // < C keys in the table
+                    hkey[slot] = key;
+                    hval[slot] = static_cast<uint16_t>(q);
+                }
+            }
+        }
+        __syncthreads();
+        int32_t top = 0;  // last level
+        for (int32_t k = 0; k < R; ++k) {
+            const int from = BIP ? (k & 1) : 0, to = BIP ? 1 - from : 0;
+            const int32_t f0 = BIP ? (k >= 2 ? lvl[k - 2] : 0) : (k >= 1 ? lvl[k - 1] : 0), f1 = lvl[k];
+            for (int32_t t = tid; t < (f1 - f0) * W; t += T) {
+                if (*ovf) break;
+                const int32_t v = nodes[from * cap + f0 + t / W];
+                if (v < 0) continue;
+                const int32_t nb = a.ell[static_cast<int64_t>(v) * W + t % W];
+                if (nb >= 0) visit(nb, to);
+            }
+            __syncthreads();
+            const int32_t now = min(cnt[to], cap);
+            const int32_t before = BIP ? (k >= 1 ? lvl[k - 1] : 0) : f1;
+            const bool stop = overflow || now == before;
+            if (!stop && k + 1 >= a.levels) {  // too deep for the level bounds
+                if (tid == 0) overflow = 1;
+                __syncthreads();
+                break;
+            }
+            if (stop) break;
+            if (tid == 0) lvl[k + 1] = now;
+            top = k + 1;
+            __syncthreads();
+        }
+        __syncthreads();
+        const bool fits = overflow == 0;
+        const int32_t n0 = min(cnt[0], cap), n1 = BIP ? min(cnt[1], cap) : 0;
+        auto forget = [&] {  // the global-adjacency class: the nodes' local ids back to "unknown"
+            if constexpr (GADJ) {
+                for (int32_t t = tid; t < n0 + n1; t += T) {
+                    const int32_t v = nodes[t < n0 ? t : cap + t - n0];
+                    if (v >= 0) hval[v] = 0xffffu;
+                }
+            }
+        };
+        if (a.count || !fits) {
+            if (tid == 0) {
+                if (a.count) {
+                    atomicMax(&a.count[0], max(n0, n1));
+                    if (!fits) atomicAdd(&a.count[1], 1);
+                } else {
+                    a.over[1 + atomicAdd(&a.over[0], 1)] = gid;
+                }
+            }
+            forget();
+            __syncthreads();
+            continue;
+        }
+
+        // ---- adjacency in local ids (past the ball or the degree: the zero cell), 1/d ----
+        for (int32_t t = tid; t < n0 + n1; t += T) {
+            const int32_t i = t < n0 ? t : cap + t - n0;
+            const int32_t v = nodes[i];
+            Adj out;
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                const int32_t nb = v >= 0 ? a.ell[static_cast<int64_t>(v) * W + w] : -1;
+                uint16_t id = static_cast<uint16_t>(N);
+                if (nb >= 0) {
+                    if constexpr (GADJ) {
+                        const uint16_t m = *reinterpret_cast<volatile uint16_t *>(&hval[nb]);
+                        if (m != 0xffffu) id = m;
+                    } else {
+                        const uint32_t key = static_cast<uint32_t>(nb) + 1u;
+                        uint32_t slot = __umulhi(key * 2654435761u, static_cast<uint32_t>(a.hash));
+                        for (int probe = 0; probe < a.hash; ++probe) {
+                            const uint32_t have = hkey[slot];
+                            if (have == key) id = hval[slot];
+                            if (have == key || have == 0u) break;
+                            slot = slot + 1 == static_cast<uint32_t>(a.hash) ? 0 : slot + 1;
+                        }
+                    }
+                }
+                out.v[w] = id;
+            }
+            adj[i] = out;
+            inv[i] = v >= 0 ? inv_deg[v] : Acc(0);
+        }
+        __syncthreads();
+        forget();
+        __syncthreads();
+
+        // ---- X_0 = e_s ----
+        {
+            Vec z;
+#pragma unroll
+            for (int c = 0; c < C; ++c) z.v[c] = Acc(0);
+            for (int b = 0; b < L::NBUF; ++b) {
+                Vec *xb = X + static_cast<size_t>(b) * (N + 1);
+                for (int32_t t = tid; t < n0 + n1; t += T) xb[t < n0 ? t : cap + t - n0] = z;
+                if (tid == 0) xb[N] = z;
+            }
+        }
+        __syncthreads();
+        if (tid < C && src[tid] >= 0 && a.len[src[tid]] > 0) X[tid].v[tid] = Acc(1);
+        // the gather's threads (the last ones: they take the fewest rows): entry `gk` of source column `gq`
+        const int gt = T - 1 - tid;
+        const int gq = gt / W;
+        int32_t gk = -1, glen = 0, gtau = 0;
+        uint32_t gj = 0;
+        double acc = 0.0, r1 = 0.0, r2 = 0.0;
+        if (gt < C * W && src[gq] >= 0 && a.len[src[gq]] > 0) {
+            const int32_t s = src[gq], b = a.row_ptr[s];
+            if (gt % W < a.row_ptr[s + 1] - b) {
+                gk = b + gt % W;
+                glen = a.len[s];
+                gtau = a.tau[gk];
+                gj = adj[gq].v[gt % W];
+                acc = a.g[gk];
+                r1 = a.t1[gk];
+                r2 = a.t2[gk];
+            }
+        }
+        auto gather = [&](int32_t h) {  // the hop-h term of Eq. 9 (gather_term, the sums in registers)
+            if (gk < 0 || h > glen) return;
+            const Vec *xb = X + (BIP ? 0 : static_cast<size_t>(h & 1) * (N + 1));
+            const double diag = BIP && (h & 1) ? 0.0 : static_cast<double>(xb[gq].v[gq]);
+            const double xj = BIP && !(h & 1) ? 0.0 : static_cast<double>(xb[gj].v[gq]);
+            const double term = diag - xj;
+            if (h <= gtau) {
+                acc += term;
+                if (a.rec.mode == 1) {
+                    if (h == gtau - 1) r1 = term;
+                    else if (h == gtau) r2 = term;
+                }
+            } else if (a.rec.mode == 0 || a.rec.mode == 3) {
+                if (h == gtau + 1) r1 = term;
+                else if (h == gtau + 2) r2 = term;
+            }
+            if (a.rec.all) {
+                if (a.rec.mode == 3) {
+                    if (h == gtau - 1 || h == gtau) a.rec.all[static_cast<int64_t>(gk) * 2 + (h - gtau + 1)] = term;
+                } else {
+                    a.rec.all[static_cast<int64_t>(gk) * a.rec.stride + h] = term;
+                }
+            }
+        };
+        __syncthreads();
+
+        // ---- the hops ----
+        for (int32_t h = 1; h <= Lg; ++h) {
+            int32_t lim = min(min(h, Lg - h + 1), top);
+            const int par = BIP ? (h & 1) : 0;
+            if (BIP) lim -= (lim ^ h) & 1;
+            const int32_t rows = lim >= 0 ? lvl[lim] : 0;
+            const Vec *xp = X + (BIP ? 0 : static_cast<size_t>((h - 1) & 1) * (N + 1));
+            Vec *xn = X + (BIP ? 0 : static_cast<size_t>(h & 1) * (N + 1));
+            const bool to_bf16 = h >= a.h0;
+            const int32_t base = par * cap;
+#pragma unroll 2
+            for (int32_t t = tid; t < rows; t += T) {
+                const Adj id = adj[base + t];
+                Vec sum = xp[id.v[0]];
+#pragma unroll
+                for (int w = 1; w < W; ++w) {
+                    const Vec x = xp[id.v[w]];
+#pragma unroll
+                    for (int c = 0; c < C; ++c) sum.v[c] += x.v[c];
+                }
+                const Acc d = inv[base + t];
+#pragma unroll
+                for (int c = 0; c < C; ++c) sum.v[c] *= d;
+                if constexpr (sizeof(Acc) == 4)
+                    if (to_bf16) {
+#pragma unroll
+                        for (int c = 0; c < C; ++c) sum.v[c] = __bfloat162float(__float2bfloat16_rn(sum.v[c]));
+                    }
+                xn[base + t] = sum;
+            }
+            if (h >= 2) gather(h - 1);
+            __syncthreads();
+        }
+        gather(Lg);
+        if (gk >= 0) {
+            a.g[gk] = acc;
+            a.t1[gk] = r1;
+            a.t2[gk] = r2;
+        }
+        __syncthreads();  // X and the lists are the next group's
+    }
+}
+
+// neighbour ids in rows of W, -1 past the degree (rows of larger degree: all -1, never taken)
+__global__ void k_res_ell(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col, int32_t n, int W,
+                          int32_t *__restrict__ ell) {
+    const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (t >= static_cast<int64_t>(n) * W) return;
+    const int32_t r = static_cast<int32_t>(t / W), w = static_cast<int32_t>(t % W);
+    const int32_t b = row_ptr[r], d = row_ptr[r + 1] - b;
+    ell[t] = d <= W && w < d ? col[b + w] : -1;
+}
+
+// ---------------------------------------------------------------------------
+// host
+// ---------------------------------------------------------------------------
+struct ResClass {
+    size_t smem;  // dynamic shared memory of a CTA
+    int threads, levels, per_sm;
+};
+// four, two and one CTA per SM (1 KB of an SM's 228 KB goes with each CTA, a few words are static)
+static const ResClass kResClass[kResClasses] = {{55 * 1024, 256, 256, 4},
+                                                {112 * 1024, 512, 1024, 2},
+                                                {226 * 1024, 1024, 1024, 1},
+                                                {226 * 1024, 1024, 1024, 1}};
+
+template <typename Acc, int W, bool BIP, bool GADJ>
+static int32_t res_capacity(int cls) {
+    constexpr int C = GADJ ? 1 : 16 / static_cast<int>(sizeof(Acc));
+    using L = ResLayout<Acc, C, W, BIP, GADJ>;
+    const size_t room = kResClass[cls].smem - kResClass[cls].levels * sizeof(int32_t) - 6 * 16 - 2 * 16;
+    size_t rows = room / L::row_bytes;
+    rows = std::min<size_t>(rows, 65000);  // 16-bit ids, and room for the marks 0xfffe, 0xffff
+    return static_cast<int32_t>(BIP ? rows / 2 : rows);
+}
+
+template <typename Acc, int W, bool BIP, bool GADJ>
+static void res_launch(sc_graph *g, ResArgs a, int cls, cudaStream_t s) {
+    constexpr int C = GADJ ? 1 : 16 / static_cast<int>(sizeof(Acc));
+    using L = ResLayout<Acc, C, W, BIP, GADJ>;
+    const ResClass &k = kResClass[cls];
+    a.cap = res_capacity<Acc, W, BIP, GADJ>(cls);
+    a.levels = k.levels;
+    const int N = (BIP ? 2 : 1) * a.cap;
+    // the tables lie over X: 4 bytes a node for the list, 6 a slot
+    a.hash = GADJ ? 0 : std::min<int>(2 * N, static_cast<int>((L::x_bytes(N) - L::up(static_cast<size_t>(N) * 4)) / 6));
+    int grid = a.ngroups;
+    if (GADJ) {
+        grid = std::min(grid, (g->num_sms > 0 ? g->num_sms : 148) * k.per_sm);
+        a.scratch_cta = L::adj_bytes(N) + L::inv_bytes(N) + L::up(static_cast<size_t>(N) * 4) +
+                        (static_cast<size_t>(g->n) * 2 + 255) / 256 * 256;
+        g->res_scratch.reserve(a.scratch_cta * grid);
+        SC_CUDA(cudaMemsetAsync(g->res_scratch.get(), 0xff, a.scratch_cta * grid, s));
+        a.scratch = g->res_scratch.get();
+    }
+    auto *fn = k_resident<Acc, C, W, BIP, GADJ>;
+    SC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(k.smem)));
+    fn<<<grid, k.threads, k.smem, s>>>(a);
+    SC_LAUNCH_CHECK();
+}
+
+template <typename Acc, int W>
+static void res_dispatch(sc_graph *g, const ResArgs &a, int cls, bool bip, cudaStream_t s) {
+    if (cls == kResClasses - 1) {
+        if (bip) res_launch<Acc, W, true, true>(g, a, cls, s);
+        else res_launch<Acc, W, false, true>(g, a, cls, s);
+    } else {
+        if (bip) res_launch<Acc, W, true, false>(g, a, cls, s);
+        else res_launch<Acc, W, false, false>(g, a, cls, s);
+    }
+}
+
+static void res_dispatch(sc_graph *g, const ResArgs &a, bool fp64, int W, int cls, bool bip, cudaStream_t s) {
+    if (fp64) {
+        if (W == 4) res_dispatch<double, 4>(g, a, cls, bip, s);
+        else res_dispatch<double, 8>(g, a, cls, bip, s);
+    } else {
+        if (W == 4) res_dispatch<float, 4>(g, a, cls, bip, s);
+        else res_dispatch<float, 8>(g, a, cls, bip, s);
+    }
+}
+
+template <typename Acc>
+static int32_t res_cap_of(int W, int cls, bool bip) {
+    if (W == 4) return bip ? res_capacity<Acc, 4, true, false>(cls) : res_capacity<Acc, 4, false, false>(cls);
+    return bip ? res_capacity<Acc, 8, true, false>(cls) : res_capacity<Acc, 8, false, false>(cls);
+}
+
+bool resident_degree_ok(int32_t max_degree) { return max_degree <= kResDegMax; }
+
+// Groups of `width` sources with neighbouring ids, one segment (and, on a
+// bipartite one, one colour) to a group, segments of more nodes first; only
+// segments of the wanted kind whose degrees fit.
+static std::vector<int32_t> res_groups(const sc_graph *g, const std::vector<int32_t> &level,
+                                       const std::vector<int32_t> &seg_start, const std::vector<char> &seg_take,
+                                       const std::vector<char> &seg_bip, bool bip, int width) {
+    const int nseg = static_cast<int>(seg_start.size()) - 1;
+    std::vector<int> segs;
+    for (int i = 0; i < nseg; ++i)
+        if (seg_take[i] && (seg_bip[i] != 0) == bip) segs.push_back(i);
+    std::stable_sort(segs.begin(), segs.end(), [&](int x, int y) {
+        return seg_start[x + 1] - seg_start[x] > seg_start[y + 1] - seg_start[y];
+    });
+    std::vector<int32_t> out;
+    for (int i : segs)
+        for (int colour = 0; colour < (bip ? 2 : 1); ++colour) {
+            for (int32_t v = seg_start[i]; v < seg_start[i + 1]; ++v)
+                if (!bip || (level[v] & 1) == colour) out.push_back(v);
+            while (out.size() % width) out.push_back(-1);
+        }
+    return out;
+}
+
+// The traversal of `sources` (len + extra hops each) as far as their balls fit;
+// returns the sources that are left for the block kernels. seg_take marks the
+// segments to handle here (degrees up to kResDegMax).
+std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_t> &sources,
+                                  const std::vector<int32_t> &len, const std::vector<int32_t> &seg_start,
+                                  const std::vector<char> &seg_take, const std::vector<char> &seg_bip,
+                                  ResidentStats *st) {
+    sc_graph *g = r.g;
+    cudaStream_t s = r.s;
+    const int32_t n = g->n;
+    const bool fp64 = r.prec == SC_PREC_FP64;
+    const int W = g->res_width;
+    std::vector<int32_t> h_len(n, 0), left;
+    for (int32_t v : sources) h_len[v] = len[v] + r.extra;
+    g->res_len.reserve(n);
+    SC_CUDA(cudaMemcpyAsync(g->res_len.get(), h_len.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    if (!g->res_ready) {
+        g->res_ell.reserve(static_cast<size_t>(n) * W);
+        k_res_ell<<<ceil_div(static_cast<int64_t>(n) * W, 256), 256, 0, s>>>(g->row_ptr.get(), g->col_idx.get(), n, W,
+                                                                           g->res_ell.get());
+        SC_LAUNCH_CHECK();
+        ++st->launches;
+        g->res_ready = true;
+    }
+    for (int kind = 0; kind < 2; ++kind) {
+        const bool bip = kind == 0;
+        bool any = false;
+        for (size_t i = 0; i + 1 < seg_start.size(); ++i) any = any || (seg_take[i] && (seg_bip[i] != 0) == bip);
+        if (!any) continue;
+        // groups of the widest class, and the same sources one by one for the last class
+        const int width = fp64 ? 2 : 4;
+        std::vector<int32_t> &order = g->res_order[kind];
+        DevBuf<int32_t> &d_order = g->res_order_dev[kind];
+        if (g->res_order_width[kind] != width) {
+            std::vector<int32_t> level(n);
+            SC_CUDA(cudaMemcpyAsync(level.data(), g->level.get(), n * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+            SC_CUDA(cudaStreamSynchronize(s));
+            order = res_groups(g, level, seg_start, seg_take, seg_bip, bip, width);
+            d_order.reserve(order.size());
+            SC_CUDA(cudaMemcpyAsync(d_order.get(), order.data(), order.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+            g->res_order_width[kind] = width;
+        }
+        const int32_t ngroups = static_cast<int32_t>(order.size() / width);
+        std::vector<int32_t> list;
+        for (int32_t q = 0; q < ngroups; ++q) {
+            int32_t Lg = 0;
+            for (int c = 0; c < width; ++c) {
+                const int32_t v = order[static_cast<size_t>(q) * width + c];
+                if (v >= 0) Lg = std::max(Lg, h_len[v]);
+            }
+            if (Lg > 0) {
+                list.push_back(q);
+                st->hops += Lg;
+            }
+        }
+        if (list.empty()) continue;
+        g->res_list.reserve(list.size());
+        g->res_over.reserve(list.size() + 1);
+        g->res_count.reserve(2);
+        SC_CUDA(cudaMemcpyAsync(g->res_list.get(), list.data(), list.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+        ResArgs a{};
+        a.row_ptr = g->row_ptr.get();
+        a.ell = g->res_ell.get();
+        a.inv_deg = fp64 ? static_cast<const void *>(g->inv_deg_d.get()) : static_cast<const void *>(g->inv_deg_f.get());
+        a.n = n;
+        a.order = d_order.get();
+        a.groups = g->res_list.get();
+        a.ngroups = static_cast<int32_t>(list.size());
+        a.len = g->res_len.get();
+        a.h0 = r.prec == SC_PREC_BF16 ? r.h0 : INT32_MAX;
+        a.tau = g->tau_entry.get();
+        a.g = g->acc_g.get();
+        a.t1 = g->acc_t1.get();
+        a.t2 = g->acc_t2.get();
+        a.rec = r.rec;
+        a.over = g->res_over.get();
+        // the first class: the one that holds the largest ball of a sample of the groups
+        int cls = 0;
+        auto cap_of = [&](int c) { return fp64 ? res_cap_of<double>(W, c, bip) : res_cap_of<float>(W, c, bip); };
+        int32_t seg_max = 0;
+        for (size_t i = 0; i + 1 < seg_start.size(); ++i)
+            if (seg_take[i] && (seg_bip[i] != 0) == bip) seg_max = std::max(seg_max, seg_start[i + 1] - seg_start[i]);
+        if (seg_max + width > cap_of(0)) {
+            std::vector<int32_t> pick;
+            const int32_t ns = std::min<int32_t>(kResSample, a.ngroups);
+            for (int32_t q = 0; q < ns; ++q) pick.push_back(list[static_cast<size_t>(q) * a.ngroups / ns]);
+            SC_CUDA(cudaMemcpyAsync(g->res_over.get(), pick.data(), ns * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+            SC_CUDA(cudaMemsetAsync(g->res_count.get(), 0, 2 * sizeof(int32_t), s));
+            ResArgs m = a;
+            m.groups = g->res_over.get();
+            m.ngroups = ns;
+            m.count = g->res_count.get();
+            res_dispatch(g, m, fp64, W, kResClasses - 2, bip, s);
+            ++st->launches;
+            int32_t h[2];
+            SC_CUDA(cudaMemcpyAsync(h, g->res_count.get(), sizeof(h), cudaMemcpyDeviceToHost, s));
+            SC_CUDA(cudaStreamSynchronize(s));
+            while (cls < kResClasses - 2 && h[0] > cap_of(cls)) ++cls;
+            if (h[1] == ns) cls = kResClasses - 1;  // no ball of the sample fits with its adjacency
+        }
+        for (; cls < kResClasses && !list.empty(); ++cls) {
+            if (cls == kResClasses - 1) {
+                // one source to a group, adjacency in global memory: bipartite graphs only (one
+                // buffer, half the rows a hop; without that the block kernels are as fast)
+                if (!bip) break;
+                std::vector<int32_t> single;
+                for (int32_t q : list)
+                    for (int c = 0; c < width; ++c) {
+                        const int32_t v = order[static_cast<size_t>(q) * width + c];
+                        if (v >= 0 && h_len[v] > 0) single.push_back(v);
+                    }
+                g->res_single.reserve(single.size());
+                g->res_over.reserve(single.size() + 1);
+                SC_CUDA(cudaMemcpyAsync(g->res_single.get(), single.data(), single.size() * sizeof(int32_t),
+                                        cudaMemcpyHostToDevice, s));
+                SC_CUDA(cudaStreamSynchronize(s));  // `single` goes out of scope
+                a.order = g->res_single.get();
+                a.groups = nullptr;
+                a.ngroups = static_cast<int32_t>(single.size());
+                a.over = g->res_over.get();
+                SC_CUDA(cudaMemsetAsync(g->res_over.get(), 0, sizeof(int32_t), s));
+                r.timed([&] { res_dispatch(g, a, fp64, W, cls, bip, s); });
+                ++st->launches;
+                std::vector<int32_t> over(single.size() + 1);
+                SC_CUDA(cudaMemcpyAsync(over.data(), g->res_over.get(), over.size() * sizeof(int32_t),
+                                        cudaMemcpyDeviceToHost, s));
+                SC_CUDA(cudaStreamSynchronize(s));
+                list.clear();
+                for (int32_t t = 0; t < over[0]; ++t) left.push_back(single[over[1 + t]]);
+                break;
+            }
+            SC_CUDA(cudaMemsetAsync(g->res_over.get(), 0, sizeof(int32_t), s));
+            a.groups = g->res_list.get();
+            a.ngroups = static_cast<int32_t>(list.size());
+            r.timed([&] { res_dispatch(g, a, fp64, W, cls, bip, s); });
+            ++st->launches;
+            int32_t nover = 0;
+            SC_CUDA(cudaMemcpyAsync(&nover, g->res_over.get(), sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+            SC_CUDA(cudaStreamSynchronize(s));
+            list.resize(nover);
+            if (nover > 0) {
+                SC_CUDA(cudaMemcpyAsync(list.data(), g->res_over.get() + 1, nover * sizeof(int32_t),
+                                        cudaMemcpyDeviceToHost, s));
+                SC_CUDA(cudaStreamSynchronize(s));
+                std::sort(list.begin(), list.end());
+                SC_CUDA(cudaMemcpyAsync(g->res_list.get(), list.data(), nover * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+            }
+        }
+        for (int32_t q : list)
+            for (int c = 0; c < width; ++c) {
+                const int32_t v = order[static_cast<size_t>(q) * width + c];
+                if (v >= 0 && h_len[v] > 0) left.push_back(v);
+            }
+    }
+    SC_CUDA(cudaStreamSynchronize(s));  // host vectors behind the async copies
+    std::sort(left.begin(), left.end());
+    return left;
+}
+
+}  // namespace sc
