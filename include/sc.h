@@ -321,12 +321,12 @@ sc_status sc_series_meet(sc_graph *g, const int32_t *tau, double *s_out);
    The values are the same again. */
 #define SC_OPT_WINDOWS_OFF 8u
 #define SC_OPT_WINDOWS_FORCE 16u
-/* Unwindowed TGT blocks compute hop 3 from the non-zero values of X_2 only,
-   and hop L-1 only on the sources' two-hop balls, where the last hop reads it
-   (Algorithm 2's frontier, which visits only nodes it reaches); the values are
-   those of full hops bit for bit. Off by default: on the power-law graphs
-   measured the hop is bound by the latency of its dependent loads per row, not
-   by the bytes it moves, and the full hop was as fast or faster. */
+/* Unwindowed blocks compute hops 2 and 3 from the non-zero values of X_1 and
+   X_2 only, and (TGT) hop L-1 only on the sources' two-hop balls, where the last
+   hop reads it (Algorithm 2's frontier, which visits only nodes it reaches); the
+   values are those of full hops bit for bit. Chosen automatically on graphs of at
+   least 16,384 nodes for blocks whose X_2 is sparse; this flag asks for it at any
+   size. */
 #define SC_OPT_SPARSE_HOPS 32u
 /* TGT+ switch tests find each column's gamma largest entries (Algorithm 3's
    candidates) from the entries at or above the gamma-th largest maximum of its
@@ -336,10 +336,11 @@ sc_status sc_series_meet(sc_graph *g, const int32_t *tau, double *s_out);
 
 /* kernel classes of the per-class timing in sc_report (SC_OPT_TIME_KERNELS) */
 #define SC_KC_DENSE_HOP 0   /* full hops (k_spmm_hop, or the TMA-gather hop), or a resident traversal */
-#define SC_KC_MASK_HOP 1    /* hops 1-2 from the sources' neighbour bits (k_mask_scatter + k_hop2_mask) */
-#define SC_KC_SPARSE_HOP 2  /* hop 3 from the non-zero values of X_2 (k_hop_sparse) */
-#define SC_KC_BALL_HOP 3    /* hop L-1 on the two-hop balls (k_hop_ball) */
-#define SC_KC_LAST_HOP 4    /* the last hop where its gather reads it (k_last_diag + k_last_rows) */
+#define SC_KC_MASK_HOP 1    /* hops 1-2 from the sources' neighbour bits (k_mask_scatter + k_hop2_mask, or
+                               k_front_scatter + k_front2) */
+#define SC_KC_SPARSE_HOP 2  /* hop 3 from the non-zero values of X_2 (k_front3) */
+#define SC_KC_BALL_HOP 3    /* hop L-1 on the two-hop balls (k_ball_rows + k_ball) */
+#define SC_KC_LAST_HOP 4    /* the last hop where its gather reads it (k_last_hop) */
 #define SC_KC_SWITCH_TEST 5 /* TGT+: a switch test (CalChi's column statistics, chi and R per entry, the
                                copy of the counts and the host's wait for it) */
 #define SC_KC_WALKS 6       /* TGT+: a walk phase (walk counts, the host's plan, the walk kernels) */

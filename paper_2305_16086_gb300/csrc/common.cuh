@@ -145,6 +145,8 @@ struct sc_graph {
     sc::DevBuf<double> inv_deg_d;
     std::vector<int32_t> h_row_ptr;  // host copy of the row pointers (degrees, scheduling)
 
+    std::vector<int32_t> h_walk2;    // per node: sum of its neighbours' degrees, empty until needed
+
     // row schedule of the SIMT propagation kernel: heavy rows (degree above
     // the threshold, one CTA each, longest first) then light rows in order
     sc::DevBuf<int32_t> row_order;
@@ -157,11 +159,16 @@ struct sc_graph {
     int32_t bandwidth = -1;
     // per-slice windows of windowed launches
     sc::DevBuf<unsigned char> win_list;
-    // bit mask of the block's first-hop rows (hop 2 from the sources alone),
-    // and the non-zero columns of X_2 (hop 3 from its non-zero values)
-    sc::DevBuf<uint32_t> mask, mask_nz;
-    // X_L at the sources (the last hop, computed where the gather reads it)
-    sc::DevBuf<double> last_diag;
+    // bit mask of the block's first-hop rows (hop 2 from the sources alone); behind it the
+    // non-zero columns of X_2 and the counters of the sparse hops
+    sc::DevBuf<uint32_t> mask;
+    // the sparse hops: chunks of the long rows and runs of the others (laid out once), partial sums, X_2's
+    // sector masks, the work lists of the ball hop
+    sc::DevBuf<int32_t> fr_hi_row, fr_hi_k0, fr_hv_id, fr_hv_first, fr_run_lo, fr_run_hi, fr_rows;
+    sc::DevBuf<uint32_t> fr_pairs;
+    sc::DevBuf<unsigned char> fr_part, fr_sec;
+    int32_t front_hchunks = 0, front_hrows = 0, front_runs = 0;
+    bool front_ready = false;
     // row runs of about equal CSR entries, one per warp, for the TMA kernel
     sc::DevBuf<int32_t> part;
     int32_t nparts = 0;

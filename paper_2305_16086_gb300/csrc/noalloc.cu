@@ -158,6 +158,10 @@ __global__ void k_na_combine(const int32_t *__restrict__ row_ptr, const int32_t 
     }
 }
 
+// CTAs per source in the last hop: the degrees are on the device, so a fixed number (a source of
+// up to 64 neighbours in one round; CTAs past a source's degree return at once)
+constexpr int kNoallocLastCtas = 8;
+
 static size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 // bytes of scratch one call needs (FP64 blocks of 32 sources)
@@ -254,8 +258,8 @@ static void noalloc_impl(int32_t n, int64_t nnz, const int32_t *row_ptr, const i
             std::swap(a, b);
         }
         if (ell >= 2)  // the last hop only where the gather reads it, with the gathers of hops ell-1, ell
-            k_last_hop<double, B><<<nb, kSpmmWarps * 32, 0, s>>>(row_ptr, col_idx, inv_deg, a, n, bsrc, nb, tau,
-                                                                  ell, acc, nullptr, nullptr, GatherRec{0, nullptr, 0});
+            k_last_hop<double, B><<<dim3(nb, kNoallocLastCtas), kSpmmWarps * 32, 0, s>>>(
+                row_ptr, col_idx, inv_deg, a, n, bsrc, nb, tau, ell, acc, nullptr, nullptr, GatherRec{0, nullptr, 0});
         else
             k_gather<double, B><<<nb, 128, 0, s>>>(row_ptr, col_idx, a, n, bsrc, nb, tau, ell, acc, nullptr, nullptr,
                                                    GatherRec{0, nullptr, 0}, nullptr);

@@ -32,6 +32,16 @@ long long tgtplus_walks(sc_graph *g, int prec, int B, const void *x, const int32
                         long long *steps_out);
 constexpr int kCostRuleHops = 4;  // the cost rule tests the last hops only
 constexpr int kEvenDepthCap = 16;  // TGT+ at learned lengths: even hops recorded for the check (hop <= 16)
+// A block's hops 2, 3 and L-1 skip what is zero or not read (sparse_hops.cuh) when the graph is
+// large and the block's X_2 sparse, by an upper bound of its density: the walks of two hops from
+// its sources over sources x nodes. Whole calls at 7 hops, full hops against sparse ones, FP32:
+// Barabasi-Albert (10 edges a node) 200,000 nodes (density 0.2 to 3%) 1009 -> 788 ms, 60,000 (0.6
+// to 10%) 110 -> 102 ms, 20,000 (2 to 26%) 13.7 -> 13.6 ms; FP64 20,000 92 -> 78 ms; tree + G(n, p)
+// 50,000 at 9 hops (0.2%) 72 -> 67 ms; R-MAT scale 15 (14% and more) 54.4 -> 56.8 ms: the line lies
+// at a tenth. TGT+ has no ball hop and takes the rest only where a block does not fit in L2 (its
+// tests and walks read the blocks in full).
+constexpr int32_t kSparseMinNodes = 16384;
+constexpr double kSparseDensity = 0.1;
 constexpr int kTuneHops = 8;       // hops of the sample block that picks the block width
 // TGT+ cost rule rates measured on GB300: a hop costs about this much per
 // source and CSR entry (BA-200k, FP32 blocks: 1.1 us per source over 4.0M
@@ -330,14 +340,10 @@ static void first_gather_p(const sc_graph *g, int B, bool first, const void *x, 
 template <typename T, int B>
 static void last_hop_t(sc_graph *g, const void *x, const int32_t *src, int nsrc, int max_deg, const int32_t *tau,
                        int ell, double *a, double *b, double *c, const GatherRec &rec, cudaStream_t s) {
-    g->last_diag.reserve(nsrc);
-    k_last_diag<T, B><<<nsrc, kSpmmWarps * 32, 0, s>>>(g->row_ptr.get(), g->col_idx.get(), inv_deg_of<T>(g),
-                                                      static_cast<const T *>(x), g->n, src, nsrc, tau, ell, a, b, c,
-                                                      rec, g->last_diag.get());
-    dim3 grid(nsrc, std::min(ceil_div(std::max(max_deg, 1), kSpmmWarps), 65535));
-    k_last_rows<T, B><<<grid, kSpmmWarps * 32, 0, s>>>(g->row_ptr.get(), g->col_idx.get(), inv_deg_of<T>(g),
-                                                      static_cast<const T *>(x), g->n, src, nsrc, tau, ell, a, b, c,
-                                                      rec, g->last_diag.get());
+    dim3 grid(nsrc, std::min(ceil_div(std::max(max_deg, 1), kLastPerCta), 65535));
+    k_last_hop<T, B><<<grid, kSpmmWarps * 32, 0, s>>>(g->row_ptr.get(), g->col_idx.get(), inv_deg_of<T>(g),
+                                                     static_cast<const T *>(x), g->n, src, nsrc, tau, ell, a, b, c,
+                                                     rec);
 }
 
 template <typename T>
@@ -354,8 +360,7 @@ static void last_hop_p(sc_graph *g, int B, const void *x, const int32_t *src, in
 
 template <typename T, int B>
 static void hop2_mask_t(const sc_graph *g, uint32_t *mask, void *x2, int slices, const int32_t *src, int nsrc,
-                        const int32_t *tau, double *a, double *b, double *c, const GatherRec &rec, uint32_t *nz,
-                        cudaStream_t s) {
+                        const int32_t *tau, double *a, double *b, double *c, const GatherRec &rec, cudaStream_t s) {
     k_mask_scatter<B><<<nsrc, 128, 0, s>>>(g->row_ptr.get(), g->col_idx.get(), src, nsrc, mask, g->n);
     MaskHopArgs<T> m{};
     m.row_ptr = g->row_ptr.get();
@@ -376,109 +381,184 @@ static void hop2_mask_t(const sc_graph *g, uint32_t *mask, void *x2, int slices,
     m.t1 = b;
     m.t2 = c;
     m.rec = rec;
-    m.nz = nz;
     dim3 grid(m.gather_ctas + m.n_heavy + m.light_ctas, slices);
     k_hop2_mask<T, B><<<grid, kSpmmWarps * 32, 0, s>>>(m);
 }
 
 template <typename T>
 static void hop2_mask_p(const sc_graph *g, int B, uint32_t *mask, void *x2, int slices, const int32_t *src, int nsrc,
-                        const int32_t *tau, double *a, double *b, double *c, const GatherRec &rec, uint32_t *nz,
-                        cudaStream_t s) {
+                        const int32_t *tau, double *a, double *b, double *c, const GatherRec &rec, cudaStream_t s) {
     switch (B) {
-    case 32: hop2_mask_t<T, 32>(g, mask, x2, slices, src, nsrc, tau, a, b, c, rec, nz, s); break;
-    case 64: hop2_mask_t<T, 64>(g, mask, x2, slices, src, nsrc, tau, a, b, c, rec, nz, s); break;
-    case 128: hop2_mask_t<T, 128>(g, mask, x2, slices, src, nsrc, tau, a, b, c, rec, nz, s); break;
+    case 32: hop2_mask_t<T, 32>(g, mask, x2, slices, src, nsrc, tau, a, b, c, rec, s); break;
+    case 64: hop2_mask_t<T, 64>(g, mask, x2, slices, src, nsrc, tau, a, b, c, rec, s); break;
+    case 128: hop2_mask_t<T, 128>(g, mask, x2, slices, src, nsrc, tau, a, b, c, rec, s); break;
     default: SC_FAIL(SC_ERR_INVALID_ARG, "block width %d", B);
     }
 }
 
 // hops 1 and 2 of a block from its sources alone (X_1 is never stored): marks
-// N(s_b) in a bit mask (zeroed here), computes X_2 into x2 and gathers hop 1;
-// with want_nz also the non-zero columns of X_2 (into g->mask_nz)
+// N(s_b) in a bit mask (zeroed here), computes X_2 into x2 and gathers hop 1
 void launch_hop2_mask(sc_graph *g, int prec, int B, void *x2, int slices, const int32_t *src, int nsrc,
-                      const int32_t *tau, double *a, double *b, double *cc, const GatherRec &rec, bool want_nz,
-                      cudaStream_t s) {
+                      const int32_t *tau, double *a, double *b, double *cc, const GatherRec &rec, cudaStream_t s) {
     const size_t words = static_cast<size_t>(slices) * g->n * (B / 32);
     g->mask.reserve(words);
-    uint32_t *nz = nullptr;
-    if (want_nz) {
-        g->mask_nz.reserve(words);
-        nz = g->mask_nz.get();
-    }
     SC_CUDA(cudaMemsetAsync(g->mask.get(), 0, words * sizeof(uint32_t), s));
     switch (prec) {
-    case SC_PREC_FP64: hop2_mask_p<double>(g, B, g->mask.get(), x2, slices, src, nsrc, tau, a, b, cc, rec, nz, s); break;
-    case SC_PREC_FP32: hop2_mask_p<float>(g, B, g->mask.get(), x2, slices, src, nsrc, tau, a, b, cc, rec, nz, s); break;
+    case SC_PREC_FP64: hop2_mask_p<double>(g, B, g->mask.get(), x2, slices, src, nsrc, tau, a, b, cc, rec, s); break;
+    case SC_PREC_FP32: hop2_mask_p<float>(g, B, g->mask.get(), x2, slices, src, nsrc, tau, a, b, cc, rec, s); break;
     case SC_PREC_BF16:
-        hop2_mask_p<__nv_bfloat16>(g, B, g->mask.get(), x2, slices, src, nsrc, tau, a, b, cc, rec, nz, s);
+        hop2_mask_p<__nv_bfloat16>(g, B, g->mask.get(), x2, slices, src, nsrc, tau, a, b, cc, rec, s);
         break;
     }
     SC_LAUNCH_CHECK();
 }
 
+// ---- the sparse ends of a block (sparse_hops.cuh) -----------------------------
+// the rows above kFrontHeavy entries cut into chunks, the others in runs; laid out once per graph
+static void ensure_front(sc_graph *g) {
+    if (g->front_ready) return;
+    std::vector<int32_t> hi_row, hi_k0, hv_id, hv_first, run_lo, run_hi;
+    int32_t lo = 0;  // first row of the open run
+    auto close_run = [&](int32_t r) {
+        if (r > lo) {
+            run_lo.push_back(lo);
+            run_hi.push_back(r);
+        }
+        lo = r;
+    };
+    for (int32_t r = 0; r < g->n; ++r) {
+        const int32_t b = g->h_row_ptr[r], e = g->h_row_ptr[r + 1];
+        if (r - lo == kFrontRunRows || e - g->h_row_ptr[lo] > kFrontRun || e - b > kFrontHeavy) close_run(r);
+        if (e - b <= kFrontHeavy) continue;
+        lo = r + 1;
+        hv_first.push_back(static_cast<int32_t>(hi_row.size()));
+        hv_id.push_back(r);
+        for (int32_t k = b; k < e; k += kChunk) {
+            hi_row.push_back(static_cast<int32_t>(hv_id.size()) - 1);
+            hi_k0.push_back(k);
+        }
+    }
+    close_run(g->n);
+    hv_first.push_back(static_cast<int32_t>(hi_row.size()));
+    auto put = [&](DevBuf<int32_t> &d, const std::vector<int32_t> &h) {
+        d.reserve(std::max<size_t>(h.size(), 1));
+        if (!h.empty())
+            SC_CUDA(cudaMemcpyAsync(d.get(), h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice, g->stream));
+    };
+    put(g->fr_hi_row, hi_row);
+    put(g->fr_hi_k0, hi_k0);
+    put(g->fr_hv_id, hv_id);
+    put(g->fr_hv_first, hv_first);
+    put(g->fr_run_lo, run_lo);
+    put(g->fr_run_hi, run_hi);
+    SC_CUDA(cudaStreamSynchronize(g->stream));
+    g->front_hchunks = static_cast<int32_t>(hi_row.size());
+    g->front_hrows = static_cast<int32_t>(hv_id.size());
+    g->front_runs = static_cast<int32_t>(run_lo.size());
+    g->front_ready = true;
+}
+
+struct FrontLaunch {
+    int which;  // 2: hop 2 (X_2's non-zero sectors into xn), 3: hop 3, 0: the ball hop
+    const void *xp;
+    void *xn;
+    int slices;
+    const int32_t *src;
+    int nsrc;
+    const int32_t *tau;
+    int gather_ell;
+    double *g, *t1, *t2;
+    GatherRec rec;
+    bool lists;  // make the ball hop's work lists (with hop 3, or after hop 2)
+};
+
 template <typename T, int B>
-static void hop_sparse_t(const sc_graph *g, bool ball, const void *xp, void *xn, int slices, const uint32_t *mask,
-                         const int32_t *src, int nsrc, const int32_t *tau, int gather_ell, double *a, double *b,
-                         double *c, const GatherRec &rec, cudaStream_t s) {
-    SparseHopArgs<T> h{};
-    h.row_ptr = g->row_ptr.get();
-    h.col = g->col_idx.get();
-    h.inv_deg = inv_deg_of<T>(g);
-    h.x_prev = static_cast<const T *>(xp);
-    h.x_next = static_cast<T *>(xn);
-    h.mask = mask;
-    h.n = g->n;
-    h.row_order = g->row_order.get();
-    h.n_heavy = g->n_heavy;
-    h.heavy_t = g->heavy_threshold_cached;
-    h.src = src;
-    h.nsrc = nsrc;
-    h.tau = tau;
-    h.gather_ell = gather_ell;
-    h.g = a;
-    h.t1 = b;
-    h.t2 = c;
-    h.rec = rec;
-    h.gather_ctas = gather_ell > 0 ? B : 0;
-    h.heavy_ctas = g->n_heavy;
-    h.light_ctas = light_ctas_for(g->n, kSpmmWarps, g->num_sms);  // one light row per warp
-    dim3 grid(h.gather_ctas + g->n_heavy + h.light_ctas, slices);
-    if (ball) k_hop_ball<T, B><<<grid, kSpmmWarps * 32, 0, s>>>(h);
-    else k_hop_sparse<T, B><<<grid, kSpmmWarps * 32, 0, s>>>(h);
+static void front_t(sc_graph *g, const FrontLaunch &h, cudaStream_t s) {
+    using Acc = typename AccOf<T>::type;
+    FrontArgs<T> a{};
+    a.row_ptr = g->row_ptr.get();
+    a.col = g->col_idx.get();
+    a.inv_deg = inv_deg_of<T>(g);
+    a.x_prev = static_cast<const T *>(h.xp);
+    a.x_next = static_cast<T *>(h.xn);
+    a.n = g->n;
+    a.hi_row = g->fr_hi_row.get();
+    a.hi_k0 = g->fr_hi_k0.get();
+    a.hv_id = g->fr_hv_id.get();
+    a.hv_first = g->fr_hv_first.get();
+    a.nhchunks = g->front_hchunks;
+    a.nhrows = g->front_hrows;
+    a.run_lo = g->fr_run_lo.get();
+    a.run_hi = g->fr_run_hi.get();
+    a.nruns = g->front_runs;
+    g->fr_part.reserve(std::max<size_t>(static_cast<size_t>(h.slices) * a.nhchunks * B * sizeof(Acc), 16));
+    a.part = reinterpret_cast<Acc *>(g->fr_part.get());
+    // one buffer zeroed per block: mask, nz, any, the arrivals of the three hops, the list lengths
+    const size_t words = static_cast<size_t>(h.slices) * g->n * (B / 32);
+    const size_t marks = static_cast<size_t>(h.slices) * ceil_div(g->n, 32);
+    const size_t arrivals = static_cast<size_t>(h.slices) * a.nhrows;
+    const size_t total = 2 * words + marks + 3 * arrivals + static_cast<size_t>(h.slices) * kBallLists;
+    g->mask.reserve(total);
+    a.mask = g->mask.get();
+    a.nz = a.mask + words;
+    a.any = a.nz + words;
+    int32_t *arrived = reinterpret_cast<int32_t *>(a.any + marks);
+    a.arrived = arrived + (h.which == 2 ? 0 : h.which == 3 ? 1 : 2) * arrivals;
+    a.lists = arrived + 3 * arrivals;
+    const size_t nodes = static_cast<size_t>(h.slices) * g->n;
+    g->fr_sec.reserve(nodes * sizeof(typename SectorMask<T, B>::Word));
+    a.sectors = g->fr_sec.get();
+    if (h.lists || h.which == 0) {
+        g->fr_pairs.reserve(4 * nodes * kBallSparseCols);
+        g->fr_rows.reserve(nodes);
+        a.pairs = g->fr_pairs.get();
+        a.rows = g->fr_rows.get();
+    }
+    const int sms = g->num_sms > 0 ? g->num_sms : 148;
+    a.gather_ctas = B;
+    a.src = h.src;
+    a.nsrc = h.nsrc;
+    a.tau = h.tau;
+    a.gather_ell = h.gather_ell;
+    a.g = h.g;
+    a.t1 = h.t1;
+    a.t2 = h.t2;
+    a.rec = h.rec;
+    const int heavy = ceil_div(a.nhchunks, kSpmmWarps), threads = kSpmmWarps * 32;
+    if (h.which == 2) {
+        SC_CUDA(cudaMemsetAsync(g->mask.get(), 0, total * sizeof(uint32_t), s));
+        k_front_scatter<B><<<h.nsrc, 128, 0, s>>>(g->row_ptr.get(), g->col_idx.get(), h.src, h.nsrc, a.mask, a.any, g->n);
+        k_front2<T, B><<<dim3(B + ceil_div(a.nhchunks + a.nruns, kSpmmWarps), h.slices), threads, 0, s>>>(a);
+        if (h.lists) k_front_lists<T, B><<<dim3(ceil_div(g->n, threads), h.slices), threads, 0, s>>>(a);
+    } else if (h.which == 3) {
+        a.list_ctas = h.lists ? std::min(ceil_div(g->n, threads), 4 * sms) : 0;
+        a.light_ctas = light_ctas_for(g->n, kSpmmWarps, sms);
+        k_front3<T, B><<<dim3(B + heavy + a.list_ctas + a.light_ctas, h.slices), threads, 0, s>>>(a);
+    } else {
+        // the lists' lengths are on the device: as many warps as the chip holds
+        k_ball_rows<T, B><<<dim3(heavy + 2 * sms, h.slices), threads, 0, s>>>(a);
+        k_ball<T, B><<<dim3(B + sms * (48 / kSpmmWarps), h.slices), threads, 0, s>>>(a);
+    }
+    SC_LAUNCH_CHECK();
 }
 
 template <typename T>
-static void hop_sparse_p(const sc_graph *g, int B, bool ball, const void *xp, void *xn, int slices,
-                         const uint32_t *mask, const int32_t *src, int nsrc, const int32_t *tau, int gather_ell,
-                         double *a, double *b, double *c, const GatherRec &rec, cudaStream_t s) {
+static void front_p(sc_graph *g, int B, const FrontLaunch &h, cudaStream_t s) {
     switch (B) {
-    case 32: hop_sparse_t<T, 32>(g, ball, xp, xn, slices, mask, src, nsrc, tau, gather_ell, a, b, c, rec, s); break;
-    case 64: hop_sparse_t<T, 64>(g, ball, xp, xn, slices, mask, src, nsrc, tau, gather_ell, a, b, c, rec, s); break;
-    case 128: hop_sparse_t<T, 128>(g, ball, xp, xn, slices, mask, src, nsrc, tau, gather_ell, a, b, c, rec, s); break;
+    case 32: front_t<T, 32>(g, h, s); break;
+    case 64: front_t<T, 64>(g, h, s); break;
+    case 128: front_t<T, 128>(g, h, s); break;
     default: SC_FAIL(SC_ERR_INVALID_ARG, "block width %d", B);
     }
 }
 
-// hop `gather_ell + 1` of a block from X_{gather_ell} (xp) into xn with the
-// fused gather of X_{gather_ell}: ball = false: the full hop reading only the
-// non-zero values of xp (mask = their columns, g->mask_nz); ball = true: the
-// values on the sources' two-hop balls only (mask = the neighbour bits, g->mask)
-void launch_hop_sparse(const sc_graph *g, int prec, int B, bool ball, const void *xp, void *xn, int slices,
-                       const uint32_t *mask, const int32_t *src, int nsrc, const int32_t *tau, int gather_ell,
-                       double *a, double *b, double *cc, const GatherRec &rec, cudaStream_t s) {
+static void launch_front(sc_graph *g, int prec, int B, const FrontLaunch &h, cudaStream_t s) {
+    ensure_front(g);
     switch (prec) {
-    case SC_PREC_FP64:
-        hop_sparse_p<double>(g, B, ball, xp, xn, slices, mask, src, nsrc, tau, gather_ell, a, b, cc, rec, s);
-        break;
-    case SC_PREC_FP32:
-        hop_sparse_p<float>(g, B, ball, xp, xn, slices, mask, src, nsrc, tau, gather_ell, a, b, cc, rec, s);
-        break;
-    case SC_PREC_BF16:
-        hop_sparse_p<__nv_bfloat16>(g, B, ball, xp, xn, slices, mask, src, nsrc, tau, gather_ell, a, b, cc, rec, s);
-        break;
+    case SC_PREC_FP64: front_p<double>(g, B, h, s); break;
+    case SC_PREC_FP32: front_p<float>(g, B, h, s); break;
+    case SC_PREC_BF16: front_p<__nv_bfloat16>(g, B, h, s); break;
     }
-    SC_LAUNCH_CHECK();
 }
 
 // hop `ell` (the block's last) computed only where its gather reads it, with
@@ -790,6 +870,34 @@ __global__ void k_learned_check(const int32_t *__restrict__ row_ptr, const int32
     }
 }
 
+// out[r] = sum of the degrees of r's neighbours (the walks of two hops), at most 2^31 - 1
+__global__ void k_walk2(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col, int32_t n,
+                        int32_t *__restrict__ out) {
+    const int32_t r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (r >= n) return;
+    long long sum = 0;
+    for (int32_t k = row_ptr[r] + lane; k < row_ptr[r + 1]; k += 32) {
+        const int32_t j = col[k];
+        sum += row_ptr[j + 1] - row_ptr[j];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) out[r] = static_cast<int32_t>(min(sum, static_cast<long long>(INT32_MAX)));
+}
+
+static void ensure_walk2(sc_graph *g) {
+    if (!g->h_walk2.empty()) return;
+    DevBuf<int32_t> d;
+    d.reserve(g->n);
+    k_walk2<<<ceil_div(g->n, 8), 256, 0, g->stream>>>(g->row_ptr.get(), g->col_idx.get(), g->n, d.get());
+    SC_LAUNCH_CHECK();
+    std::vector<int32_t> h(g->n);
+    SC_CUDA(cudaMemcpyAsync(h.data(), d.get(), g->n * sizeof(int32_t), cudaMemcpyDeviceToHost, g->stream));
+    SC_CUDA(cudaStreamSynchronize(g->stream));
+    g->h_walk2.swap(h);
+}
+
 // per-source maximum of tau over its row
 __global__ void k_row_max(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ tau, int32_t n,
                           int32_t *__restrict__ out) {
@@ -902,6 +1010,7 @@ struct Run {
     int32_t h0 = 0x7fffffff;  // SC_PREC_BF16: first hop stored in bf16 (fp32 before)
     std::vector<int32_t> *depth = nullptr;  // TGT+: per node, the last hop its traversal reached
     bool capture = false;  // windowed loop: record into one CUDA graph
+    bool full_hops = false;  // no sparse hops
     // statistics
     int64_t launches = 0, hops = 0, source_hops = 0, hop_launches = 0, walks = 0, graph_launches = 0, walk_steps = 0;
     // per kernel class (SC_KC_*): event pairs (index into the graph's pool) and algorithmic bytes
@@ -1021,7 +1130,11 @@ static void run_blocks(Run &R, std::vector<int32_t> sources, const std::vector<i
     auto test_bytes_per_slice = [&](int32_t ell) {
         return static_cast<double>(n) * B * elem_size(prec_at(R, ell)) + 4.0 * n;
     };
-    const bool dense_only = (R.o->flags & SC_OPT_SPARSE_HOPS) == 0;
+    const bool sparse_asked = !R.full_hops && (R.o->flags & SC_OPT_SPARSE_HOPS) != 0;
+    const bool sparse_fits = static_cast<int64_t>(n) * B < (int64_t(1) << 32);  // 32-bit places in a block
+    const bool sparse_auto = !R.full_hops && !sparse_asked && n >= kSparseMinNodes && sparse_fits &&
+                             (!R.plus || 2.0 * static_cast<double>(R.slice_bytes) > 0.6 * static_cast<double>(g->l2_bytes));
+    if (sparse_auto) ensure_walk2(g);
     const bool full_scan = (R.o->flags & SC_OPT_FULL_TOPGAMMA_SCAN) != 0;
     // cost rule: the hop at which the previous block of the same length switched (-1: none
     // yet). Blocks come longest first and neighbouring blocks switch within a hop of each
@@ -1048,18 +1161,33 @@ static void run_blocks(Run &R, std::vector<int32_t> sources, const std::vector<i
         // hop 3 from X_2's non-zero values (a full hop: L >= 5 keeps it before hop L - 1), and
         // hop L - 1 on the sources' two-hop balls (read by the sparse last hop only: TGT, whose
         // traversal nothing else reads; no storage change around it)
-        const bool hop3_sparse = from_mask && !dense_only && L >= 5 && prec_at(R, 2) == prec_at(R, 3);
-        const bool ball_hop = from_mask && !dense_only && !R.plus && L >= 4 && prec_at(R, L - 2) == prec_at(R, L - 1) &&
+        bool sparse = sparse_asked && sparse_fits;
+        if (sparse_auto) {
+            double reach = 0.0;
+            for (int q = 0; q < nsrc; ++q) reach += std::min(g->h_walk2[sources[first + q]], n);
+            sparse = reach < kSparseDensity * static_cast<double>(nsrc) * n;
+        }
+        // (a TGT+ test after hop 2 reads X_2 in full)
+        const bool hop3_sparse = from_mask && sparse && L >= 5 && prec_at(R, 2) == prec_at(R, 3) &&
+                                 !(R.plus && 2 >= L - kCostRuleHops);
+        const bool ball_hop = from_mask && sparse && !R.plus && L >= 4 && prec_at(R, L - 2) == prec_at(R, L - 1) &&
                               prec_at(R, L - 1) == prec_at(R, L);
         int ell0 = 2;
         if (from_mask) {
             const int64_t t = timer_open(R, s);
-            launch_hop2_mask(g, prec_at(R, 2), B, xb, used_slices, src, nsrc, g->tau_entry.get(), g->acc_g.get(),
-                             g->acc_t1.get(), g->acc_t2.get(), R.rec, hop3_sparse, s);
-            timer_close(R, t, SC_KC_MASK_HOP,
-                        used_slices * (csr_bytes + (hop3_sparse ? 3.0 : 2.0) * mask_bytes +
-                                       static_cast<double>(n) * B * elem_size(prec_at(R, 2))),
-                        s);
+            const double x2_bytes = static_cast<double>(n) * B * elem_size(prec_at(R, 2));
+            if (hop3_sparse || ball_hop) {
+                if (!hop3_sparse) SC_CUDA(cudaMemsetAsync(xb, 0, used_slices * R.slice_bytes, s));  // X_2 is read in full
+                launch_front(g, prec_at(R, 2), B, FrontLaunch{2, nullptr, xb, used_slices, src, nsrc, g->tau_entry.get(), 1,
+                                                              g->acc_g.get(), g->acc_t1.get(), g->acc_t2.get(), R.rec,
+                                                              ball_hop && !hop3_sparse}, s);
+                timer_close(R, t, SC_KC_MASK_HOP,
+                            used_slices * (csr_bytes + 3.0 * mask_bytes + (hop3_sparse ? 0.0 : x2_bytes)), s);
+            } else {
+                launch_hop2_mask(g, prec_at(R, 2), B, xb, used_slices, src, nsrc, g->tau_entry.get(), g->acc_g.get(),
+                                 g->acc_t1.get(), g->acc_t2.get(), R.rec, s);
+                timer_close(R, t, SC_KC_MASK_HOP, used_slices * (csr_bytes + 2.0 * mask_bytes + x2_bytes), s);
+            }
             std::swap(xa, xb);
             R.launches += 2;
             ell0 = 3;
@@ -1166,7 +1294,7 @@ static void run_blocks(Run &R, std::vector<int32_t> sources, const std::vector<i
                 launch_last_hop(g, prec_at(R, ell), B, xa, src, nsrc, max_deg, g->tau_entry.get(), ell,
                                 g->acc_g.get(), g->acc_t1.get(), g->acc_t2.get(), R.rec, s);
                 timer_close(R, t, SC_KC_LAST_HOP, 0.0, s);
-                R.launches += 2;
+                R.launches += 1;
                 last_done = true;
                 break;
             }
@@ -1175,11 +1303,12 @@ static void run_blocks(Run &R, std::vector<int32_t> sources, const std::vector<i
                 // fused gather of X_{ell-1}
                 const bool ball = ell == L - 1 && ball_hop;
                 const int64_t t = timer_open(R, s);
-                launch_hop_sparse(g, prec_at(R, ell), B, ball, xa, xb, used_slices,
-                                  ball ? g->mask.get() : g->mask_nz.get(), src, nsrc, g->tau_entry.get(), ell - 1,
-                                  g->acc_g.get(), g->acc_t1.get(), g->acc_t2.get(), R.rec, s);
+                launch_front(g, prec_at(R, ell), B, FrontLaunch{ball ? 0 : 3, xa, xb, used_slices, src, nsrc,
+                                                                g->tau_entry.get(), ell - 1, g->acc_g.get(),
+                                                                g->acc_t1.get(), g->acc_t2.get(), R.rec,
+                                                                !ball && ball_hop}, s);
                 timer_close(R, t, ball ? SC_KC_BALL_HOP : SC_KC_SPARSE_HOP,
-                            used_slices * (csr_bytes + mask_bytes +
+                            used_slices * (csr_bytes + (ball ? 2.0 : 1.0) * mask_bytes +
                                            (ball ? 0.0 : static_cast<double>(n) * B * elem_size(prec_at(R, ell)))),
                             s);
                 std::swap(xa, xb);
@@ -1590,6 +1719,9 @@ static TuneResult pick_block_width(const Run &base, const std::vector<TuneResult
             R.slices = slices_for(g, c.B, elem, base.o->max_slices);
             R.slice_bytes = static_cast<size_t>(n) * c.B * elem;
             R.plus = false;
+            // a TGT+ block's switch hop, and so its walks, depend on the block width: it is chosen on
+            // the full hops alike whether or not the run may take the sparse ones
+            R.full_hops = base.plus;
             R.time_kernels = false;
             R.depth = nullptr;
             R.capture = false;

@@ -474,32 +474,62 @@ __global__ void k_gather(const int32_t *__restrict__ row_ptr, const int32_t *__r
 // in the summation order of k_spmm_hop (chunks of 32 consecutive entries
 // summed in order, chunk sums added in chunk order, one scale by 1/d), then
 // rounded to the storage type: the value a full hop would have stored.
-// xs: column b of X_{ell-1}, rows addressed from `base`.
+// xs: column b of X_{ell-1}, rows addressed from `base`. The lanes load
+// kValueChunks chunks together (lane t: entry t of each) into the warp's tile,
+// where lane c adds chunk c in order: two round trips per kValueChunks chunks.
+constexpr int kValueChunks = 16;
+
 template <typename T, int B>
 __device__ __forceinline__ double hop_value(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
                                             const typename AccOf<T>::type *__restrict__ inv_deg,
-                                            const T *__restrict__ xs, int32_t base, int32_t r, int lane) {
+                                            const T *__restrict__ xs, int32_t base, int32_t r, int lane,
+                                            typename AccOf<T>::type (*tile)[kChunk + 1]) {
     using Acc = typename AccOf<T>::type;
     const int32_t rb = row_ptr[r], re = row_ptr[r + 1];
+    const Acc sc = inv_deg[r];
     Acc acc = Acc(0);
-    for (int32_t c0 = rb; c0 < re; c0 += 32 * kChunk) {  // 32 chunks per round, lane l sums chunk l
-        const int32_t kb = c0 + lane * kChunk, ke = min(kb + kChunk, re);
+    for (int32_t c0 = rb; c0 < re; c0 += kValueChunks * kChunk) {
+        int32_t j[kValueChunks];
+#pragma unroll
+        for (int c = 0; c < kValueChunks; ++c) {
+            const int32_t k = c0 + c * kChunk + lane;
+            j[c] = k < re ? col[k] : -1;
+        }
+        Acc v[kValueChunks];
+#pragma unroll
+        for (int c = 0; c < kValueChunks; ++c)
+            v[c] = j[c] >= 0 ? to_acc(xs[static_cast<int64_t>(j[c] - base) * B]) : Acc(0);
+#pragma unroll
+        for (int c = 0; c < kValueChunks; ++c) tile[c][lane] = v[c];
+        __syncwarp();
         Acc chunk = Acc(0);
+        if (lane < kValueChunks) {
+            const int cnt = min(kChunk, re - (c0 + lane * kChunk));  // <= 0: no such chunk
 #pragma unroll 8
-        for (int32_t k = kb; k < ke; ++k) chunk += to_acc(xs[static_cast<int64_t>(col[k] - base) * B]);
-        const int nch = min(32, (re - c0 + kChunk - 1) / kChunk);  // chunks in this round (warp-uniform)
-        for (int l = 0; l < nch; ++l) acc += __shfl_sync(0xffffffffu, chunk, l);
+            for (int t = 0; t < cnt; ++t) chunk += tile[lane][t];
+        }
+        __syncwarp();
+        const int nch = min(kValueChunks, (re - c0 + kChunk - 1) / kChunk);  // chunks in this round (warp-uniform)
+        for (int c = 0; c < nch; ++c) acc += __shfl_sync(0xffffffffu, chunk, c);
     }
-    acc *= inv_deg[r];
+    acc *= sc;
     return static_cast<double>(to_acc(from_acc<T>(acc)));
 }
 
 // The last hop of a block, fused with the gathers of X_{ell-1} and X_ell
 // (ell = the block's last hop, Algorithm 2's hop and accumulation): X_ell is only read at each
 // source and its neighbours, so only those values are computed, one warp per
-// value, instead of the whole n x B block. One CTA per source; the values are
-// those of a full hop (hop_value), so the result is bit for bit the one of
-// k_spmm_hop followed by k_gather.
+// value, instead of the whole n x B block; the values are those of a full hop
+// (hop_value), so the result is bit for bit the one of k_spmm_hop followed by
+// k_gather. The CTAs of a source (blockIdx.y) share its neighbours, kLastPerCta
+// at a time, so that a hub spreads over many; each computes X_ell[s, b] for
+// itself (a hub's row is read a few times over, which costs less than a launch
+// of its own for the diagonals). Bound by latency: four dependent round trips
+// (bounds, ids, values, sums), 10 us a launch for 128 sources of a 200,000-node
+// Barabasi-Albert graph; a lane per chunk with 32 loads one after the other, and a
+// launch for the diagonals, took 38 us.
+constexpr int kLastPerCta = 2 * kSpmmWarps;
+
 template <typename T, int B>
 __global__ void __launch_bounds__(kSpmmWarps * 32) k_last_hop(const int32_t *__restrict__ row_ptr,
                                                               const int32_t *__restrict__ col,
@@ -509,78 +539,42 @@ __global__ void __launch_bounds__(kSpmmWarps * 32) k_last_hop(const int32_t *__r
                                                               const int32_t *__restrict__ tau, int32_t ell,
                                                               double *__restrict__ g, double *__restrict__ t1,
                                                               double *__restrict__ t2, const GatherRec rec) {
+    __shared__ typename AccOf<T>::type tiles[kSpmmWarps][kValueChunks][kChunk + 1];
     __shared__ double diag;
     const int32_t q = blockIdx.x;
     if (q >= nsrc) return;
     const int32_t s = src[q];
     if (s < 0) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int32_t kb = row_ptr[s], ke = row_ptr[s + 1];
+    if (kb + static_cast<int32_t>(blockIdx.y) * kLastPerCta >= ke) return;
     int32_t base;
     const T *xs = slice_column<T, B>(x_prev, n, nullptr, q, &base);
-    // hop ell - 1 (as the fused gather of a full hop-ell launch would)
-    gather_source<T, B>(row_ptr, col, xs, base, s, tau, ell - 1, g, t1, t2, threadIdx.x, blockDim.x, rec);
+    const double diag_prev = static_cast<double>(to_acc(xs[static_cast<int64_t>(s - base) * B]));
     if (warp == 0) {
-        const double v = hop_value<T, B>(row_ptr, col, inv_deg, xs, base, s, lane);
+        const double v = hop_value<T, B>(row_ptr, col, inv_deg, xs, base, s, lane, tiles[0]);
         if (lane == 0) diag = v;
     }
-    __syncthreads();  // also orders the hop ell - 1 updates before the hop ell ones
-    const int32_t kb = row_ptr[s], ke = row_ptr[s + 1];
-    for (int32_t k = kb + warp; k < ke; k += kSpmmWarps) {
-        const double xj = hop_value<T, B>(row_ptr, col, inv_deg, xs, base, col[k], lane);
-        if (lane == 0) gather_term(k, diag - xj, tau, ell, g, t1, t2, rec);
-    }
-}
-
-// The same last hop in two launches, so that a source with many (or heavy)
-// neighbours spreads over many CTAs: k_last_diag gathers X_{ell-1} and
-// computes X_ell[s, b] (one CTA per source); k_last_rows computes X_ell at
-// the neighbours, one warp per neighbour, over a (source, neighbour range)
-// grid, and gathers hop ell.
-template <typename T, int B>
-__global__ void __launch_bounds__(kSpmmWarps * 32) k_last_diag(const int32_t *__restrict__ row_ptr,
-                                                               const int32_t *__restrict__ col,
-                                                               const typename AccOf<T>::type *__restrict__ inv_deg,
-                                                               const T *__restrict__ x_prev, int32_t n,
-                                                               const int32_t *__restrict__ src, int32_t nsrc,
-                                                               const int32_t *__restrict__ tau, int32_t ell,
-                                                               double *__restrict__ g, double *__restrict__ t1,
-                                                               double *__restrict__ t2, const GatherRec rec,
-                                                               double *__restrict__ diag) {
-    const int32_t q = blockIdx.x;
-    if (q >= nsrc) return;
-    const int32_t s = src[q];
-    if (s < 0) return;
-    int32_t base;
-    const T *xs = slice_column<T, B>(x_prev, n, nullptr, q, &base);
-    gather_source<T, B>(row_ptr, col, xs, base, s, tau, ell - 1, g, t1, t2, threadIdx.x, blockDim.x, rec);
-    if (threadIdx.x < 32) {
-        const double v = hop_value<T, B>(row_ptr, col, inv_deg, xs, base, s, threadIdx.x);
-        if (threadIdx.x == 0) diag[q] = v;
-    }
-}
-
-template <typename T, int B>
-__global__ void __launch_bounds__(kSpmmWarps * 32) k_last_rows(const int32_t *__restrict__ row_ptr,
-                                                               const int32_t *__restrict__ col,
-                                                               const typename AccOf<T>::type *__restrict__ inv_deg,
-                                                               const T *__restrict__ x_prev, int32_t n,
-                                                               const int32_t *__restrict__ src, int32_t nsrc,
-                                                               const int32_t *__restrict__ tau, int32_t ell,
-                                                               double *__restrict__ g, double *__restrict__ t1,
-                                                               double *__restrict__ t2, const GatherRec rec,
-                                                               const double *__restrict__ diag) {
-    const int32_t q = blockIdx.x;
-    if (q >= nsrc) return;
-    const int32_t s = src[q];
-    if (s < 0) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int32_t base;
-    const T *xs = slice_column<T, B>(x_prev, n, nullptr, q, &base);
-    const int32_t ke = row_ptr[s + 1];
-    for (int32_t k = row_ptr[s] + static_cast<int32_t>(blockIdx.y) * kSpmmWarps + warp; k < ke;
-         k += static_cast<int32_t>(gridDim.y) * kSpmmWarps) {
-        const double xj = hop_value<T, B>(row_ptr, col, inv_deg, xs, base, col[k], lane);
-        if (lane == 0) gather_term(k, diag[q] - xj, tau, ell, g, t1, t2, rec);
+    bool have = false;  // the diagonal is awaited once, after the warp's first value
+    for (int32_t c0 = kb + static_cast<int32_t>(blockIdx.y) * kLastPerCta; c0 < ke;
+         c0 += static_cast<int32_t>(gridDim.y) * kLastPerCta) {
+        // kLastPerCta entries a round for every warp alike, so that all of them meet the barrier
+#pragma unroll
+        for (int u = 0; u < kLastPerCta / kSpmmWarps; ++u) {
+            const int32_t k = c0 + u * kSpmmWarps + warp;
+            double xj = 0.0, xj_prev = 0.0;
+            if (k < ke) {
+                const int32_t j = col[k];
+                xj_prev = static_cast<double>(to_acc(xs[static_cast<int64_t>(j - base) * B]));
+                xj = hop_value<T, B>(row_ptr, col, inv_deg, xs, base, j, lane, tiles[warp]);
+            }
+            if (!have) __syncthreads();
+            have = true;
+            if (k < ke && lane == 0) {
+                gather_term(k, diag_prev - xj_prev, tau, ell - 1, g, t1, t2, rec);  // as a full hop-ell launch would
+                gather_term(k, diag - xj, tau, ell, g, t1, t2, rec);
+            }
+        }
     }
 }
 
