@@ -34,6 +34,10 @@ struct Layout {
     static constexpr int G = 32 / LG;                            // row groups per warp
     static constexpr int NACC = VPL * E;                         // accumulators per lane
     static constexpr int U = (VPL >= 4) ? 2 : (VPL == 2 ? 4 : 8);  // row loads in flight per lane
+    // a sum starts from its first term instead of adding it to zero (vset): FP64 blocks, whose hops
+    // are bound by the FP64 pipe (tree + G(n, p), 2,000 nodes of degree 10: 121 -> 110 us a hop);
+    // the test per load costs FP32 hops 4%
+    static constexpr bool SET_FIRST = sizeof(Acc) == 8;
     static_assert(V % VPL == 0, "bad split");
     static_assert(LG >= 1 && LG <= 32 && (32 % LG) == 0, "lanes per row must divide 32");
     static_assert(kChunk % U == 0, "unroll must divide the chunk");
@@ -57,6 +61,13 @@ __device__ __forceinline__ void vadd(float *acc, const uint4 &v, __nv_bfloat16) 
         acc[2 * q] += __uint_as_float(w[q] << 16);
         acc[2 * q + 1] += __uint_as_float(w[q] & 0xffff0000u);
     }
+}
+
+// the vector alone: a sum's first term (0 + v = v for the probabilities here, all >= +0) without
+// the addition (Layout::SET_FIRST)
+__device__ __forceinline__ void vset(double *acc, const uint4 &v, double) {
+    acc[0] = __hiloint2double(static_cast<int>(v.y), static_cast<int>(v.x));
+    acc[1] = __hiloint2double(static_cast<int>(v.w), static_cast<int>(v.z));
 }
 
 __device__ __forceinline__ uint4 vpack(const float *a, float) {
@@ -238,10 +249,11 @@ __device__ __forceinline__ const T *slice_column(const T *x, int32_t n, const Sl
 // The last entries [k, ce) of a row or chunk, fewer than U of them: loaded in
 // groups of U/2, U/4, ..., 1 entries (the binary digits of their count), each
 // group's loads in flight together, and added in entry order (the order of
-// the one-at-a-time loop, so every sum is unchanged bit for bit).
+// the one-at-a-time loop, so every sum is unchanged bit for bit). `fresh`: no
+// entry was added to chunk yet, which is then set by the first.
 template <typename T, int B, int VPL>
 __device__ __forceinline__ void add_tail(const int32_t *__restrict__ col, const uint4 *xp, int32_t k, int32_t ce,
-                                         int gl, typename Layout<T, B, VPL>::Acc *chunk) {
+                                         int gl, typename Layout<T, B, VPL>::Acc *chunk, bool fresh = false) {
     using L = Layout<T, B, VPL>;
     constexpr int W = L::U / 2 > 0 ? L::U / 2 : 1;
 #pragma unroll
@@ -258,7 +270,16 @@ __device__ __forceinline__ void add_tail(const int32_t *__restrict__ col, const 
 #pragma unroll
             for (int u = 0; u < w; ++u)
 #pragma unroll
-                for (int p = 0; p < VPL; ++p) vadd(chunk + p * L::E, v[u][p], T());
+                for (int p = 0; p < VPL; ++p) {
+                    if constexpr (L::SET_FIRST) {
+                        if (u == 0 && fresh) {
+                            vset(chunk + p * L::E, v[u][p], T());
+                            continue;
+                        }
+                    }
+                    vadd(chunk + p * L::E, v[u][p], T());
+                }
+            fresh = false;
             k += w;
         }
     }
@@ -399,6 +420,7 @@ __global__ void __launch_bounds__(kSpmmWarps * 32) k_spmm_hop(const HopArgs<T> a
             acc[q] = Acc(0);
             chunk[q] = Acc(0);
         }
+        bool fresh = true;  // chunk holds no entry yet
         int32_t k = cb;
         for (; k + L::U <= ce; k += L::U) {
             int32_t j[L::U];
@@ -413,18 +435,33 @@ __global__ void __launch_bounds__(kSpmmWarps * 32) k_spmm_hop(const HopArgs<T> a
 #pragma unroll
             for (int u = 0; u < L::U; ++u)
 #pragma unroll
-                for (int p = 0; p < VPL; ++p) vadd(chunk + p * L::E, v[u][p], T());
+                for (int p = 0; p < VPL; ++p) {
+                    if constexpr (L::SET_FIRST) {
+                        if (u == 0 && fresh) {
+                            vset(chunk + p * L::E, v[u][p], T());
+                            continue;
+                        }
+                    }
+                    vadd(chunk + p * L::E, v[u][p], T());
+                }
+            fresh = false;
             if (((k + L::U - cb) % kChunk) == 0) {  // a chunk of 32 positions is complete
 #pragma unroll
                 for (int q = 0; q < L::NACC; ++q) {
                     acc[q] += chunk[q];
                     chunk[q] = Acc(0);
                 }
+                fresh = true;
             }
         }
-        add_tail<T, B, VPL>(col, xp, k, ce, gl, chunk);
+        add_tail<T, B, VPL>(col, xp, k, ce, gl, chunk, fresh);
+        if (L::SET_FIRST && ce - cb < kChunk) {  // one chunk: the sum is it
 #pragma unroll
-        for (int q = 0; q < L::NACC; ++q) acc[q] += chunk[q];
+            for (int q = 0; q < L::NACC; ++q) acc[q] = chunk[q];
+        } else {
+#pragma unroll
+            for (int q = 0; q < L::NACC; ++q) acc[q] += chunk[q];
+        }
         const Acc sc = a.inv_deg[cur];
 #pragma unroll
         for (int q = 0; q < L::NACC; ++q) acc[q] *= sc;
