@@ -24,14 +24,16 @@ static void chi_check_t(sc_graph *g, const void *x, int slices, const int32_t *s
                                                             g->tp_cmax.get(), g->tp_cvol.get());
     } else {
         // tile maxima, the threshold per column, then the candidates at or above it
+        using V = typename AccOf<T>::type;
         const int ntiles = ceil_div(g->n, kTileRows);
+        V *tmax = reinterpret_cast<V *>(pmax), *tmin = reinterpret_cast<V *>(pmin);  // room for doubles
         k_chi_tiles<T, B><<<dim3(ntiles, slices), kChiScanThreads, 0, s>>>(g->row_ptr.get(),
-                                                                          static_cast<const T *>(x), g->n, pmax,
-                                                                          pmin, pvol);
-        k_chi_thresh<B><<<ncols, kChiScanThreads, 0, s>>>(ntiles, ncols, gamma, pmax, pmin, pvol, g->tp_cthr.get(),
-                                                             g->tp_cmin.get(), g->tp_cmax.get(), g->tp_cvol.get());
+                                                                          static_cast<const T *>(x), g->n, tmax,
+                                                                          tmin, pvol);
+        k_chi_thresh<V, B><<<ncols, kChiScanThreads, 0, s>>>(ntiles, ncols, gamma, tmax, tmin, pvol, g->tp_cthr.get(),
+                                                                g->tp_cmin.get(), g->tp_cmax.get(), g->tp_cvol.get());
         k_chi_select<T, B><<<ncols, kChiScanThreads, 0, s>>>(g->n, ntiles, ncols, gamma, static_cast<const T *>(x),
-                                                                pmax, pmin, g->tp_cthr.get(), g->tp_cval.get(),
+                                                                tmax, tmin, g->tp_cthr.get(), g->tp_cval.get(),
                                                                 g->tp_cid.get());
     }
     ChiArgs a{};
@@ -53,7 +55,7 @@ static void chi_check_t(sc_graph *g, const void *x, int slices, const int32_t *s
     a.rhs = g->tp_counters.get();
     k_chi_source<T, B><<<nsrc, 32, 0, s>>>(static_cast<const T *>(x), a, g->tp_srcstat.get());
     const int nw = 256 / 32;
-    dim3 grid(nsrc, std::min(ceil_div(std::max(max_deg, 1), nw), 65535));
+    dim3 grid(nsrc, std::min(ceil_div(std::max(max_deg, 1), nw * kChiEntries), 65535));
     k_chi_entries<T, B><<<grid, 256, 0, s>>>(static_cast<const T *>(x), a, g->tp_srcstat.get());
 }
 
