@@ -80,30 +80,60 @@ void tau_entries_device(sc_graph *g, double eps, double lam_star, int32_t *tau_e
 // ---------------------------------------------------------------------------
 // A2: Lanczos kernels (FP64, deterministic reductions)
 // ---------------------------------------------------------------------------
-constexpr int kDotBlocks = 256, kDotThreads = 256;
+constexpr int kDotBlocks = 256, kDotThreads = 256, kDotVectors = 2 * kDotThreads / 32;
 
-// y = D^-1/2 A D^-1/2 x, one warp per row, fixed shuffle tree
+static dim3 dot_grid(int nvec) { return dim3(kDotBlocks, std::max(1, ceil_div(nvec, kDotVectors))); }
+
+// y = D^-1/2 A xs, xs = D^-1/2 x: kSpmvLanes lanes per row, a row above
+// kSpmvHeavy entries by its whole warp, fixed shuffle trees. An FP64 addition
+// takes a warp 16 cycles of the SM's FP64 pipe whatever the lanes in use, and a
+// warp per row spent five of six on the tree: Barabasi-Albert, 100,000 nodes of
+// degree 20, 49 us; 8 lanes per row 28 us.
+constexpr int kSpmvLanes = 8, kSpmvRows = 32 / kSpmvLanes;
+constexpr int32_t kSpmvHeavy = 256;
+
 __global__ void k_spmv_norm(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                            const double *__restrict__ isd, const double *__restrict__ x, double *__restrict__ y,
+                            const double *__restrict__ isd, const double *__restrict__ xs, double *__restrict__ y,
                             int32_t n) {
-    const int32_t r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (r >= n) return;
+    const int lane = threadIdx.x & 31, grp = lane / kSpmvLanes, gl = lane % kSpmvLanes;
+    const int64_t r0 = (blockIdx.x * static_cast<int64_t>(blockDim.x >> 5) + (threadIdx.x >> 5)) * kSpmvRows;
+    const int64_t r = r0 + grp;
+    int32_t b = 0, e = 0;
+    if (r < n) {
+        b = row_ptr[r];
+        e = row_ptr[r + 1];
+    }
+    const bool heavy = e - b > kSpmvHeavy;
     double acc = 0.0;
-    for (int32_t k = row_ptr[r] + lane; k < row_ptr[r + 1]; k += 32) {
-        const int32_t j = col[k];
-        acc += isd[j] * x[j];
+    if (!heavy) {
+#pragma unroll 4
+        for (int32_t k = b + gl; k < e; k += kSpmvLanes) acc += xs[col[k]];
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) y[r] = isd[r] * acc;
+    for (int o = kSpmvLanes / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (gl == 0 && r < n && !heavy) y[r] = isd[r] * acc;
+    uint32_t todo = __ballot_sync(0xffffffffu, heavy && gl == 0);
+    while (todo) {  // warp-uniform
+        const int l = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        const int32_t b0 = __shfl_sync(0xffffffffu, b, l), e0 = __shfl_sync(0xffffffffu, e, l);
+        double sum = 0.0;
+#pragma unroll 4
+        for (int32_t k = b0 + lane; k < e0; k += 32) sum += xs[col[k]];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) y[r0 + l / kSpmvLanes] = isd[r0 + l / kSpmvLanes] * sum;
+    }
 }
+
+static int spmv_grid(int32_t n) { return ceil_div(n, 8 * kSpmvRows); }
 
 // partial[q * kDotBlocks + b] = block b's share of <V_q, w>, for q < nvec:
 // block b takes rows [b c, (b + 1) c) (c = ceil(n / kDotBlocks)), its warps
 // take the vectors q = warp, warp + 8, ..., each lane a strided share of the
-// rows in order, then a fixed shuffle tree. One launch of kDotBlocks blocks
-// for every vector of the basis (the rows of w it reads stay in L1).
+// rows in order, then a fixed shuffle tree. blockIdx.y takes kDotVectors vectors
+// of the basis (two a warp; the rows of w it reads stay in L1), so that a long
+// basis spreads over more warps than 256 blocks hold.
 // skip (nullable): when *skip != 0 the launch does nothing (a pass the device
 // decided against).
 __global__ void k_multidot_partial(const double *__restrict__ V, int64_t ldv, int nvec, const double *__restrict__ w,
@@ -112,9 +142,11 @@ __global__ void k_multidot_partial(const double *__restrict__ V, int64_t ldv, in
     const int64_t c = (static_cast<int64_t>(n) + kDotBlocks - 1) / kDotBlocks;
     const int64_t i0 = blockIdx.x * c, i1 = min(static_cast<int64_t>(n), i0 + c);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = kDotThreads / 32;
-    for (int q = warp; q < nvec; q += nw) {
+    const int q1 = min(nvec, static_cast<int>(blockIdx.y + 1) * kDotVectors);
+    for (int q = blockIdx.y * kDotVectors + warp; q < q1; q += nw) {
         const double *v = V + q * ldv;
         double acc = 0.0;
+#pragma unroll 4
         for (int64_t i = i0 + lane; i < i1; i += 32) acc += v[i] * w[i];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -122,22 +154,29 @@ __global__ void k_multidot_partial(const double *__restrict__ V, int64_t ldv, in
     }
 }
 
-// out[q] = sum of the kDotBlocks partials of row q (fixed tree); 0 when *skip
-__global__ void k_multidot_final(const double *__restrict__ partial, double *__restrict__ out,
-                                 const int *__restrict__ skip = nullptr) {
+// the sum of kDotBlocks partials by the kDotBlocks threads of a block (fixed tree)
+__device__ __forceinline__ double partial_sum(const double *__restrict__ partial) {
     __shared__ double sh[kDotBlocks];
-    const int q = blockIdx.x;
-    if (skip && *skip) {
-        if (threadIdx.x == 0) out[q] = 0.0;
-        return;
-    }
-    sh[threadIdx.x] = partial[q * kDotBlocks + threadIdx.x];
+    __syncthreads();
+    sh[threadIdx.x] = partial[threadIdx.x];
     __syncthreads();
     for (int s = kDotBlocks / 2; s > 0; s >>= 1) {
         if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[q] = sh[0];
+    return sh[0];
+}
+
+// out[q] = sum of the kDotBlocks partials of row q; 0 when *skip
+__global__ void k_multidot_final(const double *__restrict__ partial, double *__restrict__ out,
+                                 const int *__restrict__ skip = nullptr) {
+    const int q = blockIdx.x;
+    if (skip && *skip) {
+        if (threadIdx.x == 0) out[q] = 0.0;
+        return;
+    }
+    const double sum = partial_sum(partial + static_cast<int64_t>(q) * kDotBlocks);
+    if (threadIdx.x == 0) out[q] = sum;
 }
 
 // w -= sum_q c[q] V_q (q in order); nothing when *skip
@@ -147,16 +186,26 @@ __global__ void k_sub_combination(const double *__restrict__ V, int64_t ldv, int
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     double acc = w[i];
-    for (int q = 0; q < nvec; ++q) acc -= c[q] * V[q * ldv + i];
+    int q = 0;
+    for (; q + 8 <= nvec; q += 8) {  // eight rows of the basis in flight
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = V[(q + u) * ldv + i];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc -= c[q + u] * v[u];
+    }
+    for (; q < nvec; ++q) acc -= c[q] * V[q * ldv + i];
     w[i] = acc;
 }
 
-// dst = src * (1 / nrm), nrm read from the device
+// dst = src * (1 / nrm), nrm read from the device, and xs = D^-1/2 dst for the next product
 __global__ void k_scale_into(const double *__restrict__ src, const double *__restrict__ nrm2, double *__restrict__ dst,
-                             int32_t n) {
+                             int32_t n, const double *__restrict__ isd, double *__restrict__ xs) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    dst[i] = src[i] / sqrt(*nrm2);
+    const double v = src[i] / sqrt(*nrm2);
+    dst[i] = v;
+    xs[i] = isd[i] * v;
 }
 
 // alpha of a Lanczos step: the coefficients of V_vj in the two orthogonalisation passes, summed
@@ -165,29 +214,59 @@ __global__ void k_alpha_of(const double *__restrict__ c, int nbasis, int vj, dou
 }
 
 // The three-term part of a Lanczos step: w -= a V_vj + beta V_vj-1, with a =
-// <w, V_vj> (from the device) and beta = sqrt(|w_prev|^2) (nrm2_prev null:
-// no previous Lanczos vector, the first step)
-__global__ void k_three_term(const double *__restrict__ V, int64_t ldv, int vj, const double *__restrict__ a,
-                             const double *__restrict__ nrm2_prev, double *__restrict__ w, int32_t n) {
+// <w, V_vj> (its partials summed by every block; kept in *a_out) and beta =
+// sqrt(|w_prev|^2) (nrm2_prev null: no previous Lanczos vector, the first step)
+__global__ void __launch_bounds__(kDotBlocks) k_three_term(const double *__restrict__ V, int64_t ldv, int vj,
+                                                           const double *__restrict__ partial,
+                                                           double *__restrict__ a_out,
+                                                           const double *__restrict__ nrm2_prev,
+                                                           double *__restrict__ w, int32_t n) {
+    const double a = partial_sum(partial);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a_out = a;
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    double acc = w[i] - *a * V[vj * ldv + i];
+    double acc = w[i] - a * V[vj * ldv + i];
     if (nrm2_prev) acc -= sqrt(*nrm2_prev) * V[(vj - 1) * ldv + i];
     w[i] = acc;
 }
 
 // skip the second sweep unless the first removed more than half of |w|^2
 // ("twice is enough": one more sweep restores orthogonality to working
-// precision when the first lost most of the vector)
-__global__ void k_second_sweep_flag(const double *__restrict__ nrm2_before, const double *__restrict__ nrm2_after,
-                                    int *__restrict__ skip) {
-    *skip = (*nrm2_after < 0.5 * *nrm2_before) ? 0 : 1;
+// precision when the first lost most of the vector); |w|^2 before and after it
+// from their partials, the latter kept in *nrm2_after
+__global__ void __launch_bounds__(kDotBlocks) k_second_sweep_flag(const double *__restrict__ part_before,
+                                                                  const double *__restrict__ part_after,
+                                                                  double *__restrict__ nrm2_after,
+                                                                  int *__restrict__ skip) {
+    const double before = partial_sum(part_before);
+    const double after = partial_sum(part_after);
+    if (threadIdx.x == 0) {
+        *nrm2_after = after;
+        *skip = (after < 0.5 * before) ? 0 : 1;
+    }
 }
 
-// alpha of a step with the three-term part: its coefficient plus the sweeps' coefficients of V_vj
-__global__ void k_alpha_three(const double *__restrict__ a, const double *__restrict__ c, int nbasis, int vj,
-                              double *__restrict__ alpha) {
-    *alpha = *a + c[vj] + c[nbasis + vj];
+// The end of a step: alpha (the three-term coefficient plus the sweeps' of V_vj),
+// |w|^2 (the first sweep's, or from its partials after a second one), the next
+// basis vector w / |w| and xs = D^-1/2 of it
+__global__ void __launch_bounds__(kDotBlocks) k_step_end(const double *__restrict__ a, const double *__restrict__ c,
+                                                         int nbasis, int vj, const int *__restrict__ skip,
+                                                         const double *__restrict__ nrm2_after,
+                                                         const double *__restrict__ part_second,
+                                                         const double *__restrict__ w, const double *__restrict__ isd,
+                                                         double *__restrict__ alpha, double *__restrict__ nrm2,
+                                                         double *__restrict__ next, double *__restrict__ xs,
+                                                         int32_t n) {
+    const double nn = *skip ? *nrm2_after : partial_sum(part_second);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *alpha = *a + c[vj] + c[nbasis + vj];
+        *nrm2 = nn;
+    }
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double v = w[i] / sqrt(nn);
+    next[i] = v;
+    xs[i] = isd[i] * v;
 }
 
 // locked vectors: sqrt(d_x)/sqrt(2m), and (bipartite) the same with sign (-1)^level
@@ -232,6 +311,7 @@ static double bisect_eig(const std::vector<double> &a, const std::vector<double>
                          double hi) {
     for (int it = 0; it < 200 && hi - lo > 1e-17 * std::max(1.0, std::fabs(lo) + std::fabs(hi)); ++it) {
         const double mid = 0.5 * (lo + hi);
+        if (mid <= lo || mid >= hi) break;  // neighbouring numbers: no further step changes either
         if (sturm_count(a, b, k, mid) > idx) hi = mid;
         else lo = mid;
     }
@@ -312,10 +392,12 @@ sc_status estimate_lambda_impl(sc_graph *g, const sc_lambda_opts *opts, sc_lambd
         cudaStream_t s = g->stream;
         const int64_t ldv = (static_cast<int64_t>(n) + 31) / 32 * 32;
         const int nbasis = nlock + max_iter + 1;
-        DevBuf<double> V, w, isd, c, partial;
+        DevBuf<double> V, w, isd, xs, c, partial, part_norm;
         V.reserve(static_cast<size_t>(nbasis) * ldv);
         w.reserve(n);
         isd.reserve(n);
+        xs.reserve(n);
+        part_norm.reserve(2 * kDotBlocks);
         c.reserve(2 * nbasis + 8);
         partial.reserve(static_cast<size_t>(nbasis) * kDotBlocks);
         const int tb = 256;
@@ -330,7 +412,7 @@ sc_status estimate_lambda_impl(sc_graph *g, const sc_lambda_opts *opts, sc_lambd
         auto reorth = [&](int nv) {
             for (int pass = 0; pass < 2; ++pass) {
                 double *cc = c.get() + (pass ? nbasis : 0);
-                k_multidot_partial<<<kDotBlocks, kDotThreads, 0, s>>>(V.get(), ldv, nv, w.get(), n, partial.get());
+                k_multidot_partial<<<dot_grid(nv), kDotThreads, 0, s>>>(V.get(), ldv, nv, w.get(), n, partial.get());
                 k_multidot_final<<<nv, kDotBlocks, 0, s>>>(partial.get(), cc);
                 k_sub_combination<<<nb, tb, 0, s>>>(V.get(), ldv, nv, cc, w.get(), n);
                 SC_LAUNCH_CHECK();
@@ -348,31 +430,37 @@ sc_status estimate_lambda_impl(sc_graph *g, const sc_lambda_opts *opts, sc_lambd
         // exact arithmetic the recurrence leaves w orthogonal to the basis; the sweep removes
         // what rounding left, so the second sweep is rarely needed and a step costs about
         // half the FP64 work of two full sweeps.
-        double *d_scal = nullptr;  // [0] a, [1] |w|^2 before the sweep, [2] after it
+        // The scalars (a, the norms, the decision) are summed where they are used, not in launches
+        // of one block of their own: 14 launches a step.
+        double *d_scal = nullptr;  // [0] a, [1] |w|^2 after the first sweep
         DevBuf<double> scal;
         DevBuf<int> skip;
-        scal.reserve(4);
+        scal.reserve(2);
         skip.reserve(1);
         d_scal = scal.get();
-        auto step_orth = [&](int vj, const double *nrm2_prev) {
-            k_multidot_partial<<<kDotBlocks, kDotThreads, 0, s>>>(V.get() + vj * ldv, ldv, 1, w.get(), n,
-                                                                          partial.get());
-            k_multidot_final<<<1, kDotBlocks, 0, s>>>(partial.get(), d_scal);
-            k_three_term<<<nb, tb, 0, s>>>(V.get(), ldv, vj, d_scal, nrm2_prev, w.get(), n);
-            SC_LAUNCH_CHECK();
-            norm2_into(d_scal + 1);
+        static_assert(kDotBlocks == 256 && kDotThreads == 256, "a block sums the partials of a dot product");
+        auto partials = [&](const double *v, double *into, const int *skip_flag) {
+            k_multidot_partial<<<kDotBlocks, kDotThreads, 0, s>>>(v, ldv, 1, w.get(), n, into, skip_flag);
+        };
+        auto step = [&](int vj, const double *nrm2_prev, double *alpha_out, double *nrm2_out) {
+            double *before = part_norm.get(), *after = part_norm.get() + kDotBlocks;
+            partials(V.get() + vj * ldv, partial.get(), nullptr);
+            k_three_term<<<nb, tb, 0, s>>>(V.get(), ldv, vj, partial.get(), d_scal, nrm2_prev, w.get(), n);
+            partials(w.get(), before, nullptr);
             const int nv = vj + 1;
-            k_multidot_partial<<<kDotBlocks, kDotThreads, 0, s>>>(V.get(), ldv, nv, w.get(), n, partial.get());
+            k_multidot_partial<<<dot_grid(nv), kDotThreads, 0, s>>>(V.get(), ldv, nv, w.get(), n, partial.get());
             k_multidot_final<<<nv, kDotBlocks, 0, s>>>(partial.get(), c.get());
             k_sub_combination<<<nb, tb, 0, s>>>(V.get(), ldv, nv, c.get(), w.get(), n);
-            SC_LAUNCH_CHECK();
-            norm2_into(d_scal + 2);
-            k_second_sweep_flag<<<1, 1, 0, s>>>(d_scal + 1, d_scal + 2, skip.get());
+            partials(w.get(), after, nullptr);
+            k_second_sweep_flag<<<1, kDotBlocks, 0, s>>>(before, after, d_scal + 1, skip.get());
             double *c2 = c.get() + nbasis;
-            k_multidot_partial<<<kDotBlocks, kDotThreads, 0, s>>>(V.get(), ldv, nv, w.get(), n, partial.get(),
-                                                                           skip.get());
+            k_multidot_partial<<<dot_grid(nv), kDotThreads, 0, s>>>(V.get(), ldv, nv, w.get(), n, partial.get(),
+                                                                    skip.get());
             k_multidot_final<<<nv, kDotBlocks, 0, s>>>(partial.get(), c2, skip.get());
             k_sub_combination<<<nb, tb, 0, s>>>(V.get(), ldv, nv, c2, w.get(), n, skip.get());
+            partials(w.get(), before, skip.get());
+            k_step_end<<<nb, tb, 0, s>>>(d_scal, c.get(), nbasis, vj, skip.get(), d_scal + 1, before, w.get(),
+                                         isd.get(), alpha_out, nrm2_out, V.get() + (vj + 1) * ldv, xs.get(), n);
             SC_LAUNCH_CHECK();
         };
 
@@ -382,66 +470,88 @@ sc_status estimate_lambda_impl(sc_graph *g, const sc_lambda_opts *opts, sc_lambd
         reorth(nlock);
         double *nrm_dev = c.get() + 2 * nbasis;
         norm2_into(nrm_dev);
-        k_scale_into<<<nb, tb, 0, s>>>(w.get(), nrm_dev, V.get() + nlock * ldv, n);
+        k_scale_into<<<nb, tb, 0, s>>>(w.get(), nrm_dev, V.get() + nlock * ldv, n, isd.get(), xs.get());
         SC_LAUNCH_CHECK();
 
         // alpha_j and |w_j|^2 of every step stay on the device; the host reads
         // them only at the steps where it checks convergence (every 4th from
-        // step 8, and the last possible one), so the steps in between run with
-        // no synchronisation. A breakdown (|w_j| <= 1e-12) between two checks is
-        // found at the next one and the steps after it are discarded, which
-        // gives the same steps and result as stopping at the breakdown itself.
+        // step 8, and the last possible one). A check's copies go to page-locked
+        // memory, and the steps up to the next check are queued before the host
+        // waits for them, so that the GPU works on while the host solves the
+        // tridiagonal problem; steps past the one the check stops at are
+        // discarded. A breakdown (|w_j| <= 1e-12) between two checks is found at
+        // the next one and the steps after it are discarded too, which gives the
+        // same steps and result as stopping at the breakdown itself.
         DevBuf<double> ab;
         ab.reserve(2 * static_cast<size_t>(max_iter));
         double *d_alpha = ab.get(), *d_nrm2 = ab.get() + max_iter;
-        std::vector<double> alpha, beta(1, 0.0), h_alpha, h_nrm2;
+        struct Check {  // a check's copies and the event behind them, two in turn
+            double *h = nullptr;  // alpha, |w|^2: max_iter values each
+            cudaEvent_t done = nullptr;
+            int kk = 0;  // steps at the check (0: none queued)
+            ~Check() {
+                if (done) cudaEventDestroy(done);
+                if (h) cudaFreeHost(h);
+            }
+        } check[2];
+        for (Check &c2 : check) {
+            SC_CUDA(cudaMallocHost(reinterpret_cast<void **>(&c2.h), 2 * static_cast<size_t>(max_iter) * sizeof(double)));
+            SC_CUDA(cudaEventCreateWithFlags(&c2.done, cudaEventDisableTiming));
+        }
+        struct Drain {  // queued copies end before their buffers go
+            cudaStream_t s;
+            ~Drain() { cudaStreamSynchronize(s); }
+        } drain{s};
+        std::vector<double> alpha, beta(1, 0.0);
         double theta_max = 0, theta_min = 0, res_max = INFINITY, res_min = INFINITY;
         int k = 0;
-        bool converged = false;
-        for (int j = 0; j < max_iter; ++j) {
-            const int vj = nlock + j;
-            k_spmv_norm<<<ceil_div(n, 8), 256, 0, s>>>(g->row_ptr.get(), g->col_idx.get(), isd.get(),
-                                                        V.get() + vj * ldv, w.get(), n);
-            SC_LAUNCH_CHECK();
-            step_orth(vj, j > 0 ? d_nrm2 + (j - 1) : nullptr);
-            k_alpha_three<<<1, 1, 0, s>>>(d_scal, c.get(), nbasis, vj, d_alpha + j);
-            norm2_into(d_nrm2 + j);
-            const int kk = j + 1;
-            if (kk == max_iter || kk == n - nlock || (kk >= 8 && kk % 4 == 0)) {
-                h_alpha.resize(kk);
-                h_nrm2.resize(kk);
-                SC_CUDA(cudaMemcpyAsync(h_alpha.data(), d_alpha, kk * sizeof(double), cudaMemcpyDeviceToHost, s));
-                SC_CUDA(cudaMemcpyAsync(h_nrm2.data(), d_nrm2, kk * sizeof(double), cudaMemcpyDeviceToHost, s));
-                SC_CUDA(cudaStreamSynchronize(s));
-                bool exhausted = kk == n - nlock;
-                int stop = kk;
-                for (int q = static_cast<int>(alpha.size()); q < kk; ++q) {
-                    alpha.push_back(h_alpha[q]);
-                    const double b = std::sqrt(std::max(h_nrm2[q], 0.0));
-                    if (!(b > 1e-12)) {  // breakdown at step q: the Krylov space is exhausted
-                        stop = q + 1;
-                        exhausted = true;
-                        break;
-                    }
-                    if (q + 1 < kk) beta.push_back(b);
-                }
-                k = stop;
-                const double bnext = std::sqrt(std::max(h_nrm2[stop - 1], 0.0));
-                // extreme Ritz values and their residuals bnext * |y_k|
-                theta_max = bisect_eig(alpha, beta, k, k - 1, -1.0 - 1e-9, 1.0 + 1e-9);
-                theta_min = bisect_eig(alpha, beta, k, 0, -1.0 - 1e-9, 1.0 + 1e-9);
-                res_max = exhausted ? 0.0 : bnext * std::fabs(ritz_last_component(alpha, beta, k, theta_max));
-                res_min = exhausted ? 0.0 : bnext * std::fabs(ritz_last_component(alpha, beta, k, theta_min));
-                if (res_max <= tol && res_min <= tol) {
-                    converged = true;
+        bool converged = false, ended = false;
+        auto settle = [&](Check &c2) {  // the host side of a queued check
+            const int kk = c2.kk;
+            c2.kk = 0;
+            SC_CUDA(cudaEventSynchronize(c2.done));
+            const double *h_alpha = c2.h, *h_nrm2 = c2.h + max_iter;
+            bool exhausted = kk == n - nlock;
+            int stop = kk;
+            for (int q = static_cast<int>(alpha.size()); q < kk; ++q) {
+                alpha.push_back(h_alpha[q]);
+                const double b = std::sqrt(std::max(h_nrm2[q], 0.0));
+                if (!(b > 1e-12)) {  // breakdown at step q: the Krylov space is exhausted
+                    stop = q + 1;
+                    exhausted = true;
                     break;
                 }
-                if (exhausted) break;
-                beta.push_back(bnext);
+                if (q + 1 < kk) beta.push_back(b);
             }
-            k = kk;
-            k_scale_into<<<nb, tb, 0, s>>>(w.get(), d_nrm2 + j, V.get() + (vj + 1) * ldv, n);
-            SC_LAUNCH_CHECK();
+            k = stop;
+            const double bnext = std::sqrt(std::max(h_nrm2[stop - 1], 0.0));
+            // extreme Ritz values and their residuals bnext * |y_k|
+            theta_max = bisect_eig(alpha, beta, k, k - 1, -1.0 - 1e-9, 1.0 + 1e-9);
+            theta_min = bisect_eig(alpha, beta, k, 0, -1.0 - 1e-9, 1.0 + 1e-9);
+            res_max = exhausted ? 0.0 : bnext * std::fabs(ritz_last_component(alpha, beta, k, theta_max));
+            res_min = exhausted ? 0.0 : bnext * std::fabs(ritz_last_component(alpha, beta, k, theta_min));
+            converged = res_max <= tol && res_min <= tol;
+            ended = converged || exhausted;
+            if (!ended) beta.push_back(bnext);
+        };
+        int turn = 0;
+        for (int j = 0; j < max_iter && !ended; ++j) {
+            const int vj = nlock + j;
+            k_spmv_norm<<<spmv_grid(n), 256, 0, s>>>(g->row_ptr.get(), g->col_idx.get(), isd.get(), xs.get(), w.get(),
+                                                     n);
+            step(vj, j > 0 ? d_nrm2 + (j - 1) : nullptr, d_alpha + j, d_nrm2 + j);
+            const int kk = j + 1;
+            if (kk == max_iter || kk == n - nlock || (kk >= 8 && kk % 4 == 0)) {
+                Check &now = check[turn], &before = check[turn ^ 1];
+                turn ^= 1;
+                SC_CUDA(cudaMemcpyAsync(now.h, d_alpha, kk * sizeof(double), cudaMemcpyDeviceToHost, s));
+                SC_CUDA(cudaMemcpyAsync(now.h + max_iter, d_nrm2, kk * sizeof(double), cudaMemcpyDeviceToHost, s));
+                SC_CUDA(cudaEventRecord(now.done, s));
+                now.kk = kk;
+                if (before.kk) settle(before);
+                if (!ended && (kk == max_iter || kk == n - nlock)) settle(now);  // the last one: nothing to queue
+                if (ended) break;
+            }
         }
         out->lambda_plus = theta_max;
         out->lambda_minus = theta_min;
@@ -634,8 +744,9 @@ static LanczosOut lanczos_run(sc_graph *g, double *V, int64_t ldv, int nlock, in
     const int32_t n = g->n;
     cudaStream_t s = g->stream;
     const int nbasis = nlock + max_iter + 1;
-    DevBuf<double> w, c, partial, ab;
+    DevBuf<double> w, xs, c, partial, ab;
     w.reserve(n);
+    xs.reserve(n);
     c.reserve(2 * static_cast<size_t>(nbasis) + 8);
     partial.reserve(static_cast<size_t>(nbasis) * kDotBlocks);
     ab.reserve(2 * static_cast<size_t>(max_iter));
@@ -643,7 +754,7 @@ static LanczosOut lanczos_run(sc_graph *g, double *V, int64_t ldv, int nlock, in
     auto reorth = [&](int nv) {
         for (int pass = 0; pass < 2; ++pass) {
             double *cc = c.get() + (pass ? nbasis : 0);
-            k_multidot_partial<<<kDotBlocks, kDotThreads, 0, s>>>(V, ldv, nv, w.get(), n, partial.get());
+            k_multidot_partial<<<dot_grid(nv), kDotThreads, 0, s>>>(V, ldv, nv, w.get(), n, partial.get());
             k_multidot_final<<<nv, kDotBlocks, 0, s>>>(partial.get(), cc);
             k_sub_combination<<<nb, tb, 0, s>>>(V, ldv, nv, cc, w.get(), n);
             SC_LAUNCH_CHECK();
@@ -659,7 +770,7 @@ static LanczosOut lanczos_run(sc_graph *g, double *V, int64_t ldv, int nlock, in
     reorth(nlock);
     double *nrm_dev = c.get() + 2 * nbasis;
     norm2_into(nrm_dev);
-    k_scale_into<<<nb, tb, 0, s>>>(w.get(), nrm_dev, V + nlock * ldv, n);
+    k_scale_into<<<nb, tb, 0, s>>>(w.get(), nrm_dev, V + nlock * ldv, n, isd, xs.get());
     SC_LAUNCH_CHECK();
     double *d_alpha = ab.get(), *d_nrm2 = ab.get() + max_iter;
     std::vector<double> h_alpha, h_nrm2;
@@ -667,7 +778,7 @@ static LanczosOut lanczos_run(sc_graph *g, double *V, int64_t ldv, int nlock, in
     int k = 0;
     for (int j = 0; j < max_iter; ++j) {
         const int vj = nlock + j;
-        k_spmv_norm<<<ceil_div(n, 8), 256, 0, s>>>(g->row_ptr.get(), g->col_idx.get(), isd, V + vj * ldv, w.get(), n);
+        k_spmv_norm<<<spmv_grid(n), 256, 0, s>>>(g->row_ptr.get(), g->col_idx.get(), isd, xs.get(), w.get(), n);
         SC_LAUNCH_CHECK();
         reorth(vj + 1);
         k_alpha_of<<<1, 1, 0, s>>>(c.get(), nbasis, vj, d_alpha + j);
@@ -709,7 +820,7 @@ static LanczosOut lanczos_run(sc_graph *g, double *V, int64_t ldv, int nlock, in
             L.beta.push_back(L.bnext);
         }
         k = kk;
-        k_scale_into<<<nb, tb, 0, s>>>(w.get(), d_nrm2 + j, V + (vj + 1) * ldv, n);
+        k_scale_into<<<nb, tb, 0, s>>>(w.get(), d_nrm2 + j, V + (vj + 1) * ldv, n, isd, xs.get());
         SC_LAUNCH_CHECK();
     }
     L.k = k;
