@@ -29,9 +29,9 @@
 // HBM. Small balls are bound by the latency of a level (one dependent global
 // load and a table insert, then a barrier) and of a hop (one barrier), which is
 // why several CTAs share an SM when the ball is small. Whole calls, windowed
-// blocks against this: 150 x 613 strip at 67 + 2 hops 94 -> 9.0 ms, 400 x 400
-// lattice at learned lengths (37 to 353 hops) 625 -> 31 ms, 24 mixed graphs with
-// lattices of 1,000 to 5,000 nodes at 1,003 hops 223 -> 85 ms.
+// blocks against this: 150 x 613 strip at 67 + 2 hops 94 -> 8.4 ms, 400 x 400
+// lattice at learned lengths (37 to 353 hops) 625 -> 29.6 ms, 24 mixed graphs with
+// lattices of 1,000 to 5,000 nodes at 1,003 hops 223 -> 76 ms.
 #include <algorithm>
 #include <numeric>
 
@@ -41,12 +41,12 @@ namespace sc {
 
 constexpr int kResDegMax = 8;       // largest degree taken (neighbour ids kept per row)
 constexpr int kResClasses = 4;      // shared-memory sizes tried in turn; the last keeps the adjacency in global memory
+constexpr int kResIdOrder = 4;      // hops per level from which the lists are kept in id order
 constexpr int kResSample = 128;     // groups whose ball is measured to choose the first class
 
 struct ResArgs {
     const int32_t *row_ptr;
     const int32_t *ell;      // n x W neighbour ids in CSR order, -1 past the degree
-    const void *inv_deg;
     int32_t n;
     const int32_t *order;    // groups of C sources (-1: empty slot)
     const int32_t *groups;   // the launch's groups (nullable: all of 0 .. ngroups)
@@ -92,8 +92,10 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
     using Vec = ResVec<Acc, C>;
     using Adj = ResAdj<W>;
     extern __shared__ __align__(16) unsigned char sm[];
-    __shared__ int32_t cnt[2];
-    __shared__ int32_t overflow;
+    __shared__ int32_t cnt[2], span[2], spos[C];
+    __shared__ Acc recip[kResDegMax + 1];  // 1/d as the graph stores it
+    if (threadIdx.x >= 1 && threadIdx.x <= kResDegMax)
+        recip[threadIdx.x] = static_cast<Acc>(1.0 / static_cast<double>(static_cast<int>(threadIdx.x)));
     const int T = blockDim.x, tid = threadIdx.x;
     const int cap = a.cap, N = (BIP ? 2 : 1) * cap;  // local ids; id N: a cell that stays zero
     int32_t *lvl = reinterpret_cast<int32_t *>(sm);  // lvl[k]: nodes of its list up to level k
@@ -118,7 +120,6 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
         hval = reinterpret_cast<uint16_t *>(hkey + a.hash);
     }
     Vec *X = reinterpret_cast<Vec *>(p);  // NBUF x (N + 1)
-    const Acc *inv_deg = static_cast<const Acc *>(a.inv_deg);
 
     for (int32_t gi = blockIdx.x; gi < a.ngroups; gi += gridDim.x) {
         const int32_t gid = a.groups ? a.groups[gi] : gi;
@@ -135,44 +136,42 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
         if (tid == 0) {
             cnt[0] = C;
             cnt[1] = 0;
-            overflow = 0;
             lvl[0] = C;
         }
         __syncthreads();
-        volatile int32_t *ovf = &overflow;
-        // claims node v for `list` unless it is known
-        auto visit = [&](int32_t v, int list) {
+        bool fits = true;
+        // claims node v for `list` unless it is known; false: it does not fit
+        auto visit = [&](int32_t v, int list) -> bool {
             if constexpr (GADJ) {
                 unsigned short *m = reinterpret_cast<unsigned short *>(hval) + v;
-                if (*reinterpret_cast<volatile unsigned short *>(m) != 0xffffu) return;
-                if (atomicCAS(m, static_cast<unsigned short>(0xffffu), static_cast<unsigned short>(0xfffeu)) != 0xffffu) return;
+                if (*reinterpret_cast<volatile unsigned short *>(m) != 0xffffu) return true;
+                if (atomicCAS(m, static_cast<unsigned short>(0xffffu), static_cast<unsigned short>(0xfffeu)) != 0xffffu) return true;
                 const int32_t at = atomicAdd(&cnt[list], 1);
                 if (at >= cap) {
                     *m = 0xffffu;
-                    *ovf = 1;
-                    return;
+                    return false;
                 }
                 *m = static_cast<unsigned short>(list * cap + at);
                 nodes[list * cap + at] = v;
+                return true;
             } else {
                 const uint32_t key = static_cast<uint32_t>(v) + 1u;
                 uint32_t slot = __umulhi(key * 2654435761u, static_cast<uint32_t>(a.hash));
                 for (int probe = 0; probe < a.hash; ++probe) {
                     const uint32_t old = atomicCAS(&hkey[slot], 0u, key);
-                    if (old == key) return;
+                    if (old == key) return true;
                     if (old == 0u) {
+                        // the next level reads this node's neighbours
+                        asm volatile("prefetch.global.L1 [%0];" ::"l"(a.ell + static_cast<int64_t>(v) * W));
                         const int32_t at = atomicAdd(&cnt[list], 1);
-                        if (at >= cap) {
-                            *ovf = 1;
-                            return;
-                        }
+                        if (at >= cap) return false;
                         hval[slot] = static_cast<uint16_t>(list * cap + at);
                         nodes[list * cap + at] = v;
-                        return;
+                        return true;
                     }
                     slot = slot + 1 == static_cast<uint32_t>(a.hash) ? 0 : slot + 1;
                 }
-                *ovf = 1;
+                return false;
             }
         };
         if (tid == 0) {
@@ -193,33 +192,40 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
             }
         }
         __syncthreads();
-        int32_t top = 0;  // last level
+        // One barrier a level, which also carries the overflow marks. The level's bounds are in
+        // registers: on a bipartite graph a level's inserts go to the other list, so its count is
+        // not touched again before every thread has read it; with one list a second barrier is
+        // needed for that.
+        int32_t top = 0;                 // last level
+        int32_t low[2] = {C, 0};         // BIP: nodes of each list so far
+        int32_t f0 = 0, f1 = C;          // the frontier in its list
         for (int32_t k = 0; k < R; ++k) {
             const int from = BIP ? (k & 1) : 0, to = BIP ? 1 - from : 0;
-            const int32_t f0 = BIP ? (k >= 2 ? lvl[k - 2] : 0) : (k >= 1 ? lvl[k - 1] : 0), f1 = lvl[k];
+            bool over = false;
             for (int32_t t = tid; t < (f1 - f0) * W; t += T) {
-                if (*ovf) break;
                 const int32_t v = nodes[from * cap + f0 + t / W];
                 if (v < 0) continue;
                 const int32_t nb = a.ell[static_cast<int64_t>(v) * W + t % W];
-                if (nb >= 0) visit(nb, to);
+                if (nb >= 0 && !visit(nb, to)) {
+                    over = true;
+                    break;
+                }
             }
-            __syncthreads();
-            const int32_t now = min(cnt[to], cap);
-            const int32_t before = BIP ? (k >= 1 ? lvl[k - 1] : 0) : f1;
-            const bool stop = overflow || now == before;
-            if (!stop && k + 1 >= a.levels) {  // too deep for the level bounds
-                if (tid == 0) overflow = 1;
-                __syncthreads();
+            if (k + 1 >= a.levels) over = true;  // too deep for the level bounds
+            if (__syncthreads_or(over)) {
+                fits = false;
                 break;
             }
-            if (stop) break;
+            const int32_t before = BIP ? low[to] : f1, now = cnt[to];
+            if (now == before) break;
             if (tid == 0) lvl[k + 1] = now;
             top = k + 1;
-            __syncthreads();
+            low[to] = now;
+            f0 = before;
+            f1 = now;
+            if constexpr (!BIP) __syncthreads();
         }
         __syncthreads();
-        const bool fits = overflow == 0;
         const int32_t n0 = min(cnt[0], cap), n1 = BIP ? min(cnt[1], cap) : 0;
         auto forget = [&] {  // the global-adjacency class: the nodes' local ids back to "unknown"
             if constexpr (GADJ) {
@@ -243,14 +249,97 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
             continue;
         }
 
+        // ---- a run of many more hops than levels: the lists in id order ----
+        // The level prefixes save little there; in id order the neighbours of consecutive rows of a
+        // row-major lattice are consecutive too, and their 16-byte values free of bank conflicts.
+        // Ranks by a bitmap of the ids per list, over the adjacency and 1/d, not yet written.
+        int32_t m0 = n0, m1 = n1;  // list lengths (in id order the empty source slots are gone)
+        bool by_id = false;
+        if constexpr (!GADJ) {
+            if (Lg >= kResIdOrder * top) {
+                if (tid == 0) span[0] = INT32_MAX, span[1] = -1;
+                __syncthreads();
+                for (int32_t t = tid; t < n0 + n1; t += T) {
+                    const int32_t v = nodes[t < n0 ? t : cap + t - n0];
+                    if (v >= 0) {
+                        atomicMin(&span[0], v);
+                        atomicMax(&span[1], v);
+                    }
+                }
+                __syncthreads();
+                const int32_t first = span[0], words = (span[1] - first) / 32 + 1;
+                constexpr int LISTS = BIP ? 2 : 1;
+                by_id = static_cast<size_t>(LISTS) * words * 8 <= L::adj_bytes(N);
+                if (by_id) {  // CTA-uniform
+                    uint32_t *bits = reinterpret_cast<uint32_t *>(adj);
+                    int32_t *pre = reinterpret_cast<int32_t *>(bits + LISTS * words);
+                    int32_t *moved = reinterpret_cast<int32_t *>(inv);
+                    for (int32_t t = tid; t < LISTS * words; t += T) bits[t] = 0u;
+                    __syncthreads();
+                    for (int32_t t = tid; t < n0 + n1; t += T) {
+                        const int32_t v = nodes[t < n0 ? t : cap + t - n0];
+                        if (v >= 0) atomicOr(&bits[(t < n0 ? 0 : words) + (v - first) / 32], 1u << ((v - first) % 32));
+                    }
+                    __syncthreads();
+                    if (tid < LISTS * 32) {  // a warp per list: running counts over its words
+                        const int32_t l = tid / 32, lane = tid % 32;
+                        int32_t run = 0;
+                        for (int32_t w = 0; w < words; w += 32) {
+                            const int32_t c = w + lane < words ? __popc(bits[l * words + w + lane]) : 0;
+                            int32_t inc = c;
+#pragma unroll
+                            for (int o = 1; o < 32; o <<= 1) {
+                                const int32_t up = __shfl_up_sync(0xffffffffu, inc, o);
+                                if (lane >= o) inc += up;
+                            }
+                            if (w + lane < words) pre[l * words + w + lane] = run + inc - c;
+                            run += __shfl_sync(0xffffffffu, inc, 31);
+                        }
+                        if (lane == 0) cnt[l] = run;
+                    }
+                    __syncthreads();
+                    for (int32_t t = tid; t < n0 + n1; t += T) {
+                        const int32_t v = nodes[t < n0 ? t : cap + t - n0];
+                        if (v < 0) continue;
+                        const int32_t l = t < n0 ? 0 : 1, w = l * words + (v - first) / 32;
+                        const int32_t at = l * cap + pre[w] + __popc(bits[w] & ((1u << ((v - first) % 32)) - 1u));
+                        moved[at] = v;
+                        if (t < C) spos[t] = at;
+                        const uint32_t key = static_cast<uint32_t>(v) + 1u;
+                        uint32_t slot = __umulhi(key * 2654435761u, static_cast<uint32_t>(a.hash));
+                        for (int probe = 0; probe < a.hash && hkey[slot] != key; ++probe)
+                            slot = slot + 1 == static_cast<uint32_t>(a.hash) ? 0 : slot + 1;
+                        hval[slot] = static_cast<uint16_t>(at);
+                    }
+                    m0 = cnt[0];
+                    if (BIP) m1 = cnt[1];
+                    __syncthreads();
+                    for (int32_t t = tid; t < m0 + m1; t += T) {
+                        const int32_t i = t < m0 ? t : cap + t - m0;
+                        nodes[i] = moved[i];
+                    }
+                    __syncthreads();
+                }
+            }
+        }
+        if (!by_id && tid < C) spos[tid] = tid;
+
         // ---- adjacency in local ids (past the ball or the degree: the zero cell), 1/d ----
-        for (int32_t t = tid; t < n0 + n1; t += T) {
-            const int32_t i = t < n0 ? t : cap + t - n0;
+#pragma unroll 2
+        for (int32_t t = tid; t < m0 + m1; t += T) {
+            const int32_t i = t < m0 ? t : cap + t - m0;
             const int32_t v = nodes[i];
             Adj out;
+            int4 row[W / 4];
+#pragma unroll
+            for (int w = 0; w < W / 4; ++w)
+                row[w] = v >= 0 ? *reinterpret_cast<const int4 *>(a.ell + static_cast<int64_t>(v) * W + 4 * w)
+                                : make_int4(-1, -1, -1, -1);
+            int degree = 0;
 #pragma unroll
             for (int w = 0; w < W; ++w) {
-                const int32_t nb = v >= 0 ? a.ell[static_cast<int64_t>(v) * W + w] : -1;
+                const int32_t nb = w % 4 == 0 ? row[w / 4].x : w % 4 == 1 ? row[w / 4].y : w % 4 == 2 ? row[w / 4].z : row[w / 4].w;
+                degree += nb >= 0;
                 uint16_t id = static_cast<uint16_t>(N);
                 if (nb >= 0) {
                     if constexpr (GADJ) {
@@ -270,7 +359,7 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
                 out.v[w] = id;
             }
             adj[i] = out;
-            inv[i] = v >= 0 ? inv_deg[v] : Acc(0);
+            inv[i] = v >= 0 ? recip[degree] : Acc(0);
         }
         __syncthreads();
         forget();
@@ -283,25 +372,29 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
             for (int c = 0; c < C; ++c) z.v[c] = Acc(0);
             for (int b = 0; b < L::NBUF; ++b) {
                 Vec *xb = X + static_cast<size_t>(b) * (N + 1);
-                for (int32_t t = tid; t < n0 + n1; t += T) xb[t < n0 ? t : cap + t - n0] = z;
+                for (int32_t t = tid; t < m0 + m1; t += T) xb[t < m0 ? t : cap + t - m0] = z;
                 if (tid == 0) xb[N] = z;
             }
         }
         __syncthreads();
-        if (tid < C && src[tid] >= 0 && a.len[src[tid]] > 0) X[tid].v[tid] = Acc(1);
-        // the gather's threads (the last ones: they take the fewest rows): entry `gk` of source column `gq`
-        const int gt = T - 1 - tid;
-        const int gq = gt / W;
+        if (tid < C && src[tid] >= 0 && a.len[src[tid]] > 0) X[spos[tid]].v[tid] = Acc(1);
+        // the last warp gathers and computes no rows, so that the FP64 chain of a term (two
+        // conversions, a difference, a sum) runs beside the hop instead of behind it: lane gt holds
+        // entry `gk` of source column `gq`
+        const int TR = T - 32, gt = tid - TR;
+        const int gq = gt < 0 ? 0 : gt / W;
         int32_t gk = -1, glen = 0, gtau = 0;
         uint32_t gj = 0;
         double acc = 0.0, r1 = 0.0, r2 = 0.0;
-        if (gt < C * W && src[gq] >= 0 && a.len[src[gq]] > 0) {
+        int32_t gs = 0;
+        if (gt >= 0 && gt < C * W && src[gq] >= 0 && a.len[src[gq]] > 0) {
             const int32_t s = src[gq], b = a.row_ptr[s];
             if (gt % W < a.row_ptr[s + 1] - b) {
                 gk = b + gt % W;
                 glen = a.len[s];
                 gtau = a.tau[gk];
-                gj = adj[gq].v[gt % W];
+                gs = spos[gq];
+                gj = adj[gs].v[gt % W];
                 acc = a.g[gk];
                 r1 = a.t1[gk];
                 r2 = a.t2[gk];
@@ -310,7 +403,7 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
         auto gather = [&](int32_t h) {  // the hop-h term of Eq. 9 (gather_term, the sums in registers)
             if (gk < 0 || h > glen) return;
             const Vec *xb = X + (BIP ? 0 : static_cast<size_t>(h & 1) * (N + 1));
-            const double diag = BIP && (h & 1) ? 0.0 : static_cast<double>(xb[gq].v[gq]);
+            const double diag = BIP && (h & 1) ? 0.0 : static_cast<double>(xb[gs].v[gq]);
             const double xj = BIP && !(h & 1) ? 0.0 : static_cast<double>(xb[gj].v[gq]);
             const double term = diag - xj;
             if (h <= gtau) {
@@ -338,13 +431,14 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
             int32_t lim = min(min(h, Lg - h + 1), top);
             const int par = BIP ? (h & 1) : 0;
             if (BIP) lim -= (lim ^ h) & 1;
-            const int32_t rows = lim >= 0 ? lvl[lim] : 0;
+            const int32_t rows = by_id ? (par ? m1 : m0) : lim >= 0 ? lvl[lim] : 0;
             const Vec *xp = X + (BIP ? 0 : static_cast<size_t>((h - 1) & 1) * (N + 1));
             Vec *xn = X + (BIP ? 0 : static_cast<size_t>(h & 1) * (N + 1));
             const bool to_bf16 = h >= a.h0;
             const int32_t base = par * cap;
+            if (gt >= 0 && h >= 2) gather(h - 1);
 #pragma unroll 2
-            for (int32_t t = tid; t < rows; t += T) {
+            for (int32_t t = gt >= 0 ? rows : tid; t < rows; t += TR) {
                 const Adj id = adj[base + t];
                 Vec sum = xp[id.v[0]];
 #pragma unroll
@@ -363,7 +457,6 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
                     }
                 xn[base + t] = sum;
             }
-            if (h >= 2) gather(h - 1);
             __syncthreads();
         }
         gather(Lg);
@@ -549,7 +642,6 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
         ResArgs a{};
         a.row_ptr = g->row_ptr.get();
         a.ell = g->res_ell.get();
-        a.inv_deg = fp64 ? static_cast<const void *>(g->inv_deg_d.get()) : static_cast<const void *>(g->inv_deg_f.get());
         a.n = n;
         a.order = d_order.get();
         a.groups = g->res_list.get();
@@ -586,7 +678,44 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
             while (cls < kResClasses - 2 && h[0] > cap_of(cls)) ++cls;
             if (h[1] == ns) cls = kResClasses - 1;  // no ball of the sample fits with its adjacency
         }
-        for (; cls < kResClasses && !list.empty(); ++cls) {
+        // groups of small segments need no more than the class that holds the segment, which leaves
+        // room for more CTAs per SM: `list` starts with the smallest class in use, later classes get
+        // their own groups and the ones that did not fit
+        std::vector<int32_t> later[kResClasses];
+        if (cls < kResClasses - 1) {
+            std::vector<int32_t> seg_class(seg_start.size() - 1, cls);
+            int lowest = cls;
+            for (size_t i = 0; i + 1 < seg_start.size(); ++i) {
+                int &c = seg_class[i];
+                while (c > 0 && seg_start[i + 1] - seg_start[i] + width <= cap_of(c - 1)) --c;
+                if (seg_take[i] && (seg_bip[i] != 0) == bip) lowest = std::min(lowest, c);
+            }
+            if (lowest < cls) {
+                std::vector<int32_t> first;
+                for (int32_t q : list) {
+                    const int32_t v = order[static_cast<size_t>(q) * width];  // a group's first slot is taken
+                    const size_t i = std::upper_bound(seg_start.begin(), seg_start.end(), v) - seg_start.begin() - 1;
+                    (seg_class[i] == lowest ? first : later[seg_class[i]]).push_back(q);
+                }
+                list.swap(first);
+                cls = lowest;
+                SC_CUDA(cudaMemcpyAsync(g->res_list.get(), list.data(), list.size() * sizeof(int32_t),
+                                        cudaMemcpyHostToDevice, s));
+            }
+        }
+        auto more = [&](int c) {
+            for (int q = c; q < kResClasses; ++q)
+                if (!later[q].empty()) return true;
+            return false;
+        };
+        for (; cls < kResClasses && (!list.empty() || more(cls)); ++cls) {
+            if (!later[cls].empty()) {  // with what earlier classes left over
+                list.insert(list.end(), later[cls].begin(), later[cls].end());
+                later[cls].clear();
+                SC_CUDA(cudaMemcpyAsync(g->res_list.get(), list.data(), list.size() * sizeof(int32_t),
+                                        cudaMemcpyHostToDevice, s));
+            }
+            if (list.empty()) continue;
             if (cls == kResClasses - 1) {
                 // one source to a group, adjacency in global memory: bipartite graphs only (one
                 // buffer, half the rows a hop; without that the block kernels are as fast)
