@@ -1841,7 +1841,7 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
 
     // ---- truncation lengths --------------------------------------------------
     g->tau_entry.reserve(nnz);
-    DevBuf<int32_t> tau_src;
+    DevBuf<int32_t> &tau_src = g->ws_tau_src;
     tau_src.reserve(n);
     std::vector<int32_t> len(n);
     int32_t ell_global = 0;
@@ -1912,7 +1912,7 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
         rec_stride = even_stride;
     }
     // mode 3 records the terms of hops tau-1, tau here (and tau+1, tau+2 in t1 / t2)
-    DevBuf<double> pre_rec;
+    DevBuf<double> &pre_rec = g->ws_pre;
     if (learned3) {
         pre_rec.reserve(static_cast<size_t>(nnz) * 2);
         rec_all = pre_rec.get();
@@ -1996,8 +1996,8 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     // ---- propagation ----------------------------------------------------------
     SC_CUDA(cudaEventRecord(ev1, s));
     std::vector<int32_t> all;
-    DevBuf<int32_t> active;   // sc_some_edges: the endpoints of the listed entries
-    DevBuf<int64_t> d_entries;
+    DevBuf<int32_t> &active = g->ws_active;   // sc_some_edges: the endpoints of the listed entries
+    DevBuf<int64_t> &d_entries = g->ws_entries;
     if (sub) {
         active.reserve(n);
         d_entries.reserve(sub->count);
@@ -2036,7 +2036,7 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     run(all, len);
 
     // ---- combine, and for the learned lengths the check / extension loop ------
-    DevBuf<double> tmp_s, tmp_b;
+    DevBuf<double> &tmp_s = g->ws_s, &tmp_b = g->ws_b;
     double *d_s = s_hat;
     double *d_b = tail_bound;
     if (sub) {  // every entry's value in scratch; the listed ones are gathered at the end
@@ -2085,7 +2085,8 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     if (learned_plus) {
         // certify each edge's truncation (eps/2) after the run; failing edges take a longer
         // length and both endpoints run again (their walks included), until every edge passes
-        DevBuf<int32_t> row_flag, rows, d_depth, tau_target;
+        DevBuf<int32_t> &row_flag = g->ws_flag, &rows = g->ws_rows;
+        DevBuf<int32_t> d_depth, tau_target;
         row_flag.reserve(n);
         d_depth.reserve(n);
         tau_target.reserve(nnz);
@@ -2129,7 +2130,7 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
         }
         combine();
     } else if (learned) {
-        DevBuf<int32_t> row_flag, rows;
+        DevBuf<int32_t> &row_flag = g->ws_flag, &rows = g->ws_rows;
         row_flag.reserve(n);
         g->tp_counters.reserve(4);
         std::vector<int32_t> h_flag(n);
@@ -2178,7 +2179,7 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     SC_CUDA(cudaEventRecord(ev2, s));
 
     g->scratch_d.reserve(kRedBlocks + 8);
-    DevBuf<double> sub_s, sub_b;
+    DevBuf<double> &sub_s = g->ws_sub_s, &sub_b = g->ws_sub_b;
     int64_t red_count = nnz;
     if (sub) {  // the listed entries' values (and bounds), in the caller's order
         red_count = sub->count;
