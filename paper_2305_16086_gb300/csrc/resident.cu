@@ -31,7 +31,7 @@
 // why several CTAs share an SM when the ball is small. Whole calls, windowed
 // blocks against this: 150 x 613 strip at 67 + 2 hops 94 -> 8.4 ms, 400 x 400
 // lattice at learned lengths (37 to 353 hops) 625 -> 29.6 ms, 24 mixed graphs with
-// lattices of 1,000 to 5,000 nodes at 1,003 hops 223 -> 76 ms.
+// lattices of 1,000 to 5,000 nodes at 1,003 hops 223 -> 73 ms.
 #include <algorithm>
 #include <numeric>
 
