@@ -608,6 +608,14 @@ static int slices_for(const sc_graph *g, int B, size_t elem, int max_slices) {
 // source; cached per graph, precision, request and length. The gathers write
 // the accumulators, which the caller resets afterwards.
 // per_b (nullable): the best lane split of every block width, by the same model
+// A split is timed in full only while it can win: one that takes kTuneDropAtOnce
+// times the best hop of its width in its first timed launch, or kTuneDrop times
+// the width's best block after a round, is not timed again (two rounds of one
+// candidate differ by a few per cent; one row per warp won by 1.3 to 10 times in
+// every case timed, and the losers' launches, the longest, were four fifths of a
+// first call: create, estimate and run a 5,000-node graph 32.6 -> 17.4 ms).
+constexpr double kTuneDrop = 1.25, kTuneDropAtOnce = 1.75;
+
 static TuneResult autotune(sc_graph *g, int prec, int fixB, int fixV, int max_slices, int32_t L, const GatherRec &rec,
                            bool allow_tma, cudaStream_t s, std::vector<TuneResult> *per_b = nullptr) {
     L = std::max(L, 1);
@@ -622,7 +630,7 @@ static TuneResult autotune(sc_graph *g, int prec, int fixB, int fixV, int max_sl
     }
     std::vector<std::pair<int, int>> cands;
     for (int B : {32, 64, 128})
-        for (int v : {0, 1, 2, 4})
+        for (int v : {1, 2, 4, 0})  // first the split that nearly always wins (the others are measured against it)
             if ((fixB == 0 || fixB == B) && (fixV < 0 || fixV == v) && (v != 0 || allow_tma) && cfg_valid(prec, B, v))
                 cands.push_back({B, v});
     if (cands.empty()) SC_FAIL(SC_ERR_INVALID_ARG, "no admissible kernel for B=%d split=%d", fixB, fixV);
@@ -655,14 +663,39 @@ static TuneResult autotune(sc_graph *g, int prec, int fixB, int fixV, int max_sl
     // three interleaved rounds over the candidates (so that clock or cache drift
     // affects all of them alike), best round kept per candidate
     std::vector<double> best_block(cands.size(), INFINITY), best_hop(cands.size(), INFINITY);
+    auto best_of_width = [&](int B) {
+        double t = INFINITY;
+        for (size_t ci = 0; ci < cands.size(); ++ci)
+            if (cands[ci].first == B) t = std::min(t, best_block[ci]);
+        return t;
+    };
+    auto best_hop_of_width = [&](int B) {
+        double t = INFINITY;
+        for (size_t ci = 0; ci < cands.size(); ++ci)
+            if (cands[ci].first == B) t = std::min(t, best_hop[ci]);
+        return t;
+    };
     for (int round = 0; round < 3; ++round) {
         for (size_t ci = 0; ci < cands.size(); ++ci) {
             const auto &c = cands[ci];
+            if (round > 0 && best_block[ci] > kTuneDrop * best_of_width(c.first)) continue;
             const int sl = slices_for(g, c.first, elem, max_slices);
             const int nsrc = sl * c.first;
             const int32_t *src = g->src_list.get();
             HopLaunch h{g->xa.get(), g->xb.get(), sl, src, nsrc, tau, 1, acc_g, acc_t1, acc_t2, g->status.get(), rec};
-            if (round == 0) launch_hop(g, prec, c.first, c.second, h, s);  // warm-up
+            if (round == 0) {
+                launch_hop(g, prec, c.first, c.second, h, s);  // warm-up
+                const double rival = best_hop_of_width(c.first);
+                if (std::isfinite(rival)) {
+                    SC_CUDA(cudaEventRecord(ev[0], s));
+                    launch_hop(g, prec, c.first, c.second, h, s);
+                    SC_CUDA(cudaEventRecord(ev[1], s));
+                    SC_CUDA(cudaEventSynchronize(ev[1]));
+                    float t = 0.f;
+                    SC_CUDA(cudaEventElapsedTime(&t, ev[0], ev[1]));
+                    if (t / nsrc > kTuneDropAtOnce * rival) continue;
+                }
+            }
             const int reps = 4;
             SC_CUDA(cudaEventRecord(ev[0], s));
             SC_CUDA(cudaMemsetAsync(g->xa.get(), 0, static_cast<size_t>(nsrc) * g->n * elem, s));
