@@ -408,7 +408,7 @@ typedef struct sc_report {
     int32_t tt_min, tt_max;    /* TGT+: shortest / longest traversal before switching to walks */
     int32_t switch_tests;      /* TGT+: switch tests run */
     double switch_ms;          /* TGT+: wall time in switch tests (kernels, copies, host work) */
-    double walk_ms;            /* TGT+: wall time drawing walks (planning, kernels) */
+    double walk_ms;            /* TGT+: host time queueing walks plus walk_device_ms */
     int64_t source_hops;       /* sum over sources of hops traversed (the traversal's work) */
     int32_t extension_rounds;  /* learned policy: rerun rounds for edges that failed their bound */
     int32_t windowed;          /* 1 if the blocks ran windowed or resident (SC_OPT_WINDOWS_*) */

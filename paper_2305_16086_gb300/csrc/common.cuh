@@ -213,8 +213,9 @@ struct sc_graph {
     // TGT+ work buffers: CalChi partial and per-column statistics, walk counts
     sc::DevBuf<double> tp_pval, tp_pmin, tp_pmax, tp_cval, tp_cmin, tp_cmax, tp_cthr;
     sc::DevBuf<int32_t> tp_pid, tp_cid;
-    sc::DevBuf<long long> tp_pvol, tp_cvol, tp_walks, tp_counters, tp_packed, tp_chunk_w0;
-    sc::DevBuf<int32_t> tp_eq, tp_ek, tp_chunk_entry, tp_entry_chunk0;
+    sc::DevBuf<long long> tp_pvol, tp_cvol, tp_walks, tp_counters;
+    sc::DevBuf<int32_t> tp_src_chunks, tp_chunk0;  // per column, per CSR entry: chunks of walks, the first one
+    sc::DevBuf<int32_t> tp_chunk_q, tp_chunk_k;    // per chunk: its column and CSR entry
     sc::DevBuf<double> tp_chunk_sum;
     sc::DevBuf<double> tp_srcstat;  // per column: rho_hat, min and max of p over N(s)
     sc::DevBuf<long long> tp_src_rhs;  // per column: Eq. 14's right side (per-source switch)
@@ -228,8 +229,12 @@ struct sc_graph {
     bool res_ready = false;
     sc::DevBuf<unsigned char> res_scratch;
     std::vector<cudaEvent_t> hop_events;  // pairs bracketing timed propagation launches
+    std::vector<cudaEvent_t> walk_events;  // pairs bracketing TGT+ walk phases
+    long long *h_counters = nullptr;       // page-locked: a switch test's sums
     ~sc_graph() {
         for (cudaEvent_t e : hop_events) cudaEventDestroy(e);
+        for (cudaEvent_t e : walk_events) cudaEventDestroy(e);
+        if (h_counters) cudaFreeHost(h_counters);
     }
 };
 

@@ -24,13 +24,14 @@ sc_status estimate_lambda_impl(sc_graph *g, const sc_lambda_opts *opts, sc_lambd
 void tgtplus_reserve(sc_graph *g, int slices, int B);
 void tgtplus_check(sc_graph *g, int prec, int B, const void *x, int slices, const int32_t *src, const int32_t *h_src,
                    int nsrc, const int32_t *tau, int ell, int gamma, double eps, double log2md, bool full_scan,
-                   long long *lhs, long long *rhs, long long *steps, cudaStream_t s, long long *vol_src = nullptr,
-                   long long *rhs_src = nullptr);
+                   long long *lhs, long long *rhs, long long *steps, cudaStream_t s,
+                   std::vector<long long> *per_source = nullptr);
 void tgtplus_cap_rows(sc_graph *g, const int32_t *h_list, int count, int32_t cap, int32_t *tau, cudaStream_t s);
-long long tgtplus_walks(sc_graph *g, int prec, int B, const void *x, const int32_t *src, const int32_t *h_src,
-                        int nsrc, const int32_t *tau, int tt, uint64_t seed, double *acc_g, cudaStream_t s,
-                        long long *steps_out);
+void tgtplus_walks(sc_graph *g, int prec, int B, const void *x, const int32_t *src, const int32_t *h_src, int nsrc,
+                   const int32_t *now, long long pairs, const int32_t *tau, int tt, uint64_t seed, double *acc_g,
+                   cudaStream_t s);
 constexpr int kCostRuleHops = 4;  // the cost rule tests the last hops only
+constexpr size_t kWalkEventPairs = 512;  // walk phases timed before their events are read
 constexpr int kEvenDepthCap = 16;  // TGT+ at learned lengths: even hops recorded for the check (hop <= 16)
 // A block's hops 2, 3 and L-1 skip what is zero or not read (sparse_hops.cuh) when the graph is
 // large and the block's X_2 sparse, by an upper bound of its density: the walks of two hops from
@@ -1143,16 +1144,40 @@ static void run_blocks(Run &R, std::vector<int32_t> sources, const std::vector<i
     std::copy(sources.begin(), sources.end(), h_src.begin());
     g->src_list.reserve(h_src.size());
     SC_CUDA(cudaMemcpyAsync(g->src_list.get(), h_src.data(), h_src.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    cudaEvent_t ev_w0, ev_w1;
-    SC_CUDA(cudaEventCreate(&ev_w0));
-    SC_CUDA(cudaEventCreate(&ev_w1));
-    struct EvGuard {
-        cudaEvent_t a, b;
-        ~EvGuard() {
-            cudaEventDestroy(a);
-            cudaEventDestroy(b);
+    size_t walk_phases = 0;  // bracketed by events not yet read
+    auto read_walk_events = [&] {
+        for (size_t q = 0; q < walk_phases; ++q) {
+            float ms = 0.f;
+            SC_CUDA(cudaEventSynchronize(g->walk_events[2 * q + 1]));
+            SC_CUDA(cudaEventElapsedTime(&ms, g->walk_events[2 * q], g->walk_events[2 * q + 1]));
+            R.walk_device_ms += ms;
+            R.walk_ms += ms;
         }
-    } evg{ev_w0, ev_w1};
+        walk_phases = 0;
+    };
+    // Algorithm 4's walk phase from X_tt, with the counts of the last test; now: the sources it is
+    // for (null: the launch's)
+    auto draw_walks = [&](const void *x, int32_t tt, const int32_t *src, const int32_t *h_list, int nsrc,
+                          const int32_t *now, long long pairs, long long steps) {
+        if (walk_phases == kWalkEventPairs) read_walk_events();
+        const double t0 = wall_ms();
+        while (g->walk_events.size() < 2 * (walk_phases + 1)) {
+            cudaEvent_t e;
+            SC_CUDA(cudaEventCreate(&e));
+            g->walk_events.push_back(e);
+        }
+        const int64_t t = timer_open(R, s);
+        SC_CUDA(cudaEventRecord(g->walk_events[2 * walk_phases], s));
+        tgtplus_walks(g, prec_at(R, tt), B, x, src, h_list, nsrc, now, pairs, g->tau_entry.get(), tt, R.o->seed,
+                      g->acc_g.get(), s);
+        SC_CUDA(cudaEventRecord(g->walk_events[2 * walk_phases + 1], s));
+        timer_close(R, t, SC_KC_WALKS, 0.0, s);
+        ++walk_phases;
+        R.walk_ms += wall_ms() - t0;
+        R.launches += 3;
+        R.walks += pairs;
+        R.walk_steps += steps;
+    };
     // algorithmic bytes of hop ell per slice: CSR, 1/d, read X_{ell-1}, write X_ell
     const double csr_bytes = 4.0 * nnz + 4.0 * (n + 1) + (R.prec == SC_PREC_FP64 ? 8.0 : 4.0) * n;  // + 1/d
     const double mask_bytes = static_cast<double>(n) * B / 8.0;
@@ -1231,11 +1256,12 @@ static void run_blocks(Run &R, std::vector<int32_t> sources, const std::vector<i
             R.launches += 1;  // the memset is not a kernel of ours
         }
         int32_t tt = L;  // hops traversed; TGT+ may switch to walks earlier
+        long long walk_pairs = 0, walk_steps = 0;
         bool last_done = false;
         // per-source switch (Algorithm 4's loop per source): each source's switch hop, -1 while traversing
         const bool per_source = R.plus && R.o->switch_rule == SC_SWITCH_PER_SOURCE;
         std::vector<int32_t> src_tt(per_source ? nsrc : 0, -1), now_list(per_source ? nsrc : 0, -1);
-        std::vector<long long> vol_src(per_source ? nsrc : 0), rhs_src(per_source ? nsrc : 0);
+        std::vector<long long> side;  // per source: frontier volume, walks, walk steps
         int n_active = 0;
         for (int q = 0; per_source && q < nsrc; ++q) n_active += h_src[first + q] >= 0 ? 1 : 0;
         for (int ell = ell0; ell <= L; ++ell) {
@@ -1249,39 +1275,26 @@ static void run_blocks(Run &R, std::vector<int32_t> sources, const std::vector<i
                 const int64_t tc = timer_open(R, s);
                 tgtplus_check(g, prec_at(R, ell - 1), B, xa, used_slices, src, h_src.data() + first, nsrc,
                               g->tau_entry.get(), ell - 1, R.gamma, R.o->eps, R.log2md, full_scan, &lhs, &rhs,
-                              &steps, s, vol_src.data(), rhs_src.data());
+                              &steps, s, &side);
                 timer_close(R, tc, SC_KC_SWITCH_TEST, used_slices * test_bytes_per_slice(ell - 1), s);
                 R.switch_ms += wall_ms() - t0;
                 ++R.switch_tests;
                 R.launches += 4;
                 int nnow = 0;
+                long long now_pairs = 0, now_steps = 0;
                 for (int q = 0; q < nsrc; ++q) {
                     now_list[q] = -1;
                     const int32_t v = h_src[first + q];
-                    if (v >= 0 && src_tt[q] < 0 && vol_src[q] > rhs_src[q]) {
+                    if (v >= 0 && src_tt[q] < 0 && side[q] > side[nsrc + q]) {
                         now_list[q] = v;
                         src_tt[q] = ell - 1;
                         ++nnow;
+                        now_pairs += side[nsrc + q];
+                        now_steps += side[2 * static_cast<size_t>(nsrc) + q];
                     }
                 }
                 if (nnow > 0) {
-                    const double tw = wall_ms();
-                    const int64_t tw_ev = timer_open(R, s);
-                    SC_CUDA(cudaEventRecord(ev_w0, s));
-                    long long wsteps = 0;
-                    const long long pairs = tgtplus_walks(g, prec_at(R, ell - 1), B, xa, src, now_list.data(), nsrc,
-                                                          g->tau_entry.get(), ell - 1, R.o->seed, g->acc_g.get(), s,
-                                                          &wsteps);
-                    SC_CUDA(cudaEventRecord(ev_w1, s));
-                    timer_close(R, tw_ev, SC_KC_WALKS, 0.0, s);
-                    SC_CUDA(cudaEventSynchronize(ev_w1));
-                    R.walk_ms += wall_ms() - tw;
-                    R.launches += 3;
-                    R.walks += pairs;
-                    float wms = 0.f;
-                    SC_CUDA(cudaEventElapsedTime(&wms, ev_w0, ev_w1));
-                    R.walk_steps += wsteps;
-                    R.walk_device_ms += wms;
+                    draw_walks(xa, ell - 1, src, h_src.data() + first, nsrc, now_list.data(), now_pairs, now_steps);
                     tgtplus_cap_rows(g, now_list.data(), nsrc, ell - 1, g->tau_entry.get(), s);
                     R.launches += 1;
                     n_active -= nnow;
@@ -1312,6 +1325,8 @@ static void run_blocks(Run &R, std::vector<int32_t> sources, const std::vector<i
                                               static_cast<double>(L - (ell - 1)) * hop_ns);
                 if (go) {
                     tt = ell - 1;
+                    walk_pairs = rhs;
+                    walk_steps = steps;
                     break;
                 }
             }
@@ -1381,26 +1396,11 @@ static void run_blocks(Run &R, std::vector<int32_t> sources, const std::vector<i
             prev_L = L;
             prev_tt = tt < L ? tt : -1;
             if (tt < L) {
-                // Algorithm 4's walk phase: walk tails from X_tt with the counts of the last check
-                const double t0 = wall_ms();
-                const int64_t tw_ev = timer_open(R, s);
-                SC_CUDA(cudaEventRecord(ev_w0, s));
-                long long wsteps = 0;
-                const long long pairs = tgtplus_walks(g, prec_at(R, tt), B, xa, src, h_src.data() + first, nsrc,
-                                                      g->tau_entry.get(), tt, R.o->seed, g->acc_g.get(), s, &wsteps);
-                SC_CUDA(cudaEventRecord(ev_w1, s));
-                timer_close(R, tw_ev, SC_KC_WALKS, 0.0, s);
-                SC_CUDA(cudaEventSynchronize(ev_w1));
-                R.walk_ms += wall_ms() - t0;
-                R.launches += 3;
-                R.walks += pairs;
-                float wms = 0.f;
-                SC_CUDA(cudaEventElapsedTime(&wms, ev_w0, ev_w1));
-                R.walk_steps += wsteps;
-                R.walk_device_ms += wms;
+                draw_walks(xa, tt, src, h_src.data() + first, nsrc, nullptr, walk_pairs, walk_steps);
             }
         }
     }
+    read_walk_events();
     int32_t h_status = 0;
     SC_CUDA(cudaMemcpyAsync(&h_status, g->status.get(), sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     SC_CUDA(cudaStreamSynchronize(s));

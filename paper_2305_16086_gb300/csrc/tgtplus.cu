@@ -53,6 +53,8 @@ static void chi_check_t(sc_graph *g, const void *x, int slices, const int32_t *s
     a.log_2m_delta = log2md;
     a.walk_count = g->tp_walks.get();
     a.rhs = g->tp_counters.get();
+    a.cvol = g->tp_cvol.get();
+    a.src_chunks = g->tp_src_chunks.get();
     k_chi_source<T, B><<<nsrc, 32, 0, s>>>(static_cast<const T *>(x), a, g->tp_srcstat.get());
     const int nw = 256 / 32;
     dim3 grid(nsrc, std::min(ceil_div(std::max(max_deg, 1), nw * kChiEntries), 65535));
@@ -61,7 +63,7 @@ static void chi_check_t(sc_graph *g, const void *x, int slices, const int32_t *s
 
 template <typename T, int B>
 static void walks_t(sc_graph *g, const void *x, const int32_t *src, int nsrc, const int32_t *tau, int tt,
-                    uint64_t seed, const WalkChunkArgs &c, cudaStream_t s) {
+                    uint64_t seed, const WalkChunkArgs &c, int64_t max_chunks, cudaStream_t s) {
     WalkArgs a{};
     a.row_ptr = g->row_ptr.get();
     a.col = g->col_idx.get();
@@ -74,7 +76,7 @@ static void walks_t(sc_graph *g, const void *x, const int32_t *src, int nsrc, co
     a.g = nullptr;
     a.key0 = static_cast<uint32_t>(seed);
     a.key1 = static_cast<uint32_t>(seed >> 32);
-    k_walk_chunks<T, B><<<ceil_div(c.nchunks, 8), 256, 0, s>>>(static_cast<const T *>(x), a, c);
+    k_walk_chunks<T, B><<<ceil_div(max_chunks, 8), 256, 0, s>>>(static_cast<const T *>(x), a, c);
 }
 
 #define SC_DISPATCH_TB(prec, B, FN, ...)                                                   \
@@ -109,112 +111,85 @@ void tgtplus_reserve(sc_graph *g, int slices, int B) {
     g->tp_cthr.reserve(cols);
     g->tp_cvol.reserve(cols);
     g->tp_srcstat.reserve(3 * cols);
-    g->tp_src_rhs.reserve(cols);
+    g->tp_src_rhs.reserve(2 * cols);
+    g->tp_src_chunks.reserve(cols + 1);  // and their total
     g->tp_cap_list.reserve(cols);
     g->tp_walks.reserve(g->nnz);
+    g->tp_chunk0.reserve(g->nnz);
     g->tp_counters.reserve(4);
+    if (!g->h_counters) SC_CUDA(cudaMallocHost(reinterpret_cast<void **>(&g->h_counters), 4 * sizeof(long long)));
 }
 
 // Eq. 14 after hop `ell` for the launch's sources: returns the two sides
 // (frontier volume, sum of walk counts); the per-entry walk counts for
-// L = tau_k - ell stay in g->tp_walks for the walk kernel. vol_src / rhs_src
-// (host, nsrc each; may be null): the two sides per source.
+// L = tau_k - ell stay in g->tp_walks for the walk kernel, and *steps is their
+// number of walk steps. per_source (may be null): the two sides and the walk
+// steps per source (nsrc each, in turn).
 void tgtplus_check(sc_graph *g, int prec, int B, const void *x, int slices, const int32_t *src, const int32_t *h_src,
                    int nsrc, const int32_t *tau, int ell, int gamma, double eps, double log2md, bool full_scan,
-                   long long *lhs, long long *rhs, long long *steps, cudaStream_t s, long long *vol_src,
-                   long long *rhs_src) {
+                   long long *lhs, long long *rhs, long long *steps, cudaStream_t s,
+                   std::vector<long long> *per_source) {
     SC_CUDA(cudaMemsetAsync(g->tp_counters.get(), 0, 4 * sizeof(long long), s));
     int max_deg = 0;
     for (int q = 0; q < nsrc; ++q)
         if (h_src[q] >= 0) max_deg = std::max(max_deg, g->h_row_ptr[h_src[q] + 1] - g->h_row_ptr[h_src[q]]);
     SC_DISPATCH_TB(prec, B, chi_check_t, g, x, slices, src, nsrc, max_deg, tau, ell, gamma, eps, log2md, full_scan, s);
     SC_LAUNCH_CHECK();
-    std::vector<long long> vol(static_cast<size_t>(slices) * B);
-    long long h_cnt[3] = {0, 0, 0};
-    SC_CUDA(cudaMemcpyAsync(vol.data(), g->tp_cvol.get(), vol.size() * sizeof(long long), cudaMemcpyDeviceToHost, s));
-    SC_CUDA(cudaMemcpyAsync(h_cnt, g->tp_counters.get(), 3 * sizeof(long long), cudaMemcpyDeviceToHost, s));
-    if (rhs_src) {
-        k_walks_per_source<<<nsrc, 32, 0, s>>>(g->row_ptr.get(), src, nsrc, g->tp_walks.get(), g->tp_src_rhs.get());
+    SC_CUDA(cudaMemcpyAsync(g->h_counters, g->tp_counters.get(), 3 * sizeof(long long), cudaMemcpyDeviceToHost, s));
+    if (per_source) {
+        per_source->assign(3 * static_cast<size_t>(nsrc), 0);
+        k_walks_per_source<<<nsrc, 32, 0, s>>>(g->row_ptr.get(), src, nsrc, g->tp_walks.get(), tau, ell,
+                                               g->tp_src_rhs.get());
         SC_LAUNCH_CHECK();
-        SC_CUDA(cudaMemcpyAsync(rhs_src, g->tp_src_rhs.get(), nsrc * sizeof(long long), cudaMemcpyDeviceToHost, s));
+        SC_CUDA(cudaMemcpyAsync(per_source->data(), g->tp_cvol.get(), nsrc * sizeof(long long), cudaMemcpyDeviceToHost, s));
+        SC_CUDA(cudaMemcpyAsync(per_source->data() + nsrc, g->tp_src_rhs.get(), 2 * nsrc * sizeof(long long),
+                                cudaMemcpyDeviceToHost, s));
     }
     SC_CUDA(cudaStreamSynchronize(s));
-    if (vol_src)
-        for (int q = 0; q < nsrc; ++q) vol_src[q] = h_src[q] >= 0 ? vol[q] : 0;
-    long long h_lhs = 0;
-    for (int q = 0; q < nsrc; ++q)
-        if (h_src[q] >= 0) h_lhs += vol[q];
-    *lhs = h_lhs;
-    *rhs = h_cnt[0];
-    *steps = h_cnt[2];
+    if (per_source)
+        for (int q = 0; q < nsrc; ++q)
+            if (h_src[q] < 0) (*per_source)[q] = 0;
+    *rhs = g->h_counters[0];
+    *lhs = g->h_counters[1];
+    *steps = g->h_counters[2];
 }
 
-// Algorithm 4's walk phase for the launch's sources: the entries' walk pairs are cut
-// into chunks of kWalkChunk (planned on the host from the packed counts), one
-// warp per chunk, and each entry adds its chunk sums in chunk order.
-// Returns the number of walk pairs drawn; *steps_out (nullable) receives their
-// walk steps, 2 R (tau_k - tt) summed over the planned entries.
-long long tgtplus_walks(sc_graph *g, int prec, int B, const void *x, const int32_t *src, const int32_t *h_src,
-                        int nsrc, const int32_t *tau, int tt, uint64_t seed, double *acc_g, cudaStream_t s,
-                        long long *steps_out) {
-    if (steps_out) *steps_out = 0;
-    std::vector<int32_t> eq, ek;
+// Algorithm 4's walk phase for the launch's sources, or (now not null, on the
+// host) those of them it lists, -1 for the others: the entries' walk pairs are cut
+// into chunks of kWalkChunk, one warp per chunk, and each entry adds its chunk
+// sums in chunk order. pairs: their walk pairs, from the test. Nothing waits for
+// the host.
+void tgtplus_walks(sc_graph *g, int prec, int B, const void *x, const int32_t *src, const int32_t *h_src, int nsrc,
+                   const int32_t *now, long long pairs, const int32_t *tau, int tt, uint64_t seed, double *acc_g,
+                   cudaStream_t s) {
+    if (pairs <= 0) return;
+    int64_t max_chunks = pairs / kWalkChunk;  // an entry's last chunk may be short
     for (int q = 0; q < nsrc; ++q) {
-        const int32_t v = h_src[q];
-        if (v < 0) continue;
-        for (int32_t k = g->h_row_ptr[v]; k < g->h_row_ptr[v + 1]; ++k) {
-            eq.push_back(q);
-            ek.push_back(k);
-        }
+        const int32_t v = now ? now[q] : h_src[q];
+        if (v >= 0) max_chunks += g->h_row_ptr[v + 1] - g->h_row_ptr[v];
     }
-    const int32_t ne = static_cast<int32_t>(ek.size());
-    if (ne == 0) return 0;
-    g->tp_eq.reserve(ne);
-    g->tp_ek.reserve(ne);
-    g->tp_packed.reserve(2 * static_cast<size_t>(ne));
-    SC_CUDA(cudaMemcpyAsync(g->tp_eq.get(), eq.data(), ne * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    SC_CUDA(cudaMemcpyAsync(g->tp_ek.get(), ek.data(), ne * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    k_pack_counts<<<ceil_div(ne, 256), 256, 0, s>>>(g->tp_ek.get(), ne, g->tp_walks.get(), tau, tt,
-                                                    g->tp_packed.get());
-    SC_LAUNCH_CHECK();
-    std::vector<long long> R(2 * static_cast<size_t>(ne));
-    SC_CUDA(cudaMemcpyAsync(R.data(), g->tp_packed.get(), 2 * static_cast<size_t>(ne) * sizeof(long long),
-                            cudaMemcpyDeviceToHost, s));
-    SC_CUDA(cudaStreamSynchronize(s));
-    if (steps_out)
-        for (int32_t e = 0; e < ne; ++e) *steps_out += R[ne + e];
-    std::vector<int32_t> chunk_entry, entry_chunk0(ne + 1);
-    std::vector<long long> chunk_w0;
-    long long pairs = 0;
-    for (int32_t e = 0; e < ne; ++e) {
-        entry_chunk0[e] = static_cast<int32_t>(chunk_entry.size());
-        for (long long w = 0; w < R[e]; w += kWalkChunk) {
-            chunk_entry.push_back(e);
-            chunk_w0.push_back(w);
-        }
-        pairs += R[e] > 0 ? R[e] : 0;
+    if (max_chunks > INT32_MAX) SC_FAIL(SC_ERR_UNSUPPORTED, "too many walks in a launch");
+    if (static_cast<size_t>(max_chunks) > g->tp_chunk_sum.count) {  // with room for the launches to come
+        const size_t room = static_cast<size_t>(max_chunks) + static_cast<size_t>(max_chunks) / 2;
+        g->tp_chunk_q.reserve(room);
+        g->tp_chunk_k.reserve(room);
+        g->tp_chunk_sum.reserve(room);
     }
-    entry_chunk0[ne] = static_cast<int32_t>(chunk_entry.size());
-    const int32_t nch = static_cast<int32_t>(chunk_entry.size());
-    if (nch == 0) return 0;
-    g->tp_chunk_entry.reserve(nch);
-    g->tp_chunk_w0.reserve(nch);
-    g->tp_chunk_sum.reserve(nch);
-    g->tp_entry_chunk0.reserve(ne + 1);
-    SC_CUDA(cudaMemcpyAsync(g->tp_chunk_entry.get(), chunk_entry.data(), nch * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    SC_CUDA(cudaMemcpyAsync(g->tp_chunk_w0.get(), chunk_w0.data(), nch * sizeof(long long), cudaMemcpyHostToDevice, s));
-    SC_CUDA(cudaMemcpyAsync(g->tp_entry_chunk0.get(), entry_chunk0.data(), (ne + 1) * sizeof(int32_t),
-                            cudaMemcpyHostToDevice, s));
-    WalkChunkArgs c{g->tp_eq.get(), g->tp_ek.get(), g->tp_chunk_entry.get(), g->tp_chunk_w0.get(), nch,
-                    g->tp_chunk_sum.get()};
-    SC_DISPATCH_TB(prec, B, walks_t, g, x, src, nsrc, tau, tt, seed, c, s);
+    const int32_t *list = src;
+    if (now) {
+        SC_CUDA(cudaMemcpyAsync(g->tp_cap_list.get(), now, nsrc * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+        list = g->tp_cap_list.get();
+    }
+    int32_t *total = g->tp_src_chunks.get() + g->tp_src_chunks.count - 1;
+    k_walk_plan<<<nsrc, 128, 0, s>>>(g->row_ptr.get(), list, nsrc, g->tp_src_chunks.get(), g->tp_walks.get(),
+                                     g->tp_chunk0.get(), g->tp_chunk_q.get(), g->tp_chunk_k.get(), total);
     SC_LAUNCH_CHECK();
-    k_walk_finish<<<ceil_div(ne, 256), 256, 0, s>>>(g->tp_ek.get(), g->tp_entry_chunk0.get(), ne,
-                                                    g->tp_chunk_sum.get(), g->tp_walks.get(), acc_g);
+    WalkChunkArgs c{g->tp_chunk_q.get(), g->tp_chunk_k.get(), g->tp_chunk0.get(), total, g->tp_chunk_sum.get()};
+    SC_DISPATCH_TB(prec, B, walks_t, g, x, src, nsrc, tau, tt, seed, c, max_chunks, s);
     SC_LAUNCH_CHECK();
-    // the host buffers above are read by the async copies: finish before they go out of scope
-    SC_CUDA(cudaStreamSynchronize(s));
-    return pairs;
+    k_walk_finish<<<nsrc, 128, 0, s>>>(g->row_ptr.get(), list, g->tp_chunk0.get(), g->tp_chunk_sum.get(),
+                                       g->tp_walks.get(), acc_g);
+    SC_LAUNCH_CHECK();
 }
 
 // Caps tau at `cap` on the rows of the listed nodes (host list of count, -1 = skip).

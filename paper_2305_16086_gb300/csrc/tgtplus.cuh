@@ -551,8 +551,16 @@ struct ChiArgs {
     const int32_t *cid;
     double eps, log_2m_delta;
     long long *walk_count;   // per CSR entry (0 = no walks)
-    long long *rhs;          // [0] sum of the launch's walk counts (Eq. 14 right side), [2] walk steps
+    long long *rhs;          // [0] sum of the launch's walk counts (Eq. 14 right side), [1] left side, [2] walk steps
+    const long long *cvol;   // per column: frontier volume
+    int32_t *src_chunks;     // per column: chunks of kWalkChunk walk pairs of its entries
 };
+
+constexpr int kWalkChunk = 128;  // walk pairs per warp-sized chunk
+
+__host__ __device__ __forceinline__ long long walk_chunks(long long pairs) {
+    return pairs > 0 ? (pairs + kWalkChunk - 1) / kWalkChunk : 0;
+}
 
 // Per source (one warp): rho_hat (Alg. 3) and min / max of p over N(i),
 // into stat[3 q .. 3 q + 2].
@@ -562,6 +570,10 @@ __global__ void k_chi_source(const T *__restrict__ x, const ChiArgs a, double *_
     const int lane = threadIdx.x & 31;
     if (q >= a.nsrc) return;
     const int32_t s = a.src[q];
+    if (lane == 0) {
+        a.src_chunks[q] = 0;
+        if (s >= 0) atomicAdd(reinterpret_cast<unsigned long long *>(a.rhs + 1), static_cast<unsigned long long>(a.cvol[q]));
+    }
     if (s < 0) return;
     const T *xs = x + static_cast<int64_t>(q / B) * a.n * B + (q % B);
     using V = typename AccOf<T>::type;
@@ -618,13 +630,10 @@ __global__ void k_chi_entries(const T *__restrict__ x, const ChiArgs a, const do
     const int g = a.gamma;
     const int32_t rb = a.row_ptr[s], re = a.row_ptr[s + 1];
     if (rb + static_cast<int32_t>(blockIdx.y) * nw * kChiEntries >= re) return;  // CTA-uniform
-    __shared__ unsigned long long sh_cnt[2];
-    if (threadIdx.x == 0) {
-        sh_cnt[0] = 0;
-        sh_cnt[1] = 0;
-    }
+    __shared__ unsigned long long sh_cnt[3];
+    if (threadIdx.x < 3) sh_cnt[threadIdx.x] = 0;
     __syncthreads();
-    unsigned long long local = 0, steps = 0;
+    unsigned long long local = 0, steps = 0, chunks = 0;
     for (int32_t k0 = rb + (static_cast<int32_t>(blockIdx.y) * nw + warp) * kChiEntries; k0 < re;
          k0 += static_cast<int32_t>(gridDim.y) * nw * kChiEntries) {
         const bool in = lane < kChiEntries && k0 + lane < re;
@@ -684,15 +693,19 @@ __global__ void k_chi_entries(const T *__restrict__ x, const ChiArgs a, const do
         a.walk_count[k] = R;
         local += static_cast<unsigned long long>(R);
         steps += static_cast<unsigned long long>(R) * 2ull * static_cast<unsigned long long>(L);
+        chunks += static_cast<unsigned long long>(walk_chunks(R));
     }
     if (local) {
         atomicAdd(&sh_cnt[0], local);
         atomicAdd(&sh_cnt[1], steps);
+        atomicAdd(&sh_cnt[2], chunks);
     }
     __syncthreads();
     if (threadIdx.x == 0 && sh_cnt[0]) {
         atomicAdd(reinterpret_cast<unsigned long long *>(a.rhs), sh_cnt[0]);
         atomicAdd(reinterpret_cast<unsigned long long *>(a.rhs + 2), sh_cnt[1]);
+        // (a count past 32 bits belongs to a test whose walks are not drawn)
+        atomicAdd(&a.src_chunks[q], static_cast<int32_t>(min(sh_cnt[2], 0x7fffffffull)));
     }
 }
 
@@ -704,93 +717,171 @@ struct WalkArgs {
     uint32_t key0, key1;
 };
 
-// sum_{t=1..L} X[W[t]] for walk w of entry k on one side (Eq. 11)
-template <typename T, int B>
-__device__ __forceinline__ double walk_sum(const WalkArgs &a, const T *__restrict__ xs, int32_t start, int32_t L,
-                                           uint32_t k, uint32_t w, uint32_t side) {
-    int32_t cur = start;
-    double sum = 0.0;
-    Philox4 words{};
-    for (int32_t t = 1; t <= L; ++t) {
-        const int r = (t - 1) & 3;
-        if (r == 0)
-            words = philox4x32_10(k, w, (side << 31) | static_cast<uint32_t>((t - 1) >> 2), kWalkTag, a.key0, a.key1);
-        const int32_t b = a.row_ptr[cur];
-        const uint32_t d = static_cast<uint32_t>(a.row_ptr[cur + 1] - b);
-        const uint32_t idx = static_cast<uint32_t>((static_cast<uint64_t>(words.v[r]) * d) >> 32);
-        cur = a.col[b + idx];
-        sum += static_cast<double>(to_acc(xs[static_cast<int64_t>(cur) * B]));
+// The walks of Algorithm 4's second phase run without the host: it knows their
+// number from the test that chose them, which bounds the chunks, and the plan is
+// made on the device: for 192 sources of a 40,000-node Barabasi-Albert graph the
+// phase took 81 us planned on the host, of which its kernels 19, and takes 31 so
+// (events on both sides included). The walks themselves are bound by the latency
+// of a step's three dependent loads, so a pair's two walks advance together.
+
+// The plan, one CTA per column of `list` (-1: draws none): its entries' chunks
+// follow those of the columns before it, in CSR order. chunk0[k]: the first chunk
+// of entry k; chunk_q / chunk_k: a chunk's column and entry; *total: all chunks.
+static __global__ void __launch_bounds__(128) k_walk_plan(const int32_t *__restrict__ row_ptr,
+                                                          const int32_t *__restrict__ list, int32_t nsrc,
+                                                          const int32_t *__restrict__ src_chunks,
+                                                          const long long *__restrict__ walk_count,
+                                                          int32_t *__restrict__ chunk0, int32_t *__restrict__ chunk_q,
+                                                          int32_t *__restrict__ chunk_k, int32_t *__restrict__ total) {
+    __shared__ int32_t part[4], warp_sum[4];
+    const int32_t q = blockIdx.x;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int32_t before = 0;
+    for (int32_t p = threadIdx.x; p < q; p += 128)
+        if (list[p] >= 0) before += src_chunks[p];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    if (lane == 0) part[warp] = before;
+    __syncthreads();
+    int32_t at = part[0] + part[1] + part[2] + part[3];
+    const int32_t s = list[q];
+    if (q == nsrc - 1 && threadIdx.x == 0) *total = at + (s >= 0 ? src_chunks[q] : 0);
+    if (s < 0) return;
+    const int32_t rb = row_ptr[s], re = row_ptr[s + 1];
+    for (int32_t k0 = rb; k0 < re; k0 += 128) {  // CTA-uniform
+        const int32_t k = k0 + static_cast<int32_t>(threadIdx.x);
+        const int32_t mine = k < re ? static_cast<int32_t>(walk_chunks(walk_count[k])) : 0;
+        int32_t inc = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t up = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += up;
+        }
+        if (lane == 31) warp_sum[warp] = inc;
+        __syncthreads();
+        int32_t here = at + inc - mine;
+        for (int w = 0; w < warp; ++w) here += warp_sum[w];
+        if (k < re) chunk0[k] = here;
+        for (uint32_t todo = __ballot_sync(0xffffffffu, mine > 0); todo; todo &= todo - 1u) {  // warp-uniform
+            const int l = __ffs(todo) - 1;
+            const int32_t first = __shfl_sync(0xffffffffu, here, l), count = __shfl_sync(0xffffffffu, mine, l);
+            const int32_t kl = __shfl_sync(0xffffffffu, k, l);
+            for (int32_t c = lane; c < count; c += 32) {
+                chunk_q[first + c] = q;
+                chunk_k[first + c] = kl;
+            }
+        }
+        at += warp_sum[0] + warp_sum[1] + warp_sum[2] + warp_sum[3];
+        __syncthreads();
     }
-    return sum;
 }
 
-constexpr int kWalkChunk = 128;  // walk pairs per warp-sized chunk
-
 struct WalkChunkArgs {
-    const int32_t *entry_q;     // per planned entry: launch source index q
-    const int32_t *entry_k;     // per planned entry: CSR entry k
-    const int32_t *chunk_entry; // per chunk: planned entry index
-    const long long *chunk_w0;  // per chunk: first walk index
-    int32_t nchunks;
-    double *chunk_sum;          // per chunk: sum over its walks of (S_i - S_j)
+    const int32_t *chunk_q, *chunk_k, *chunk0;  // of k_walk_plan
+    const int32_t *total;                       // chunks
+    double *chunk_sum;                          // per chunk: sum over its walks of (S_i - S_j)
 };
+
+// Walk pair w of entry k: sum_{t=1..L} X[W[t]] from both ends (Eq. 11), their difference
+template <typename T, int B>
+__device__ __forceinline__ double walk_pair(const WalkArgs &a, const T *__restrict__ xs, int32_t i, int32_t j,
+                                            int32_t L, uint32_t k, uint32_t w) {
+    int32_t cur[2] = {i, j};
+    double sum[2] = {0.0, 0.0};
+    Philox4 words[2] = {};
+    for (int32_t t = 1; t <= L; ++t) {
+        const int r = (t - 1) & 3;
+        if (r == 0) {
+#pragma unroll
+            for (uint32_t side = 0; side < 2; ++side)
+                words[side] = philox4x32_10(k, w, (side << 31) | static_cast<uint32_t>((t - 1) >> 2), kWalkTag, a.key0,
+                                            a.key1);
+        }
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+            const int32_t b = a.row_ptr[cur[side]];
+            const uint32_t d = static_cast<uint32_t>(a.row_ptr[cur[side] + 1] - b);
+            const uint32_t word = r == 0 ? words[side].v[0] : r == 1 ? words[side].v[1]
+                                : r == 2 ? words[side].v[2] : words[side].v[3];
+            cur[side] = a.col[b + static_cast<uint32_t>((static_cast<uint64_t>(word) * d) >> 32)];
+        }
+#pragma unroll
+        for (int side = 0; side < 2; ++side)
+            sum[side] += static_cast<double>(to_acc(xs[static_cast<int64_t>(cur[side]) * B]));
+    }
+    return sum[0] - sum[1];
+}
 
 // One warp per chunk of walk pairs of one entry; lanes take walks w0 + lane,
 // w0 + lane + 32, ... in the chunk; the chunk sum is reduced by a fixed tree.
 template <typename T, int B>
 __global__ void k_walk_chunks(const T *__restrict__ x, const WalkArgs a, const WalkChunkArgs c) {
-    const int32_t ch = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int64_t ch = blockIdx.x * static_cast<int64_t>(blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    if (ch >= c.nchunks) return;
-    const int32_t e = c.chunk_entry[ch];
-    const int32_t q = c.entry_q[e], k = c.entry_k[e];
+    if (ch >= *c.total) return;
+    const int32_t q = c.chunk_q[ch], k = c.chunk_k[ch];
     const int32_t s = a.src[q];
     const T *xs = x + static_cast<int64_t>(q / B) * a.n * B + (q % B);
     const long long R = a.walk_count[k];
-    const long long w0 = c.chunk_w0[ch];
+    const long long w0 = (ch - c.chunk0[k]) * kWalkChunk;
     const long long w1 = min(R, w0 + kWalkChunk);
     const int32_t L = a.tau[k] - a.tt;
     const int32_t j = a.col[k];
     double acc = 0.0;
-    for (long long w = w0 + lane; w < w1; w += 32) {
-        const double si = walk_sum<T, B>(a, xs, s, L, static_cast<uint32_t>(k), static_cast<uint32_t>(w), 0u);
-        const double sj = walk_sum<T, B>(a, xs, j, L, static_cast<uint32_t>(k), static_cast<uint32_t>(w), 1u);
-        acc += si - sj;
-    }
+    for (long long w = w0 + lane; w < w1; w += 32)
+        acc += walk_pair<T, B>(a, xs, s, j, L, static_cast<uint32_t>(k), static_cast<uint32_t>(w));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) c.chunk_sum[ch] = acc;
 }
 
-// g[k] += (sum of the entry's chunk sums, in chunk order) / R_k  (Algorithm 4's walk estimate)
-static __global__ void k_walk_finish(const int32_t *__restrict__ entry_k, const int32_t *__restrict__ entry_chunk0,
-                              int32_t nentries, const double *__restrict__ chunk_sum,
-                              const long long *__restrict__ walk_count, double *__restrict__ g) {
-    const int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nentries) return;
-    const int32_t k = entry_k[e];
-    const long long R = walk_count[k];
-    if (R <= 0) return;
-    double t = 0.0;
-    for (int32_t ch = entry_chunk0[e]; ch < entry_chunk0[e + 1]; ++ch) t += chunk_sum[ch];
-    g[k] += t / static_cast<double>(R);
+// g[k] += (sum of the entry's chunk sums, in chunk order) / R_k  (Algorithm 4's
+// walk estimate); one CTA per column of `list`
+static __global__ void __launch_bounds__(128) k_walk_finish(const int32_t *__restrict__ row_ptr,
+                                                            const int32_t *__restrict__ list,
+                                                            const int32_t *__restrict__ chunk0,
+                                                            const double *__restrict__ chunk_sum,
+                                                            const long long *__restrict__ walk_count,
+                                                            double *__restrict__ g) {
+    const int32_t s = list[blockIdx.x];
+    if (s < 0) return;
+    for (int32_t k = row_ptr[s] + static_cast<int32_t>(threadIdx.x); k < row_ptr[s + 1]; k += 128) {
+        const long long R = walk_count[k];
+        if (R <= 0) continue;
+        const int32_t c0 = chunk0[k], c1 = c0 + static_cast<int32_t>(walk_chunks(R));
+        double t = 0.0;
+        for (int32_t ch = c0; ch < c1; ++ch) t += chunk_sum[ch];
+        g[k] += t / static_cast<double>(R);
+    }
 }
 
-// Eq. 14's right side for one source: out[q] = the sum of the walk counts of
-// source q's entries (one warp per source; 0 for an empty slot)
+// Per source (one warp each; 0 for an empty slot): out[q] = Eq. 14's right side,
+// the sum of the walk counts of its entries; out[nsrc + q] = their walk steps
+// 2 R (tau_k - ell)
 static __global__ void k_walks_per_source(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ src,
                                           int32_t nsrc, const long long *__restrict__ walk_count,
-                                          long long *__restrict__ out) {
+                                          const int32_t *__restrict__ tau, int32_t ell, long long *__restrict__ out) {
     const int32_t q = blockIdx.x;
     const int lane = threadIdx.x & 31;
     if (q >= nsrc) return;
     const int32_t s = src[q];
-    long long acc = 0;
+    long long acc = 0, steps = 0;
     if (s >= 0)
-        for (int32_t k = row_ptr[s] + lane; k < row_ptr[s + 1]; k += 32) acc += walk_count[k];
+        for (int32_t k = row_ptr[s] + lane; k < row_ptr[s + 1]; k += 32) {
+            const long long R = walk_count[k];
+            const int32_t L = tau[k] - ell;
+            acc += R;
+            if (R > 0 && L > 0) steps += 2ll * R * static_cast<long long>(L);
+        }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) out[q] = acc;
+    for (int o = 16; o > 0; o >>= 1) {
+        acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        steps += __shfl_xor_sync(0xffffffffu, steps, o);
+    }
+    if (lane == 0) {
+        out[q] = acc;
+        out[nsrc + q] = steps;
+    }
 }
 
 // tau[k] = min(tau[k], cap) over the rows of the listed nodes (entries < 0
@@ -803,19 +894,6 @@ static __global__ void k_cap_rows(const int32_t *__restrict__ row_ptr, const int
     if (v < 0) return;
     for (int32_t k = row_ptr[v] + static_cast<int32_t>(threadIdx.x); k < row_ptr[v + 1]; k += blockDim.x)
         tau[k] = min(tau[k], cap);
-}
-
-// out[e] = R of planned entry e; out[nentries + e] = its walk steps 2 R (tau_k - tt)
-static __global__ void k_pack_counts(const int32_t *__restrict__ entry_k, int32_t nentries,
-                                     const long long *__restrict__ walk_count, const int32_t *__restrict__ tau,
-                                     int32_t tt, long long *__restrict__ out) {
-    const int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nentries) return;
-    const int32_t k = entry_k[e];
-    const long long R = walk_count[k];
-    const int32_t L = tau[k] - tt;
-    out[e] = R;
-    out[nentries + e] = (R > 0 && L > 0) ? 2ll * R * static_cast<long long>(L) : 0ll;
 }
 
 }  // namespace sc
