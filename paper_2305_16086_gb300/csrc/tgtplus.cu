@@ -11,6 +11,7 @@ template <typename T, int B>
 static void chi_check_t(sc_graph *g, const void *x, int slices, const int32_t *src, int nsrc, int max_deg,
                         const int32_t *tau, int ell, int gamma, double eps, double log2md, bool full_scan,
                         cudaStream_t s) {
+    gamma = std::min(gamma, g->n);  // a list holds the graph's nodes at most
     const int ncols = slices * B;
     double *pmin = g->tp_pmin.get(), *pmax = g->tp_pmax.get();
     long long *pvol = g->tp_pvol.get();
