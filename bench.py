@@ -71,9 +71,9 @@ KERNEL_SOURCES = ["paper_2305_16086_gb300/csrc/propagate.cuh", "paper_2305_16086
 # kernel classes the library times separately (SC_KC_* order) and their kernels
 KERNEL_CLASSES = {"dense_hop": "k_spmm_hop", "mask_hop": "k_front_scatter + k_front2, or k_mask_scatter + k_hop2_mask", "sparse_hop": "k_front3",
                   "ball_hop": "k_ball_rows + k_ball", "last_hop": "k_last_hop",
-                  "switch_test": "k_chi_tiles + k_chi_thresh + k_chi_select + k_chi_source + k_chi_entries "
-                                 "(+ the counts' copy and the host's wait)",
-                  "walks": "k_pack_counts + k_walk_chunks + k_walk_finish (+ the host's plan)"}
+                  "switch_test": "k_chi_tiles + k_chi_column + k_chi_entries "
+                                 "(+ the sums' copy and the host's wait)",
+                  "walks": "k_walk_plan + k_walk_chunks + k_walk_finish"}
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "spmm_hop_ba200k_traffic.json")
 
 

@@ -211,7 +211,7 @@ struct sc_graph {
     sc::DevBuf<int64_t> ws_entries;
     sc::DevBuf<double> ws_pre, ws_s, ws_b, ws_sub_s, ws_sub_b;
     // TGT+ work buffers: CalChi partial and per-column statistics, walk counts
-    sc::DevBuf<double> tp_pval, tp_pmin, tp_pmax, tp_cval, tp_cmin, tp_cmax, tp_cthr;
+    sc::DevBuf<double> tp_pval, tp_pmin, tp_pmax, tp_cval, tp_cmin, tp_cmax;
     sc::DevBuf<int32_t> tp_pid, tp_cid;
     sc::DevBuf<long long> tp_pvol, tp_cvol, tp_walks, tp_counters;
     sc::DevBuf<int32_t> tp_src_chunks, tp_chunk0;  // per column, per CSR entry: chunks of walks, the first one

@@ -15,28 +15,6 @@ static void chi_check_t(sc_graph *g, const void *x, int slices, const int32_t *s
     const int ncols = slices * B;
     double *pmin = g->tp_pmin.get(), *pmax = g->tp_pmax.get();
     long long *pvol = g->tp_pvol.get();
-    if (full_scan) {
-        // every row of a column through a sorted list per 64-row tile, lists merged per column
-        const int nct = ceil_div(g->n, kChiRowsPerCta);
-        k_chi_scan<T, B><<<dim3(nct, slices), kChiScanThreads, 0, s>>>(
-            g->row_ptr.get(), static_cast<const T *>(x), g->n, g->tp_pval.get(), g->tp_pid.get(), pmin, pmax, pvol);
-        k_chi_merge<B><<<ncols, kChiScanThreads, 0, s>>>(nct, ncols, g->tp_pval.get(), g->tp_pid.get(), pmin, pmax,
-                                                            pvol, g->tp_cval.get(), g->tp_cid.get(), g->tp_cmin.get(),
-                                                            g->tp_cmax.get(), g->tp_cvol.get());
-    } else {
-        // tile maxima, the threshold per column, then the candidates at or above it
-        using V = typename AccOf<T>::type;
-        const int ntiles = ceil_div(g->n, kTileRows);
-        V *tmax = reinterpret_cast<V *>(pmax), *tmin = reinterpret_cast<V *>(pmin);  // room for doubles
-        k_chi_tiles<T, B><<<dim3(ntiles, slices), kChiScanThreads, 0, s>>>(g->row_ptr.get(),
-                                                                          static_cast<const T *>(x), g->n, tmax,
-                                                                          tmin, pvol);
-        k_chi_thresh<V, B><<<ncols, kChiScanThreads, 0, s>>>(ntiles, ncols, gamma, tmax, tmin, pvol, g->tp_cthr.get(),
-                                                                g->tp_cmin.get(), g->tp_cmax.get(), g->tp_cvol.get());
-        k_chi_select<T, B><<<ncols, kChiScanThreads, 0, s>>>(g->n, ntiles, ncols, gamma, static_cast<const T *>(x),
-                                                                tmax, tmin, g->tp_cthr.get(), g->tp_cval.get(),
-                                                                g->tp_cid.get());
-    }
     ChiArgs a{};
     a.row_ptr = g->row_ptr.get();
     a.col = g->col_idx.get();
@@ -56,7 +34,27 @@ static void chi_check_t(sc_graph *g, const void *x, int slices, const int32_t *s
     a.rhs = g->tp_counters.get();
     a.cvol = g->tp_cvol.get();
     a.src_chunks = g->tp_src_chunks.get();
-    k_chi_source<T, B><<<nsrc, 32, 0, s>>>(static_cast<const T *>(x), a, g->tp_srcstat.get());
+    if (full_scan) {
+        // every row of a column through a sorted list per 64-row tile, lists merged per column
+        const int nct = ceil_div(g->n, kChiRowsPerCta);
+        k_chi_scan<T, B><<<dim3(nct, slices), kChiScanThreads, 0, s>>>(
+            g->row_ptr.get(), static_cast<const T *>(x), g->n, g->tp_pval.get(), g->tp_pid.get(), pmin, pmax, pvol);
+        k_chi_merge<B><<<ncols, kChiScanThreads, 0, s>>>(nct, ncols, g->tp_pval.get(), g->tp_pid.get(), pmin, pmax,
+                                                            pvol, g->tp_cval.get(), g->tp_cid.get(), g->tp_cmin.get(),
+                                                            g->tp_cmax.get(), g->tp_cvol.get());
+        k_chi_source<T, B><<<nsrc, kChiScanThreads, 0, s>>>(static_cast<const T *>(x), a, g->tp_srcstat.get());
+    } else {
+        // tile maxima, then per column the threshold and the candidates at or above it
+        using V = typename AccOf<T>::type;
+        const int ntiles = ceil_div(g->n, kTileRows);
+        V *tmax = reinterpret_cast<V *>(pmax), *tmin = reinterpret_cast<V *>(pmin);  // room for doubles
+        k_chi_tiles<T, B><<<dim3(ntiles, slices), kChiScanThreads, 0, s>>>(g->row_ptr.get(),
+                                                                          static_cast<const T *>(x), g->n, tmax,
+                                                                          tmin, pvol);
+        k_chi_column<T, B><<<nsrc, kChiScanThreads, 0, s>>>(ntiles, static_cast<const T *>(x), a, tmax, tmin, pvol,
+                                                               g->tp_cmin.get(), g->tp_cmax.get(), g->tp_cvol.get(),
+                                                               g->tp_srcstat.get());
+    }
     const int nw = 256 / 32;
     dim3 grid(nsrc, std::min(ceil_div(std::max(max_deg, 1), nw * kChiEntries), 65535));
     k_chi_entries<T, B><<<grid, 256, 0, s>>>(static_cast<const T *>(x), a, g->tp_srcstat.get());
@@ -109,7 +107,6 @@ void tgtplus_reserve(sc_graph *g, int slices, int B) {
     g->tp_cid.reserve(cols * kGammaMax);
     g->tp_cmin.reserve(cols);
     g->tp_cmax.reserve(cols);
-    g->tp_cthr.reserve(cols);
     g->tp_cvol.reserve(cols);
     g->tp_srcstat.reserve(3 * cols);
     g->tp_src_rhs.reserve(2 * cols);

@@ -210,11 +210,11 @@ __global__ void __launch_bounds__(kChiScanThreads)
 // largest of its tile maxima (tiles of kTileRows rows). The gamma tiles with
 // the largest maxima hold gamma entries >= thr, so the gamma-th largest entry
 // is >= thr, and every entry of the top-gamma list lies in a tile whose
-// maximum reaches thr. Three launches: tile maxima, minima and volumes
-// (k_chi_tiles); per column thr, min, max and volume (k_chi_thresh); per
-// column the entries >= thr of the tiles reaching it, and the top-gamma list
-// among them in the total order (k_chi_select). thr = 0 (fewer than gamma
-// tiles hold a positive entry) takes the positive entries of those tiles and
+// maximum reaches thr. Two launches: tile maxima, minima and volumes
+// (k_chi_tiles); per column thr, min, max and volume, the entries >= thr of the
+// tiles reaching it, and the top-gamma list among them in the total order
+// (k_chi_column). thr = 0 (fewer than gamma tiles hold a positive entry) takes
+// the positive entries of those tiles and
 // the gamma smallest-id zero rows (the ties at 0 go to smaller ids). A column
 // with more than kCandMax candidates (many ties at thr) is scanned in full.
 // The first gamma entries of each list equal the full scan's; entries past
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kChiScanThreads)
 // blocks): widening is exact and keeps the order, so every comparison falls out
 // as in double, and a comparison in double takes a warp 16 cycles of an SM's FP64
 // pipe here. A test of 192 columns of a 40,000-node Barabasi-Albert graph:
-// 137 us with the statistics in double, 89 us so.
+// 137 us with the statistics in double, 89 us so (62 with k_chi_column).
 // ---------------------------------------------------------------------------
 constexpr int kTileRows = 256;
 constexpr int kCandMax = 2048;
@@ -351,80 +351,184 @@ __global__ void __launch_bounds__(kChiScanThreads)
     }
 }
 
-// per column q = slice * B + b: thr, min, max and volume. One CTA per
-// column; thread t takes tiles t, t + 128, ... and keeps their largest
-// maximum. thr = the gamma-th largest of those 128 maxima (0 if fewer than
-// gamma are positive): they are maxima of distinct tiles, so at least gamma
-// tiles reach thr, every top-gamma entry is >= thr, and thr is at most the
-// gamma-th largest tile maximum (a few more candidate tiles than that, no
-// merge of sorted lists).
-template <typename V, int B>
-__global__ void __launch_bounds__(kChiScanThreads)
-    k_chi_thresh(int ntiles, int ncols, int gamma, const V *__restrict__ tmax, const V *__restrict__ tmin,
-                 const long long *__restrict__ tvol, double *__restrict__ cthr, double *__restrict__ cmin,
-                 double *__restrict__ cmax, long long *__restrict__ cvol) {
-    const int q = blockIdx.x;
-    if (q >= ncols) return;
-    const int slice = q / B, c = q % B, t = threadIdx.x;
-    constexpr int NT = kChiScanThreads;
-    __shared__ V smax[NT], smin[NT];
-    __shared__ long long svol[NT];
-    V vmax = V(-INFINITY), vmin = V(INFINITY);
-    long long vol = 0;
-    for (int p = t; p < ntiles; p += NT) {
-        const int64_t o = (static_cast<int64_t>(slice) * ntiles + p) * B + c;
-        vmax = max(vmax, tmax[o]);
-        vmin = min(vmin, tmin[o]);
-        vol += tvol[o];
+__device__ __forceinline__ bool has_edge(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
+                                         int32_t a, int32_t b) {
+    int32_t lo = row_ptr[a], hi = row_ptr[a + 1];
+    while (lo < hi) {
+        const int32_t mid = lo + ((hi - lo) >> 1);
+        const int32_t c = col[mid];
+        if (c == b) return true;
+        if (c < b) lo = mid + 1;
+        else hi = mid;
     }
-    smax[t] = vmax;
-    smin[t] = vmin;
-    svol[t] = vol;
-    __syncthreads();
-    // rank of each thread's maximum among the 128 (ties by thread index); rank gamma - 1 is thr
-    int rank = 0;
-    for (int u = 0; u < NT; ++u) rank += (smax[u] > vmax || (smax[u] == vmax && u < t)) ? 1 : 0;
-    if (gamma > 0 && rank == gamma - 1) cthr[q] = vmax > V(0) ? static_cast<double>(vmax) : 0.0;
-    if (rank == 0) cmax[q] = static_cast<double>(vmax);
-    __syncthreads();
-    for (int half = NT / 2; half > 0; half >>= 1) {
-        if (t < half) {
-            smin[t] = min(smin[t], smin[t + half]);
-            svol[t] += svol[t + half];
-        }
-        __syncthreads();
-    }
-    if (t == 0) {
-        cmin[q] = static_cast<double>(smin[0]);
-        cvol[q] = svol[0];
-        if (gamma > NT || gamma <= 0) cthr[q] = 0.0;  // (gamma <= kGammaMax < NT on the product path)
-    }
+    return false;
 }
 
-// per column: the candidates (entries >= thr in the tiles whose maximum
-// reaches thr; for thr = 0 the positive entries of the tiles holding one, and
-// the gamma smallest-id zero rows), then the top-kGammaMax list among them.
+struct ChiArgs {
+    const int32_t *row_ptr, *col, *src, *tau;
+    int32_t n, nsrc, ell, gamma;
+    const double *cval, *cmin, *cmax;
+    const int32_t *cid;
+    double eps, log_2m_delta;
+    long long *walk_count;   // per CSR entry (0 = no walks)
+    long long *rhs;          // [0] sum of the launch's walk counts (Eq. 14 right side), [1] left side, [2] walk steps
+    const long long *cvol;   // per column: frontier volume
+    int32_t *src_chunks;     // per column: chunks of kWalkChunk walk pairs of its entries
+};
+
+constexpr int kWalkChunk = 128;  // walk pairs per warp-sized chunk
+
+__host__ __device__ __forceinline__ long long walk_chunks(long long pairs) {
+    return pairs > 0 ? (pairs + kWalkChunk - 1) / kWalkChunk : 0;
+}
+
+// Source s of column q, by a CTA of kChiScanThreads threads: rho_hat (Alg. 3) and
+// min / max of p over N(s), into stat[3 q .. 3 q + 2]; cv / ci: the column's
+// top-gamma list. Also counts the column's frontier volume into Eq. 14's left side.
+template <typename T, int B, typename CV>
+__device__ __forceinline__ void source_stats(const T *__restrict__ x, const ChiArgs &a, int32_t q, int32_t s,
+                                             const CV *cv, const int32_t *ci, long long volume,
+                                             double *__restrict__ stat) {
+    using V = typename AccOf<T>::type;
+    constexpr int NT = kChiScanThreads, NW = NT / 32;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const T *xs = x + static_cast<int64_t>(q / B) * a.n * B + (q % B);
+    const int g = a.gamma;
+    // rho_hat = max(max over edges inside C of p(c_a) + p(c_b), p(c_1) + p(c_gamma))
+    double best = -INFINITY;
+    for (int e = t; e < g * g; e += NT) {
+        const int u = e / g, v = e % g;
+        if (u < v && has_edge(a.row_ptr, a.col, ci[u], ci[v]))
+            best = fmax(best, __dadd_rn(static_cast<double>(cv[u]), static_cast<double>(cv[v])));
+    }
+    V nmin = V(INFINITY), nmax = V(-INFINITY);
+    for (int32_t k = a.row_ptr[s] + t; k < a.row_ptr[s + 1]; k += NT) {
+        const V v = to_acc(xs[static_cast<int64_t>(a.col[k]) * B]);
+        nmin = min(nmin, v);
+        nmax = max(nmax, v);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
+        nmin = min(nmin, __shfl_xor_sync(0xffffffffu, nmin, o));
+        nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
+    }
+    __shared__ double wbest[NW];
+    __shared__ V wmin[NW], wmax[NW];
+    if (lane == 0) {
+        wbest[warp] = best;
+        wmin[warp] = nmin;
+        wmax[warp] = nmax;
+    }
+    __syncthreads();
+    if (t != 0) return;
+    for (int w = 1; w < NW; ++w) {
+        best = fmax(best, wbest[w]);
+        nmin = min(nmin, wmin[w]);
+        nmax = max(nmax, wmax[w]);
+    }
+    stat[3 * q] = g > 0 ? fmax(best, __dadd_rn(static_cast<double>(cv[0]), static_cast<double>(cv[g - 1]))) : 0.0;
+    stat[3 * q + 1] = static_cast<double>(nmin);
+    stat[3 * q + 2] = static_cast<double>(nmax);
+    atomicAdd(reinterpret_cast<unsigned long long *>(a.rhs + 1), static_cast<unsigned long long>(volume));
+}
+
+// The full scan's last step: one CTA per column of the launch
 template <typename T, int B>
 __global__ void __launch_bounds__(kChiScanThreads)
-    k_chi_select(int32_t n, int ntiles, int ncols, int gamma, const T *__restrict__ x,
+    k_chi_source(const T *__restrict__ x, const ChiArgs a, double *__restrict__ stat) {
+    const int32_t q = blockIdx.x;
+    const int32_t s = a.src[q];
+    if (threadIdx.x == 0) a.src_chunks[q] = 0;
+    if (s < 0) return;
+    source_stats<T, B>(x, a, q, s, a.cval + static_cast<int64_t>(q) * kGammaMax,
+                       a.cid + static_cast<int64_t>(q) * kGammaMax, a.cvol[q], stat);
+}
+
+// A column from its tiles' statistics to its source's, one CTA per column of the
+// launch. (1) min, max, volume and thr: thread t takes tiles t, t + 128, ... and
+// keeps their largest maximum; thr = the gamma-th largest of those 128 maxima (0
+// if fewer than gamma are positive): they are maxima of distinct tiles, so at
+// least gamma tiles reach thr, every top-gamma entry is >= thr, and thr is at
+// most the gamma-th largest tile maximum (a few more candidate tiles than that,
+// no merge of sorted lists). (2) The candidates (entries >= thr in the tiles whose
+// maximum reaches thr; for thr = 0 the positive entries of the tiles holding one,
+// and the gamma smallest-id zero rows), then the top-kGammaMax list among them: up
+// to kRankMax candidates by counting each one's betters (a thread per candidate,
+// broadcast reads), more by sorted lists per thread and a tree of merges, whose
+// chain of dependent shared-memory reads is the longer one below that. (3) The
+// source's statistics. Latency bound: a CTA's dependent steps, not its bytes; as
+// three kernels, the last with a warp per source and all lists merged, a test of
+// 192 columns of a 40,000-node Barabasi-Albert graph took 81 us, so 62.
+constexpr int kRankMax = 2 * kChiScanThreads;
+
+template <typename T, int B>
+__global__ void __launch_bounds__(kChiScanThreads)
+    k_chi_column(int ntiles, const T *__restrict__ x, const ChiArgs a,
                  const typename AccOf<T>::type *__restrict__ tmax, const typename AccOf<T>::type *__restrict__ tmin,
-                 const double *__restrict__ cthr, double *__restrict__ cval,
-                 int32_t *__restrict__ cid) {
+                 const long long *__restrict__ tvol, double *__restrict__ cmin, double *__restrict__ cmax,
+                 long long *__restrict__ cvol, double *__restrict__ stat) {
     using V = typename AccOf<T>::type;
-    const int q = blockIdx.x;
-    if (q >= ncols || gamma <= 0) return;
+    const int q = blockIdx.x, n = a.n, gamma = a.gamma;
+    const int32_t s = a.src[q];
     const int slice = q / B, c = q % B, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (t == 0) a.src_chunks[q] = 0;
+    if (s < 0) return;
     constexpr int NT = kChiScanThreads, NW = kChiScanThreads / 32;
     const T *xs = x + static_cast<int64_t>(slice) * n * B + c;
-    const V thr = static_cast<V>(cthr[q]);  // exact: a tile maximum or 0
-    const bool zero_thr = !(thr > V(0));
     __shared__ V cand_v[kCandMax];
     __shared__ int32_t cand_i[kCandMax];
     __shared__ int ncand;
+    __shared__ V sthr, top_v[kGammaMax];
+    __shared__ int32_t top_i[kGammaMax];
+    __shared__ long long volume;
     __shared__ V sv[kGammaMax * NT];
     __shared__ int32_t si[kGammaMax * NT];
-    if (t == 0) ncand = 0;
-    __syncthreads();
+    // ---- thr, min, max, volume ----
+    {
+        V *smax = sv, *smin = sv + NT;
+        long long *svol = reinterpret_cast<long long *>(si);
+        static_assert(sizeof(si) >= NT * sizeof(long long), "the lists' ids hold the threads' volumes");
+        V vmax = V(-INFINITY), vmin = V(INFINITY);
+        long long vol = 0;
+        for (int p = t; p < ntiles; p += NT) {
+            const int64_t o = (static_cast<int64_t>(slice) * ntiles + p) * B + c;
+            vmax = max(vmax, tmax[o]);
+            vmin = min(vmin, tmin[o]);
+            vol += tvol[o];
+        }
+        smax[t] = vmax;
+        smin[t] = vmin;
+        svol[t] = vol;
+        if (t == 0) {
+            ncand = 0;
+            sthr = V(0);
+        }
+        __syncthreads();
+        // rank of each thread's maximum among the 128 (ties by thread index); rank gamma - 1 is thr
+        int rank = 0;
+        for (int u = 0; u < NT; ++u) rank += (smax[u] > vmax || (smax[u] == vmax && u < t)) ? 1 : 0;
+        if (rank == gamma - 1 && vmax > V(0)) sthr = vmax;  // (gamma <= kGammaMax < NT)
+        if (rank == 0) cmax[q] = static_cast<double>(vmax);
+        for (int half = NT / 2; half > 0; half >>= 1) {
+            if (t < half) {
+                smin[t] = min(smin[t], smin[t + half]);
+                svol[t] += svol[t + half];
+            }
+            __syncthreads();
+        }
+        if (t == 0) {
+            cmin[q] = static_cast<double>(smin[0]);
+            cvol[q] = volume = svol[0];
+        }
+        __syncthreads();
+    }
+    if (gamma <= 0) {  // no list: Eq. 15
+        source_stats<T, B>(x, a, q, s, top_v, top_i, volume, stat);
+        return;
+    }
+    const V thr = sthr;
+    const bool zero_thr = !(thr > V(0));
     // candidates: each warp tests 32 tile maxima at once, then takes the tiles that reach thr
     // one by one, 32 rows at a time
     for (int pb = warp * 32; pb < ntiles; pb += NW * 32) {
@@ -491,121 +595,64 @@ __global__ void __launch_bounds__(kChiScanThreads)
         }
     }
     __syncthreads();
-    V *val = sv + t;
-    int32_t *id = si + t;
-    for (int s = 0; s < kGammaMax; ++s) {
-        val[s * NT] = V(-INFINITY);
-        id[s * NT] = INT32_MAX;
-    }
-    V bv[kGammaMax];
-    int32_t bi[kGammaMax];
-#pragma unroll
-    for (int s = 1; s < kGammaMax; ++s) {
-        bv[s] = V(-INFINITY);
-        bi[s] = INT32_MAX;
-    }
     const int count = ncand;
-    if (count <= kCandMax) {
+    if (count <= kRankMax) {
+        if (t < kGammaMax) {
+            top_v[t] = V(-INFINITY);
+            top_i[t] = INT32_MAX;
+        }
+        __syncthreads();
         for (int e = t; e < count; e += NT) {
-            bv[0] = cand_v[e];
-            bi[0] = cand_i[e];
-            merge_sorted(val, id, NT, bv, bi, 1);
+            const V v = cand_v[e];
+            const int32_t i = cand_i[e];
+            int rank = 0;
+#pragma unroll 4
+            for (int u = 0; u < count; ++u) rank += u != e && better(cand_v[u], cand_i[u], v, i) ? 1 : 0;
+            if (rank < kGammaMax) {
+                top_v[rank] = v;
+                top_i[rank] = i;
+            }
         }
     } else {
-        // too many ties at thr for the buffer: every row of the column
-        for (int32_t r = t; r < n; r += NT) {
-            bv[0] = to_acc(xs[static_cast<int64_t>(r) * B]);
-            bi[0] = r;
-            merge_sorted(val, id, NT, bv, bi, 1);
+        V *val = sv + t;
+        int32_t *id = si + t;
+        for (int r = 0; r < kGammaMax; ++r) {
+            val[r * NT] = V(-INFINITY);
+            id[r * NT] = INT32_MAX;
+        }
+        V bv[kGammaMax];
+        int32_t bi[kGammaMax];
+#pragma unroll
+        for (int r = 1; r < kGammaMax; ++r) {
+            bv[r] = V(-INFINITY);
+            bi[r] = INT32_MAX;
+        }
+        if (count <= kCandMax) {
+            for (int e = t; e < count; e += NT) {
+                bv[0] = cand_v[e];
+                bi[0] = cand_i[e];
+                merge_sorted(val, id, NT, bv, bi, 1);
+            }
+        } else {
+            // too many ties at thr for the buffer: every row of the column
+            for (int32_t r = t; r < n; r += NT) {
+                bv[0] = to_acc(xs[static_cast<int64_t>(r) * B]);
+                bi[0] = r;
+                merge_sorted(val, id, NT, bv, bi, 1);
+            }
+        }
+        __syncthreads();
+        for (int half = NT / 2; half > 0; half >>= 1) {
+            if (t < half) merge_sorted(val, id, NT, sv + t + half, si + t + half, NT);
+            __syncthreads();
+        }
+        if (t < kGammaMax) {
+            top_v[t] = sv[t * NT];
+            top_i[t] = si[t * NT];
         }
     }
     __syncthreads();
-    for (int half = NT / 2; half > 0; half >>= 1) {
-        if (t < half) merge_sorted(val, id, NT, sv + t + half, si + t + half, NT);
-        __syncthreads();
-    }
-    if (t == 0)
-        for (int s = 0; s < kGammaMax; ++s) {
-            cval[static_cast<int64_t>(q) * kGammaMax + s] = static_cast<double>(sv[s * NT]);
-            cid[static_cast<int64_t>(q) * kGammaMax + s] = si[s * NT];
-        }
-}
-
-__device__ __forceinline__ bool has_edge(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                                         int32_t a, int32_t b) {
-    int32_t lo = row_ptr[a], hi = row_ptr[a + 1];
-    while (lo < hi) {
-        const int32_t mid = lo + ((hi - lo) >> 1);
-        const int32_t c = col[mid];
-        if (c == b) return true;
-        if (c < b) lo = mid + 1;
-        else hi = mid;
-    }
-    return false;
-}
-
-struct ChiArgs {
-    const int32_t *row_ptr, *col, *src, *tau;
-    int32_t n, nsrc, ell, gamma;
-    const double *cval, *cmin, *cmax;
-    const int32_t *cid;
-    double eps, log_2m_delta;
-    long long *walk_count;   // per CSR entry (0 = no walks)
-    long long *rhs;          // [0] sum of the launch's walk counts (Eq. 14 right side), [1] left side, [2] walk steps
-    const long long *cvol;   // per column: frontier volume
-    int32_t *src_chunks;     // per column: chunks of kWalkChunk walk pairs of its entries
-};
-
-constexpr int kWalkChunk = 128;  // walk pairs per warp-sized chunk
-
-__host__ __device__ __forceinline__ long long walk_chunks(long long pairs) {
-    return pairs > 0 ? (pairs + kWalkChunk - 1) / kWalkChunk : 0;
-}
-
-// Per source (one warp): rho_hat (Alg. 3) and min / max of p over N(i),
-// into stat[3 q .. 3 q + 2].
-template <typename T, int B>
-__global__ void k_chi_source(const T *__restrict__ x, const ChiArgs a, double *__restrict__ stat) {
-    const int32_t q = blockIdx.x;
-    const int lane = threadIdx.x & 31;
-    if (q >= a.nsrc) return;
-    const int32_t s = a.src[q];
-    if (lane == 0) {
-        a.src_chunks[q] = 0;
-        if (s >= 0) atomicAdd(reinterpret_cast<unsigned long long *>(a.rhs + 1), static_cast<unsigned long long>(a.cvol[q]));
-    }
-    if (s < 0) return;
-    const T *xs = x + static_cast<int64_t>(q / B) * a.n * B + (q % B);
-    using V = typename AccOf<T>::type;
-    auto px = [&](int32_t v) { return to_acc(xs[static_cast<int64_t>(v) * B]); };
-    const double *cv = a.cval + static_cast<int64_t>(q) * kGammaMax;
-    const int32_t *ci = a.cid + static_cast<int64_t>(q) * kGammaMax;
-    const int g = a.gamma;
-    // rho_hat = max(max over edges inside C of p(c_a) + p(c_b), p(c_1) + p(c_gamma))
-    double best = -INFINITY;
-    if (g > 0) {
-        for (int t = lane; t < g * g; t += 32) {
-            const int u = t / g, v = t % g;
-            if (u < v && has_edge(a.row_ptr, a.col, ci[u], ci[v])) best = fmax(best, __dadd_rn(cv[u], cv[v]));
-        }
-    }
-    V nmin = V(INFINITY), nmax = V(-INFINITY);
-    for (int32_t k = a.row_ptr[s] + lane; k < a.row_ptr[s + 1]; k += 32) {
-        const V v = px(a.col[k]);
-        nmin = min(nmin, v);
-        nmax = max(nmax, v);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
-        nmin = min(nmin, __shfl_xor_sync(0xffffffffu, nmin, o));
-        nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
-    }
-    if (lane == 0) {
-        stat[3 * q] = g > 0 ? fmax(best, __dadd_rn(cv[0], cv[g - 1])) : 0.0;
-        stat[3 * q + 1] = static_cast<double>(nmin);
-        stat[3 * q + 2] = static_cast<double>(nmax);
-    }
+    source_stats<T, B>(x, a, q, s, top_v, top_i, volume, stat);
 }
 
 // Per entry k = (i -> j) of source q = blockIdx.x, kChiEntries of them to a
