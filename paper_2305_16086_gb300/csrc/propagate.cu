@@ -1965,7 +1965,7 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
                          ((o.flags & SC_OPT_WINDOWS_FORCE) ||
                           2.0 * (Lmax / 2 + 2.0) * static_cast<double>(beta) + 128.0 < 0.5 * static_cast<double>(n));
     // graphs of small degree run resident (each source's ball in shared memory) as far as it
-    // fits: a 150 x 613 strip at 67 hops takes 9.0 ms a call, windowed 94 ms
+    // fits: a 150 x 613 strip at 67 hops takes 8.4 ms a call, windowed 94 ms
     const bool use_res = resident_allowed(o) && resident_degree_ok(g->max_degree) && Lmax > 0;
     g->res_width = g->max_degree <= 4 ? 4 : 8;
     // a bf16 run whose early hops are fp32 is tuned (and its buffers sized) in fp32

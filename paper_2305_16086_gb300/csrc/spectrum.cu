@@ -509,9 +509,10 @@ sc_status estimate_lambda_impl(sc_graph *g, const sc_lambda_opts *opts, sc_lambd
         // orthogonal to the basis; the sweep removes what rounding left, so the second one is
         // rarely needed. A step therefore makes one sweep, in six launches that sum their scalars
         // themselves, and records whether it was enough (with 14 launches and the second sweep asked
-        // for on the device at every step a call on 100,000 nodes of degree 20 took 39.1 ms, 31.8 so). A check that finds a step
-        // where it was not goes back to that step, and from there on every step asks on the device
-        // before it goes on (careful: the second sweep's launches return at once when not needed).
+        // for on the device at every step a call on 100,000 nodes of degree 20 took 39.1 ms, 31.8
+        // so). A check that finds a step where it was not goes back to that step, and from there on
+        // every step asks on the device before it goes on (careful: the second sweep's launches
+        // return at once when not needed).
         DevBuf<double> scal;
         DevBuf<int> skip;
         scal.reserve(2);  // a, |w|^2 after the first sweep (careful)
