@@ -411,7 +411,7 @@ typedef struct sc_report {
     double walk_ms;            /* TGT+: host time queueing walks plus walk_device_ms */
     int64_t source_hops;       /* sum over sources of hops traversed (the traversal's work) */
     int32_t extension_rounds;  /* learned policy: rerun rounds for edges that failed their bound */
-    int32_t windowed;          /* 1 if the blocks ran windowed or resident (SC_OPT_WINDOWS_*) */
+    int32_t windowed;          /* 1 if the blocks ran windowed or sources ran resident (SC_OPT_WINDOWS_*) */
     int64_t walk_steps;        /* TGT+: walk steps taken (both walks of every pair) */
     double walk_device_ms;     /* TGT+: device time of the walk launches (events) */
     /* with SC_OPT_TIME_KERNELS, per kernel class SC_KC_*: summed duration (events around
@@ -422,7 +422,8 @@ typedef struct sc_report {
     double kc_bytes[SC_KC_COUNT];
     int32_t uncertified;       /* 1 if the learned lengths were accepted by the tail estimate of
                                   sc_estimated_lengths (bipartite graph), not by a bound */
-    int32_t reserved_r;
+    int32_t resident_sources;  /* sources whose traversal ran resident, the others in blocks (a source
+                                  that runs again for a longer length counts again) */
 } sc_report;
 
 /*

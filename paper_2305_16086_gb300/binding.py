@@ -90,7 +90,7 @@ class Report(ctypes.Structure):
                 ("walk_steps", ctypes.c_int64), ("walk_device_ms", ctypes.c_double),
                 ("kc_ms", ctypes.c_double * 7), ("kc_launches", ctypes.c_int64 * 7),
                 ("kc_bytes", ctypes.c_double * 7), ("uncertified", ctypes.c_int32),
-                ("reserved_r", ctypes.c_int32)]
+                ("resident_sources", ctypes.c_int32)]
 
     def as_dict(self):
         d = {name: getattr(self, name) for name, _ in self._fields_}

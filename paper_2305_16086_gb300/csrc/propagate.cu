@@ -1047,6 +1047,7 @@ struct Run {
     bool full_hops = false;  // no sparse hops
     // statistics
     int64_t launches = 0, hops = 0, source_hops = 0, hop_launches = 0, walks = 0, graph_launches = 0, walk_steps = 0;
+    int64_t resident_sources = 0;
     // per kernel class (SC_KC_*): event pairs (index into the graph's pool) and algorithmic bytes
     std::vector<std::pair<int, int64_t>> timed;
     int64_t event_pairs = 0;
@@ -1696,6 +1697,7 @@ static std::vector<int32_t> resident_blocks(Run &R, const std::vector<int32_t> &
         R.source_hops += l;
         R.ell_min_src = std::min(R.ell_min_src, l);
         R.ell_max_src = std::max(R.ell_max_src, l);
+        if (l > 0) ++R.resident_sources;
     }
     return left;
 }
@@ -2280,8 +2282,9 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
         rep->walks = R.walks;
         rep->edges_extended = static_cast<int32_t>(extended);
         rep->extension_rounds = rounds;
-        rep->windowed = use_win || use_res ? 1 : 0;
+        rep->windowed = use_win || R.resident_sources > 0 ? 1 : 0;
         rep->uncertified = est_learned ? 1 : 0;
+        rep->resident_sources = static_cast<int32_t>(std::min<int64_t>(R.resident_sources, INT32_MAX));
         rep->tt_min = plus ? (R.tt_min == INT32_MAX ? 0 : R.tt_min) : 0;
         rep->tt_max = plus ? R.tt_max : 0;
         rep->switch_tests = R.switch_tests;
@@ -2647,8 +2650,11 @@ static void batch_impl(sc_graph *const *graphs, int32_t count, const sc_options 
     std::vector<int32_t> seg_start(count + 1);
     for (int32_t i = 0; i < count; ++i) seg_start[i] = static_cast<int32_t>(n_off[i]);
     seg_start[count] = N;
-    // per graph: source-hops, shortest and longest source run
-    std::vector<int64_t> g_hops(count, 0);
+    // per graph: source-hops, sources run resident, shortest and longest source run
+    std::vector<int64_t> g_hops(count, 0), g_resident(count, 0);
+    auto seg_at = [&](int32_t v) {
+        return static_cast<size_t>(std::upper_bound(seg_start.begin(), seg_start.end(), v) - seg_start.begin()) - 1;
+    };
     std::vector<int32_t> g_lmin(count, INT32_MAX), g_lmax(count, 0);
     auto book = [&](const std::vector<int32_t> &src) {
         int32_t i = 0;
@@ -2672,6 +2678,8 @@ static void batch_impl(sc_graph *const *graphs, int32_t count, const sc_options 
         }
         if (!res.empty()) {
             const std::vector<int32_t> left = resident_blocks(R, res, len, seg_start, seg_take, seg_bip);
+            for (int32_t v : res) g_resident[seg_at(v)] += len[v] + extra > 0 ? 1 : 0;
+            for (int32_t v : left) --g_resident[seg_at(v)];
             rest.insert(rest.end(), left.begin(), left.end());
         }
         run_blocks_win(R, rest, len, seg_start, beta, seg_bip);
@@ -2786,6 +2794,7 @@ static void batch_impl(sc_graph *const *graphs, int32_t count, const sc_options 
             rep->lambda_star = lam[i];
             rep->windowed = 1;
             rep->uncertified = learned && graphs[i]->bipartite ? 1 : 0;
+            rep->resident_sources = static_cast<int32_t>(std::min<int64_t>(g_resident[i], INT32_MAX));
             // batch totals
             rep->extension_rounds = rounds;
             rep->edges_extended = static_cast<int32_t>(std::min<int64_t>(extended, INT32_MAX));
