@@ -317,8 +317,8 @@ sc_status sc_series_meet(sc_graph *g, const int32_t *tau, double *s_out);
    Without either flag, a block width, a split or a slice count of its own, a TGT
    request on a graph of degree at most 8 runs resident instead: the nodes a few
    neighbouring sources reach (by hops, not by ids) are kept in shared memory and
-   one kernel runs all their hops; sources whose ball does not fit run windowed.
-   The values are the same again. */
+   one kernel runs all their hops; sources whose ball does not fit run in blocks,
+   windowed or not. The values are the same again. */
 #define SC_OPT_WINDOWS_OFF 8u
 #define SC_OPT_WINDOWS_FORCE 16u
 /* Unwindowed blocks compute hops 2 and 3 from the non-zero values of X_1 and

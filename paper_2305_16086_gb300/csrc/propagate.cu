@@ -1667,9 +1667,55 @@ static bool resident_allowed(const sc_options &o) {
            !(o.flags & (SC_OPT_WINDOWS_OFF | SC_OPT_WINDOWS_FORCE | SC_OPT_SPARSE_HOPS));
 }
 
-// the launch shape of the sources a resident run leaves over (balls past shared memory):
-// one row per warp in the widest block, without timing candidates for a few blocks
-static TuneResult leftover_shape(int prec) { return TuneResult{prec == SC_PREC_FP64 ? 64 : 128, 1, 0.0}; }
+// The sources a resident run leaves over (balls past shared memory) go to windowed blocks if the
+// windows pay (leftover_windows), else to the full ones with their sparse ends. On a graph whose
+// balls grow fast they are all of them, so that the full blocks' shape is timed as for any request
+// once they fill more than kUntimedBlocks of them (10 to 20 ms of a graph's first call). Few, or
+// windowed ones, take one row per warp in the widest block: the timed sample of 8 hops takes
+// narrower windows than the run has (a 300 x 301 lattice at 401 hops: 1.97 s a call in blocks of
+// 128, 2.37 in the 64 that the timing picks). Random 8-regular graphs at 7 hops, FP32: 30,000
+// nodes 21.1 ms a call in windows of the whole graph, 13.5 ms so; 100,000 nodes 214 and 114 ms.
+constexpr int64_t kUntimedBlocks = 4;
+static TuneResult untimed_shape(int prec) { return TuneResult{prec == SC_PREC_FP64 ? 64 : 128, 1, 0.0}; }
+
+// Whether windowed blocks serve left-over sources better: a windowed row costs 1.3 of a full block's
+// (its slices stream through HBM), so that the windows have to hold under 0.75 of the graph over the
+// hops on average (a 141 x 142 lattice with diagonals at 121 hops: 0.45, 64 ms against 129). On a
+// bipartite graph they compute half the rows: up to 0.9, or whatever they hold in FP64, which the
+// arithmetic bounds (random 4-regular, 20,000 nodes, 51 hops: 178 ms against 236), and when two full
+// blocks overflow the L2's share of a launch (100,000 nodes, FP32, 15 hops: 230 ms against 294;
+// 40,000 nodes, where they do not: 55 against 51).
+static bool leftover_windows(const sc_graph *g, int32_t beta, int32_t L, int B, size_t elem, bool fp64) {
+    double rows = 0.0;
+    for (int32_t l = 1; l <= L; ++l)
+        rows += std::min(static_cast<double>(g->n), 2.0 * window_reach(L, l) * static_cast<double>(beta) + B);
+    const double share = rows / (static_cast<double>(g->n) * std::max(L, 1));
+    if (!g->bipartite) return share < 0.75;
+    return share < 0.9 || fp64 ||
+           2.0 * static_cast<double>(g->n) * B * elem > 0.6 * static_cast<double>(g->l2_bytes);
+}
+
+// accumulators of their own for timed sample blocks while the graph's hold results
+struct ScratchAccumulators {
+    sc_graph *g;
+    DevBuf<double> a, b, c;
+    explicit ScratchAccumulators(sc_graph *gr) : g(gr) {
+        for (DevBuf<double> *d : {&a, &b, &c}) d->reserve(g->nnz);
+        swap();
+    }
+    ScratchAccumulators(const ScratchAccumulators &) = delete;
+    ~ScratchAccumulators() {
+        cudaStreamSynchronize(g->stream);  // the sample blocks end before their accumulators go
+        swap();
+    }
+    void swap() {
+        DevBuf<double> *mine[] = {&a, &b, &c}, *graphs[] = {&g->acc_g, &g->acc_t1, &g->acc_t2};
+        for (int q = 0; q < 3; ++q) {
+            std::swap(mine[q]->ptr, graphs[q]->ptr);
+            std::swap(mine[q]->count, graphs[q]->count);
+        }
+    }
+};
 
 // the resident traversal of `sources`; returns those left for the block kernels
 static std::vector<int32_t> resident_blocks(Run &R, const std::vector<int32_t> &sources,
@@ -1963,7 +2009,7 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     // the longest run of the first pass (a learned length's cap is reached only by extensions,
     // which rerun few sources; the windows and the launch shape are chosen for the first pass)
     const int32_t Lmax = (len.empty() ? 0 : *std::max_element(len.begin(), len.end())) + (record_after ? 2 : 0);
-    const bool use_win = !plus && o.rows_split != -1 && !(o.flags & SC_OPT_WINDOWS_OFF) &&
+    bool use_win = !plus && o.rows_split != -1 && !(o.flags & SC_OPT_WINDOWS_OFF) &&
                          ((o.flags & SC_OPT_WINDOWS_FORCE) ||
                           2.0 * (Lmax / 2 + 2.0) * static_cast<double>(beta) + 128.0 < 0.5 * static_cast<double>(n));
     // graphs of small degree run resident (each source's ball in shared memory) as far as it
@@ -1973,21 +2019,19 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     // a bf16 run whose early hops are fp32 is tuned (and its buffers sized) in fp32
     const int32_t h0 = bf16_first_hop(o);
     const int tune_prec = (o.precision == SC_PREC_BF16 && h0 > 1) ? SC_PREC_FP32 : o.precision;
-    std::vector<TuneResult> per_b;
-    const TuneResult tr = use_res ? leftover_shape(tune_prec)
-                                  : autotune(g, tune_prec, o.block_width, fixV, o.max_slices, Lmax,
-                                             GatherRec{rec.mode, nullptr, 0}, !use_win, s, &per_b);
     Run R;
     R.g = g;
     R.o = &o;
     R.s = s;
     R.prec = o.precision;
     R.h0 = h0;
-    R.B = tr.B;
-    R.vpl = tr.vpl;
     const size_t elem = alloc_elem(R.prec, R.h0);
-    R.slice_bytes = static_cast<size_t>(n) * R.B * elem;
-    R.slices = slices_for(g, R.B, elem, o.max_slices);
+    auto take_shape = [&](const TuneResult &t) {
+        R.B = t.B;
+        R.vpl = t.vpl;
+        R.slice_bytes = static_cast<size_t>(n) * R.B * elem;
+        R.slices = slices_for(g, R.B, elem, o.max_slices);
+    };
     R.plus = plus;
     R.time_kernels = time_kernels;
     R.gamma = gamma;
@@ -1995,28 +2039,36 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     R.log2md = std::log(2.0 * static_cast<double>(nnz / 2) / delta);
     R.extra = record_after ? 2 : 0;
     R.rec = rec;
-    if (per_b.size() > 1 && Lmax >= 2) {
-        // the block width from one real block of each (the request's lengths, kernels and records)
-        const long long key = (static_cast<long long>(tune_prec) << 56) ^ (static_cast<long long>(fixV + 1) << 52) ^
-                              (static_cast<long long>(o.max_slices & 0xfff) << 40) ^
-                              (static_cast<long long>(Lmax) << 16) ^ (static_cast<long long>(use_win) << 15) ^
-                              (static_cast<long long>(rec.mode) << 12) ^
-                              (static_cast<long long>((o.flags & SC_OPT_SPARSE_HOPS) != 0) << 11) ^
-                              (static_cast<long long>(o.ell_policy) << 8) ^ (static_cast<long long>(o.estimator) << 6) ^
-                              (static_cast<long long>(plus) << 5) ^ static_cast<long long>(std::min(h0, 31));
-        const TuneResult t2 = pick_block_width(R, per_b, len, Lmax, use_win, beta,
-                                               std::vector<char>{static_cast<char>(g->bipartite ? 1 : 0)}, key);
-        R.B = t2.B;
-        R.vpl = t2.vpl;
-        R.slice_bytes = static_cast<size_t>(n) * R.B * elem;
-        R.slices = slices_for(g, R.B, elem, o.max_slices);
+    // the launch shape by timing (cached per graph and request)
+    auto time_shape = [&] {
+        std::vector<TuneResult> per_b;
+        take_shape(autotune(g, tune_prec, o.block_width, fixV, o.max_slices, Lmax, GatherRec{rec.mode, nullptr, 0},
+                            !use_win, s, &per_b));
+        if (per_b.size() > 1 && Lmax >= 2) {
+            // the block width from one real block of each (the request's lengths, kernels and records)
+            const long long key = (static_cast<long long>(tune_prec) << 56) ^ (static_cast<long long>(fixV + 1) << 52) ^
+                                  (static_cast<long long>(o.max_slices & 0xfff) << 40) ^
+                                  (static_cast<long long>(Lmax) << 16) ^ (static_cast<long long>(use_win) << 15) ^
+                                  (static_cast<long long>(rec.mode) << 12) ^
+                                  (static_cast<long long>((o.flags & SC_OPT_SPARSE_HOPS) != 0) << 11) ^
+                                  (static_cast<long long>(o.ell_policy) << 8) ^
+                                  (static_cast<long long>(o.estimator) << 6) ^ (static_cast<long long>(plus) << 5) ^
+                                  static_cast<long long>(std::min(h0, 31));
+            take_shape(pick_block_width(R, per_b, len, Lmax, use_win, beta,
+                                        std::vector<char>{static_cast<char>(g->bipartite ? 1 : 0)}, key));
+        }
+    };
+    if (use_res) {
+        take_shape(untimed_shape(tune_prec));
+        use_win = use_win || leftover_windows(g, beta, Lmax, R.B, elem, o.precision == SC_PREC_FP64);
+    } else {
+        time_shape();
     }
     std::vector<int32_t> depth;
     if (learned_plus) {
         depth.assign(n, 0);
         R.depth = &depth;
     }
-    const int64_t nblocks_total = (static_cast<int64_t>(n) + R.B - 1) / R.B;
 
     if (!use_res) {
         g->xa.reserve(R.slices * R.slice_bytes);
@@ -2053,15 +2105,25 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     }
     const std::vector<int32_t> seg_whole{0, n};
     const std::vector<char> seg_bip{static_cast<char>(g->bipartite ? 1 : 0)};
+    bool timed_shape = !use_res;
     auto run = [&](const std::vector<int32_t> &src, const std::vector<int32_t> &l) {
+        std::vector<int32_t> left;
         if (use_res) {
-            const std::vector<int32_t> left = resident_blocks(R, src, l, seg_whole, std::vector<char>{1}, seg_bip);
-            if (!left.empty()) run_blocks_win(R, left, l, seg_whole, beta, seg_bip);
-        } else if (use_win) {
-            run_blocks_win(R, src, l, seg_whole, beta, seg_bip);
-        } else {
-            run_blocks(R, src, l);
+            left = resident_blocks(R, src, l, seg_whole, std::vector<char>{1}, seg_bip);
+            if (left.empty()) return;
+            if (!use_win && !timed_shape && static_cast<int64_t>(left.size()) > kUntimedBlocks * R.B) {
+                ScratchAccumulators scratch(g);  // the sources that ran have their sums in the graph's
+                time_shape();
+                timed_shape = true;
+            }
+            if (!use_win) {
+                g->xa.reserve(R.slices * R.slice_bytes);
+                g->xb.reserve(R.slices * R.slice_bytes);
+            }
         }
+        const std::vector<int32_t> &rest = use_res ? left : src;
+        if (use_win) run_blocks_win(R, rest, l, seg_whole, beta, seg_bip);
+        else run_blocks(R, rest, l);
     };
     DevBuf<int32_t> tau_saved;
     if (learned_plus) {
@@ -2266,7 +2328,7 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
         rep->block_width = R.B;
         rep->rows_split = R.vpl == 0 ? -1 : R.vpl;
         rep->slices = R.slices;
-        rep->blocks = nblocks_total;
+        rep->blocks = (static_cast<int64_t>(n) + R.B - 1) / R.B;
         rep->launches = R.launches;
         rep->hops = R.hops;
         rep->source_hops = R.source_hops;
@@ -2609,7 +2671,7 @@ static void batch_impl(sc_graph *const *graphs, int32_t count, const sc_options 
         else all_res = false;
     }
     U->res_width = res_deg <= 4 ? 4 : 8;
-    const TuneResult tr = all_res ? leftover_shape(tune_prec)
+    const TuneResult tr = all_res ? untimed_shape(tune_prec)
                                   : autotune(gb, tune_prec, o.block_width, fixV, o.max_slices, ell[big] + extra,
                                              GatherRec{0, nullptr, 0}, false, gb->stream);
     SC_CUDA(cudaStreamSynchronize(gb->stream));

@@ -61,3 +61,54 @@ def test_batch_reports_each_graph(cuda_lib):
         for G in Gs:
             G.close()
     assert [r["resident_sources"] for r in reps] == [gs[0].n, 0, gs[2].n, 0]
+
+
+def _regular(n, d, seed):
+    """A random graph of degree d (even) without short cycles to speak of: d / 2 random Hamiltonian cycles."""
+    rng = np.random.default_rng(seed)
+    p = [rng.permutation(n) for _ in range(d // 2)]
+    return gg.from_edges(n, np.concatenate(p), np.concatenate([np.roll(q, 1) for q in p]))
+
+
+def _regular_with_path(n, length, seed):
+    """A random graph of degree 8, one edge of it replaced by a long path."""
+    c = _regular(n, 8, seed)
+    e = c.edges()
+    ids = np.concatenate([e[0, :1], n + np.arange(length), e[0, 1:]])
+    return gg.from_edges(n + length, np.concatenate([e[1:, 0], ids[:-1]]), np.concatenate([e[1:, 1], ids[1:]]))
+
+
+@pytest.mark.parametrize("maker,ell,precision,estimator,share,windows", [
+    (lambda: _regular(9000, 8, 1), 7, "fp32", "plain", "none", False),   # balls of nearly the whole graph
+    (lambda: _regular(9000, 8, 1), 9, "bf16", "end_corrected", "none", False),
+    (lambda: _regular(18000, 8, 2), 7, "fp64", "plain", "none", False),  # sparse ends of a large graph's blocks
+    # the path's sources run resident, then the blocks' shape is timed
+    (lambda: _regular_with_path(9000, 900, 3), 9, "fp32", "end_corrected", "some", False),
+    (lambda: _kings(90, 91), 121, "fp32", "end_corrected", "some", True),  # windows of 0.6 of the graph
+])
+def test_left_over_sources_take_the_better_blocks(cuda_lib, maker, ell, precision, estimator, share, windows):
+    """Sources whose balls fit nowhere go to the blocks that a request without the
+    resident form would take (hops 1-2 from masks, the last hop on the gather's
+    rows), or to windows where they hold little of the graph, in a timed launch
+    shape; the sums of the sources that ran before the timing stay as they are."""
+    from paper_2305_16086_gb300 import binding
+
+    g = maker()
+    kw = dict(policy="fixed", ell_fixed=ell, precision=precision, estimator=estimator, bf16_from_hop=4)
+    with _graph(g) as G:
+        G.set_lambda(0.999, -0.999, 0.999)
+        s, b, rep = G.all_edges(**kw)
+        s0, b0, rep0 = G.all_edges(windows=False, **kw)
+        ent = np.random.default_rng(3).integers(0, g.nnz, 40)  # few enough to go untimed
+        q, rq = binding.some_edges(G, ent, **kw)
+    got = rep["resident_sources"]
+    assert (got == 0) if share == "none" else (0 < got < g.n)
+    assert rep["windowed"] == (1 if got or windows else 0)
+    kc = rep["kernel_classes"]
+    assert (kc["mask_hop"]["launches"] > 0) == (not windows)
+    assert (kc["last_hop"]["launches"] > 0) == (not windows)
+    if share == "none":
+        assert rq["kernel_classes"]["last_hop"]["launches"] > 0
+    assert np.array_equal(s, s0) and np.array_equal(q, s0[ent])
+    if b is not None:
+        assert np.array_equal(b, b0)
