@@ -222,7 +222,8 @@ struct sc_graph {
     sc::DevBuf<int32_t> tp_cap_list;   // the sources that switch at a test (per-source switch)
     // resident traversal (resident.cu): neighbour ids in rows of res_width, the
     // groups of sources per kind of segment (0: bipartite, 1: not), work lists
-    sc::DevBuf<int32_t> res_ell, res_len, res_list, res_over, res_count, res_single, res_order_dev[2];
+    sc::DevBuf<int32_t> res_ell, res_len, res_list, res_over, res_single, res_order_dev[2];
+    sc::DevBuf<unsigned long long> res_count;
     std::vector<int32_t> res_order[2];
     int res_order_width[2] = {0, 0};
     int res_width = 0;

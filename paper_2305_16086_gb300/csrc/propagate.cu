@@ -1685,11 +1685,15 @@ static TuneResult untimed_shape(int prec) { return TuneResult{prec == SC_PREC_FP
 // arithmetic bounds (random 4-regular, 20,000 nodes, 51 hops: 178 ms against 236), and when two full
 // blocks overflow the L2's share of a launch (100,000 nodes, FP32, 15 hops: 230 ms against 294;
 // 40,000 nodes, where they do not: 55 against 51).
-static bool leftover_windows(const sc_graph *g, int32_t beta, int32_t L, int B, size_t elem, bool fp64) {
+static double window_share(int32_t n, int32_t beta, int32_t L, int B) {  // of the rows, over the hops
     double rows = 0.0;
     for (int32_t l = 1; l <= L; ++l)
-        rows += std::min(static_cast<double>(g->n), 2.0 * window_reach(L, l) * static_cast<double>(beta) + B);
-    const double share = rows / (static_cast<double>(g->n) * std::max(L, 1));
+        rows += std::min(static_cast<double>(n), 2.0 * window_reach(L, l) * static_cast<double>(beta) + B);
+    return rows / (static_cast<double>(n) * std::max(L, 1));
+}
+
+static bool leftover_windows(const sc_graph *g, int32_t beta, int32_t L, int B, size_t elem, bool fp64) {
+    const double share = window_share(g->n, beta, L, B);
     if (!g->bipartite) return share < 0.75;
     return share < 0.9 || fp64 ||
            2.0 * static_cast<double>(g->n) * B * elem > 0.6 * static_cast<double>(g->l2_bytes);
@@ -1717,10 +1721,21 @@ struct ScratchAccumulators {
     }
 };
 
-// the resident traversal of `sources`; returns those left for the block kernels
+// A source's share of a block's time, estimated: 1.4 ps a row and hop and 0.2 an entry in FP32, 5 and
+// 1.85 in FP64 (blocks of small-degree graphs of 10,000 to 100,000 nodes, which fit L2); three hops of
+// a full block cost little. A bipartite graph's windowed row counts like a full one (half the rows, in
+// launches half as efficient).
+static double block_share_ns(const sc_graph *g, int32_t lo, int32_t hi, int32_t L, bool fp64, double share) {
+    const double rows = static_cast<double>(hi - lo), entries = g->h_row_ptr[hi] - g->h_row_ptr[lo];
+    return 1e-3 * share * (fp64 ? 5.0 * rows + 1.85 * entries : 1.4 * rows + 0.2 * entries) * std::max(L - 3, 1);
+}
+
+// the resident traversal of `sources`; returns those left for the block kernels, windowed
+// (bandwidth beta) or not (beta < 0)
 static std::vector<int32_t> resident_blocks(Run &R, const std::vector<int32_t> &sources,
                                             const std::vector<int32_t> &len, const std::vector<int32_t> &seg_start,
-                                            const std::vector<char> &seg_take, const std::vector<char> &seg_bip) {
+                                            const std::vector<char> &seg_take, const std::vector<char> &seg_bip,
+                                            int32_t beta) {
     sc_graph *g = R.g;
     // what a launch cannot do without: the graph, once
     const double bytes = 4.0 * g->nnz + 4.0 * (g->n + 1) + (R.prec == SC_PREC_FP64 ? 8.0 : 4.0) * g->n;
@@ -1730,6 +1745,11 @@ static std::vector<int32_t> resident_blocks(Run &R, const std::vector<int32_t> &
                        timer_close(R, t, SC_KC_DENSE_HOP, bytes, R.s);
                        ++R.hop_launches;
                        R.alg_bytes += bytes;
+                   },
+                   [&](int32_t v, int32_t L) {
+                       const auto hi = std::upper_bound(seg_start.begin(), seg_start.end(), v);
+                       const double share = beta < 0 ? 1.0 : window_share(*hi - *(hi - 1), beta, L, R.B);
+                       return block_share_ns(g, *(hi - 1), *hi, L, R.prec == SC_PREC_FP64, share);
                    }};
     ResidentStats st;
     std::vector<int32_t> left = run_resident(rr, sources, len, seg_start, seg_take, seg_bip, &st);
@@ -2109,7 +2129,7 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     auto run = [&](const std::vector<int32_t> &src, const std::vector<int32_t> &l) {
         std::vector<int32_t> left;
         if (use_res) {
-            left = resident_blocks(R, src, l, seg_whole, std::vector<char>{1}, seg_bip);
+            left = resident_blocks(R, src, l, seg_whole, std::vector<char>{1}, seg_bip, use_win ? beta : -1);
             if (left.empty()) return;
             if (!use_win && !timed_shape && static_cast<int64_t>(left.size()) > kUntimedBlocks * R.B) {
                 ScratchAccumulators scratch(g);  // the sources that ran have their sums in the graph's
@@ -2739,7 +2759,7 @@ static void batch_impl(sc_graph *const *graphs, int32_t count, const sc_options 
             (seg_take[i] ? res : rest).push_back(v);
         }
         if (!res.empty()) {
-            const std::vector<int32_t> left = resident_blocks(R, res, len, seg_start, seg_take, seg_bip);
+            const std::vector<int32_t> left = resident_blocks(R, res, len, seg_start, seg_take, seg_bip, beta);
             for (int32_t v : res) g_resident[seg_at(v)] += len[v] + extra > 0 ? 1 : 0;
             for (int32_t v : left) --g_resident[seg_at(v)];
             rest.insert(rest.end(), left.begin(), left.end());

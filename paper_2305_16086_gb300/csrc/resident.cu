@@ -44,6 +44,10 @@ constexpr int kResClasses = 4;      // shared-memory sizes tried in turn; the la
 constexpr int kResIdOrder = 4;      // hops per level from which the lists are kept in id order
 constexpr int kResSample = 128;     // groups whose ball is measured to choose the first class
 
+// what a measuring launch counts: the largest list, the groups that did not fit; of the others the
+// nodes, the rows of all hops and the levels
+enum ResCount { kResLargest, kResOver, kResNodes, kResRows, kResLevels, kResCounts };
+
 struct ResArgs {
     const int32_t *row_ptr;
     const int32_t *ell;      // n x W neighbour ids in CSR order, -1 past the degree
@@ -60,7 +64,7 @@ struct ResArgs {
     double *g, *t1, *t2;
     GatherRec rec;
     int32_t *over;           // [0]: groups that did not fit, [1 ..]: their ids
-    int32_t *count;          // nullable: measure only; [0] = largest list, [1] = groups that did not fit
+    unsigned long long *count;  // nullable: measure the balls only (ResCount)
     unsigned char *scratch;  // global-adjacency class: per CTA adjacency, 1/d, nodes, local id per node
     size_t scratch_cta;
 };
@@ -238,8 +242,20 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
         if (a.count || !fits) {
             if (tid == 0) {
                 if (a.count) {
-                    atomicMax(&a.count[0], max(n0, n1));
-                    if (!fits) atomicAdd(&a.count[1], 1);
+                    atomicMax(&a.count[kResLargest], static_cast<unsigned long long>(max(n0, n1)));
+                    if (!fits) {
+                        atomicAdd(&a.count[kResOver], 1ull);
+                    } else {
+                        unsigned long long rows = 0;
+                        for (int32_t h = 1; h <= Lg; ++h) {
+                            int32_t lim = min(min(h, Lg - h + 1), top);
+                            if (BIP) lim -= (lim ^ h) & 1;
+                            rows += lim >= 0 ? lvl[lim] : 0;
+                        }
+                        atomicAdd(&a.count[kResNodes], static_cast<unsigned long long>(n0 + n1));
+                        atomicAdd(&a.count[kResRows], rows);
+                        atomicAdd(&a.count[kResLevels], static_cast<unsigned long long>(top));
+                    }
                 } else {
                     a.over[1 + atomicAdd(&a.over[0], 1)] = gid;
                 }
@@ -554,6 +570,35 @@ static int32_t res_cap_of(int W, int cls, bool bip) {
     return bip ? res_capacity<Acc, 8, true, false>(cls) : res_capacity<Acc, 8, false, false>(cls);
 }
 
+// nodes the global-adjacency class holds
+template <typename Acc>
+static int32_t res_global_rows(int W) {
+    constexpr int c = kResClasses - 1;
+    return 2 * (W == 4 ? res_capacity<Acc, 4, true, true>(c) : res_capacity<Acc, 8, true, true>(c));
+}
+
+// The global-adjacency class runs a source and its ball alone on an SM, where a block shares each row
+// of ids among 32 to 128 sources, so it pays for long runs on balls that are small against the graph
+// and not for short ones on most of it: an SM's time for the measured sources, predicted from counts,
+// against the blocks' (ResidentRun::block_ns). Fitted on lattices, trees and random regular graphs of
+// 10,000 to 100,000 nodes at 15 to 201 hops: 3.5 ns a node and slot to build a ball (slots: the mean
+// of the degree and the width of a row of ids; in vain where it does not fit), 1 us a level, 0.4 ns a
+// row and hop at four slots and 0.6 at eight, 0.2 us a hop. Calls, FP32, blocks against this class:
+// random 4-regular bipartite of 20,000 nodes at 15 hops 12.8 and 22.6 ms, 51 hops 44 and 73, 201 hops
+// 175 and 149; 8-regular of 40,000 at 9 hops 37 and 83; renamed lattice of 40,000 at 201 hops 720 and
+// 170. Within kResGain the blocks are taken.
+constexpr double kResGain = 1.1;
+
+// h: the measured sources' counts, of ns sources of `hops` hops together and `blocks_ns` in blocks
+static bool global_class_pays(const unsigned long long *h, int32_t ns, double hops, double blocks_ns, int W,
+                              double degree, int32_t cap_rows, int sms) {
+    const double over = static_cast<double>(h[kResOver]), fit = (ns - over) / ns;
+    const double build = 3.5 * 0.5 * (degree + W) * (static_cast<double>(h[kResNodes]) + over * cap_rows);
+    const double run = (0.2 + 0.05 * W) * static_cast<double>(h[kResRows]) +
+                       1000.0 * static_cast<double>(h[kResLevels]) + 200.0 * fit * hops;
+    return kResGain * (build + run) < fit * blocks_ns * sms;
+}
+
 bool resident_degree_ok(int32_t max_degree) { return max_degree <= kResDegMax; }
 
 // Groups of `width` sources with neighbouring ids, one segment (and, on a
@@ -637,7 +682,7 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
         if (list.empty()) continue;
         g->res_list.reserve(list.size());
         g->res_over.reserve(list.size() + 1);
-        g->res_count.reserve(2);
+        g->res_count.reserve(kResCounts);
         SC_CUDA(cudaMemcpyAsync(g->res_list.get(), list.data(), list.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
         ResArgs a{};
         a.row_ptr = g->row_ptr.get();
@@ -656,6 +701,15 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
         a.over = g->res_over.get();
         // the first class: the one that holds the largest ball of a sample of the groups
         int cls = 0;
+        auto measure = [&](ResArgs m, int c, unsigned long long *h) {  // the balls of m's groups
+            SC_CUDA(cudaMemsetAsync(g->res_count.get(), 0, kResCounts * sizeof(unsigned long long), s));
+            m.count = g->res_count.get();
+            res_dispatch(g, m, fp64, W, c, bip, s);
+            ++st->launches;
+            SC_CUDA(cudaMemcpyAsync(h, g->res_count.get(), kResCounts * sizeof(unsigned long long),
+                                    cudaMemcpyDeviceToHost, s));
+            SC_CUDA(cudaStreamSynchronize(s));
+        };
         auto cap_of = [&](int c) { return fp64 ? res_cap_of<double>(W, c, bip) : res_cap_of<float>(W, c, bip); };
         int32_t seg_max = 0;
         for (size_t i = 0; i + 1 < seg_start.size(); ++i)
@@ -665,18 +719,14 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
             const int32_t ns = std::min<int32_t>(kResSample, a.ngroups);
             for (int32_t q = 0; q < ns; ++q) pick.push_back(list[static_cast<size_t>(q) * a.ngroups / ns]);
             SC_CUDA(cudaMemcpyAsync(g->res_over.get(), pick.data(), ns * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-            SC_CUDA(cudaMemsetAsync(g->res_count.get(), 0, 2 * sizeof(int32_t), s));
             ResArgs m = a;
             m.groups = g->res_over.get();
             m.ngroups = ns;
-            m.count = g->res_count.get();
-            res_dispatch(g, m, fp64, W, kResClasses - 2, bip, s);
-            ++st->launches;
-            int32_t h[2];
-            SC_CUDA(cudaMemcpyAsync(h, g->res_count.get(), sizeof(h), cudaMemcpyDeviceToHost, s));
-            SC_CUDA(cudaStreamSynchronize(s));
-            while (cls < kResClasses - 2 && h[0] > cap_of(cls)) ++cls;
-            if (h[1] == ns) cls = kResClasses - 1;  // no ball of the sample fits with its adjacency
+            unsigned long long h[kResCounts];
+            measure(m, kResClasses - 2, h);
+            while (cls < kResClasses - 2 && h[kResLargest] > static_cast<unsigned long long>(cap_of(cls))) ++cls;
+            // no ball of the sample fits with its adjacency
+            if (h[kResOver] == static_cast<unsigned long long>(ns)) cls = kResClasses - 1;
         }
         // groups of small segments need no more than the class that holds the segment, which leaves
         // room for more CTAs per SM: `list` starts with the smallest class in use, later classes get
@@ -735,6 +785,30 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
                 a.groups = nullptr;
                 a.ngroups = static_cast<int32_t>(single.size());
                 a.over = g->res_over.get();
+                const int32_t ns = kResSample;
+                if (a.ngroups > ns) {  // fewer run in one wave, as soon as measured
+                    std::vector<int32_t> pick;
+                    double blocks_ns = 0.0, hops = 0.0;
+                    for (int32_t q = 0; q < ns; ++q) {
+                        pick.push_back(static_cast<int32_t>(static_cast<int64_t>(q) * a.ngroups / ns));
+                        const int32_t v = single[pick.back()];
+                        blocks_ns += r.block_ns(v, h_len[v]);
+                        hops += h_len[v];
+                    }
+                    SC_CUDA(cudaMemcpyAsync(g->res_over.get(), pick.data(), ns * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+                    ResArgs m = a;
+                    m.groups = g->res_over.get();
+                    m.ngroups = ns;
+                    unsigned long long h[kResCounts];
+                    measure(m, cls, h);
+                    const int32_t cap_rows = fp64 ? res_global_rows<double>(W) : res_global_rows<float>(W);
+                    if (!global_class_pays(h, ns, hops, blocks_ns, W, static_cast<double>(g->nnz) / n, cap_rows,
+                                           g->num_sms > 0 ? g->num_sms : 148)) {
+                        left.insert(left.end(), single.begin(), single.end());
+                        list.clear();
+                        break;
+                    }
+                }
                 SC_CUDA(cudaMemsetAsync(g->res_over.get(), 0, sizeof(int32_t), s));
                 r.timed([&] { res_dispatch(g, a, fp64, W, cls, bip, s); });
                 ++st->launches;

@@ -16,6 +16,7 @@ struct ResidentRun {
     int extra;   // hops past each source's length (records)
     GatherRec rec;
     std::function<void(const std::function<void()> &)> timed;  // runs one traversal launch, with its events
+    std::function<double(int32_t, int32_t)> block_ns;  // source, hops: its share of the blocks' time, estimated
 };
 
 struct ResidentStats {

@@ -70,6 +70,33 @@ def _regular(n, d, seed):
     return gg.from_edges(n, np.concatenate(p), np.concatenate([np.roll(q, 1) for q in p]))
 
 
+def _bipartite(n, d, seed):
+    """A random bipartite graph of degree d: d random perfect matchings, renamed."""
+    rng = np.random.default_rng(seed)
+    h = n // 2
+    name = rng.permutation(n)
+    v = np.concatenate([h + rng.permutation(h) for _ in range(d)])
+    return gg.largest_component(gg.from_edges(n, name[np.tile(np.arange(h), d)], name[v]))
+
+
+@pytest.mark.parametrize("maker,ell,precision,resident", [
+    (lambda: _bipartite(14000, 4, 2), 15, "fp32", False),  # most of the graph within 8 hops: blocks
+    (lambda: _bipartite(14000, 4, 2), 15, "fp64", True),   # the same where a block's arithmetic is slow
+    (lambda: gg.relabel(gg.perturbed_grid(130, 131, 0.05, 5), np.random.default_rng(1).permutation(17030)), 121,
+     "fp32", True),
+])
+def test_balls_without_their_adjacency_by_cost(cuda_lib, maker, ell, precision, resident):
+    """Balls past the classes that hold their adjacency: resident only where that
+    is the faster form."""
+    g = maker()
+    kw = dict(policy="fixed", ell_fixed=ell, precision=precision)
+    with _graph(g) as G:
+        s, _, rep = G.all_edges(**kw)
+        s0, _, _ = G.all_edges(windows=False, **kw)
+    assert rep["resident_sources"] == (g.n if resident else 0)
+    assert np.array_equal(s, s0)
+
+
 def _regular_with_path(n, length, seed):
     """A random graph of degree 8, one edge of it replaced by a long path."""
     c = _regular(n, 8, seed)
