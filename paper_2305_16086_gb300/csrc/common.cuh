@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <map>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "../../include/sc.h"
@@ -228,6 +229,12 @@ struct sc_graph {
     int res_order_width[2] = {0, 0};
     int res_width = 0;
     bool res_ready = false;
+    // what a sample of its balls said, by (fp64, longest and mean run): the first class, and whether
+    // the class without the adjacency pays (-1: not asked)
+    struct ResChoice {
+        int first = 0, global = -1;
+    };
+    std::map<std::tuple<bool, int32_t, int32_t>, ResChoice> res_choice;
     sc::DevBuf<unsigned char> res_scratch;
     std::vector<cudaEvent_t> hop_events;  // pairs bracketing timed propagation launches
     std::vector<cudaEvent_t> walk_events;  // pairs bracketing TGT+ walk phases

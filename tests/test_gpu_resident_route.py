@@ -97,6 +97,33 @@ def test_balls_without_their_adjacency_by_cost(cuda_lib, maker, ell, precision, 
     assert np.array_equal(s, s0)
 
 
+@pytest.mark.parametrize("maker,ell,precision", [
+    (lambda: _regular(9000, 8, 1), 7, "fp32"),       # no ball fits
+    (lambda: _bipartite(14000, 4, 2), 15, "fp32"),   # balls that fit at a cost
+    (lambda: gg.perturbed_grid(90, 100, 0.05, 5), 61, "fp32"),
+])
+def test_the_sample_of_a_whole_request_is_kept(cuda_lib, maker, ell, precision):
+    """A repeated call launches what the first did but for the sample's launches
+    (and the neighbour rows laid out once); another length, then the first again,
+    and a query stay right."""
+    from paper_2305_16086_gb300 import binding
+
+    g = maker()
+    kw = dict(policy="fixed", ell_fixed=ell, precision=precision)
+    with _graph(g) as G:
+        _, _, first = G.all_edges(**kw)
+        s, _, again = G.all_edges(**kw)
+        short, _, _ = G.all_edges(policy="fixed", ell_fixed=4, precision=precision)
+        _, _, third = G.all_edges(**kw)
+        ent = np.random.default_rng(3).integers(0, g.nnz, 300)
+        q, _ = binding.some_edges(G, ent, **kw)
+        s0, _, _ = G.all_edges(windows=False, **kw)
+        short0, _, _ = G.all_edges(policy="fixed", ell_fixed=4, precision=precision, windows=False)
+    assert again["launches"] == third["launches"] < first["launches"] - 1
+    assert again["resident_sources"] == third["resident_sources"] == first["resident_sources"]
+    assert np.array_equal(s, s0) and np.array_equal(q, s0[ent]) and np.array_equal(short, short0)
+
+
 def _regular_with_path(n, length, seed):
     """A random graph of degree 8, one edge of it replaced by a long path."""
     c = _regular(n, 8, seed)
