@@ -2059,30 +2059,32 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
     R.log2md = std::log(2.0 * static_cast<double>(nnz / 2) / delta);
     R.extra = record_after ? 2 : 0;
     R.rec = rec;
-    // the launch shape by timing (cached per graph and request)
-    auto time_shape = [&] {
+    // The launch shape by timing, cached per graph and request. In the middle of a run (held) the sample
+    // blocks write accumulators of their own.
+    auto time_shape = [&](bool held) {
+        const long long key = (static_cast<long long>(tune_prec) << 56) ^ (static_cast<long long>(fixV + 1) << 52) ^
+                              (static_cast<long long>(o.max_slices & 0xfff) << 40) ^
+                              (static_cast<long long>(Lmax) << 16) ^ (static_cast<long long>(use_win) << 15) ^
+                              (static_cast<long long>(rec.mode) << 12) ^
+                              (static_cast<long long>((o.flags & SC_OPT_SPARSE_HOPS) != 0) << 11) ^
+                              (static_cast<long long>(o.ell_policy) << 8) ^ (static_cast<long long>(o.estimator) << 6) ^
+                              (static_cast<long long>(plus) << 5) ^ static_cast<long long>(std::min(h0, 31));
+        const auto hit = g->tuned_block.find(key);
+        if (held && hit != g->tuned_block.end()) return take_shape(hit->second);
+        std::unique_ptr<ScratchAccumulators> scratch(held ? new ScratchAccumulators(g) : nullptr);
         std::vector<TuneResult> per_b;
         take_shape(autotune(g, tune_prec, o.block_width, fixV, o.max_slices, Lmax, GatherRec{rec.mode, nullptr, 0},
                             !use_win, s, &per_b));
-        if (per_b.size() > 1 && Lmax >= 2) {
-            // the block width from one real block of each (the request's lengths, kernels and records)
-            const long long key = (static_cast<long long>(tune_prec) << 56) ^ (static_cast<long long>(fixV + 1) << 52) ^
-                                  (static_cast<long long>(o.max_slices & 0xfff) << 40) ^
-                                  (static_cast<long long>(Lmax) << 16) ^ (static_cast<long long>(use_win) << 15) ^
-                                  (static_cast<long long>(rec.mode) << 12) ^
-                                  (static_cast<long long>((o.flags & SC_OPT_SPARSE_HOPS) != 0) << 11) ^
-                                  (static_cast<long long>(o.ell_policy) << 8) ^
-                                  (static_cast<long long>(o.estimator) << 6) ^ (static_cast<long long>(plus) << 5) ^
-                                  static_cast<long long>(std::min(h0, 31));
+        if (per_b.size() > 1 && Lmax >= 2)  // the block width from one real block of each (the request's lengths,
+                                            // kernels and records)
             take_shape(pick_block_width(R, per_b, len, Lmax, use_win, beta,
                                         std::vector<char>{static_cast<char>(g->bipartite ? 1 : 0)}, key));
-        }
     };
     if (use_res) {
         take_shape(untimed_shape(tune_prec));
         use_win = use_win || leftover_windows(g, beta, Lmax, R.B, elem, o.precision == SC_PREC_FP64);
     } else {
-        time_shape();
+        time_shape(false);
     }
     std::vector<int32_t> depth;
     if (learned_plus) {
@@ -2132,8 +2134,7 @@ static void all_edges_impl(sc_graph *g, const sc_options *o_in, double *s_hat, d
             left = resident_blocks(R, src, l, seg_whole, std::vector<char>{1}, seg_bip, use_win ? beta : -1);
             if (left.empty()) return;
             if (!use_win && !timed_shape && static_cast<int64_t>(left.size()) > kUntimedBlocks * R.B) {
-                ScratchAccumulators scratch(g);  // the sources that ran have their sums in the graph's
-                time_shape();
+                time_shape(true);  // the sources that ran have their sums in the graph's accumulators
                 timed_shape = true;
             }
             if (!use_win) {
