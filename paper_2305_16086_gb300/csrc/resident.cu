@@ -41,7 +41,8 @@ namespace sc {
 
 constexpr int kResDegMax = 8;       // largest degree taken (neighbour ids kept per row)
 constexpr int kResClasses = 4;      // shared-memory sizes tried in turn; the last keeps the adjacency in global memory
-constexpr int kResIdOrder = 4;      // hops per level from which the lists are kept in id order
+constexpr int kResIdOrder = 4;      // hops per level from which the lists are kept in id order,
+constexpr int kResIdHops = 64;      // and hops: the ranks cost an SM 40 us on 4,200 nodes, six of its hops
 constexpr int kResSample = 128;     // groups whose ball is measured to choose the first class
 
 // what a measuring launch counts: the largest list, the groups that did not fit; of the others the
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
         int32_t m0 = n0, m1 = n1;  // list lengths (in id order the empty source slots are gone)
         bool by_id = false;
         if constexpr (!GADJ) {
-            if (Lg >= kResIdOrder * top) {
+            if (Lg >= kResIdOrder * top && Lg >= kResIdHops) {
                 if (tid == 0) span[0] = INT32_MAX, span[1] = -1;
                 __syncthreads();
                 for (int32_t t = tid; t < n0 + n1; t += T) {

@@ -30,6 +30,19 @@ def test_small_graphs_run_resident(cuda_lib, name, precision, ell, estimator):
     assert rep1["resident_sources"] == 0 and rep1["windowed"] == 1
 
 
+@pytest.mark.parametrize("name", ["lattice", "renamed", "odd_cycle", "kings", "cube", "small"])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("ell", [63, 64, 331])
+def test_runs_of_many_more_hops_than_levels(cuda_lib, name, precision, ell):
+    """From 64 hops and four a level on the lists are in id order."""
+    g = GRAPHS[name]()
+    with _graph(g) as G:
+        s, _, rep = G.all_edges(policy="fixed", ell_fixed=ell, precision=precision)
+        s0, _, _ = G.all_edges(policy="fixed", ell_fixed=ell, precision=precision, windows=False)
+    assert rep["resident_sources"] == g.n
+    assert np.array_equal(s, s0)
+
+
 @pytest.mark.parametrize("maker,ell,precision,share", [
     (lambda: gg.perturbed_grid(60, 140, 0.05, 5), 81, "fp32", "all"),    # 8,400 nodes, balls of half of them
     (lambda: gg.perturbed_grid(130, 131, 0.05, 5), 201, "fp32", "all"),  # 17,030 nodes: without the adjacency
