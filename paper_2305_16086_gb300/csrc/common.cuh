@@ -236,6 +236,7 @@ struct sc_graph {
     };
     std::map<std::tuple<bool, int32_t, int32_t>, ResChoice> res_choice;
     sc::DevBuf<unsigned char> res_scratch;
+    sc::DevBuf<uint16_t> res_marks;  // per CTA a local id per node, 0xffff between launches
     std::vector<cudaEvent_t> hop_events;  // pairs bracketing timed propagation launches
     std::vector<cudaEvent_t> walk_events;  // pairs bracketing TGT+ walk phases
     long long *h_counters = nullptr;       // page-locked: a switch test's sums

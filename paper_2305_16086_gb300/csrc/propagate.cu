@@ -11,6 +11,7 @@
 
 #include <cudaTypedefs.h>
 
+#include "budget.h"
 #include "hop2_mask.cuh"
 #include "hop_tma.cuh"
 #include "resident.cuh"
@@ -1534,7 +1535,7 @@ static void run_blocks_win(Run &R, std::vector<int32_t> sources, const std::vect
     size_t free_b = 0, total_b = 0;
     SC_CUDA(cudaMemGetInfo(&free_b, &total_b));
     const double budget = std::max(static_cast<double>(R.slice_bytes),
-                                   std::min(4.0 * (1ull << 30), 0.125 * static_cast<double>(free_b)));
+                                   traversal_budget(free_b));
     const int max_sl = R.o->max_slices > 0 ? std::min(R.o->max_slices, 65535) : 65535;
     std::vector<size_t> sb_begin;
     size_t need = 0;

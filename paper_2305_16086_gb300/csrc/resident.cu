@@ -35,6 +35,7 @@
 #include <algorithm>
 #include <numeric>
 
+#include "budget.h"
 #include "resident.cuh"
 
 namespace sc {
@@ -66,8 +67,13 @@ struct ResArgs {
     GatherRec rec;
     int32_t *over;           // [0]: groups that did not fit, [1 ..]: their ids
     unsigned long long *count;  // nullable: measure the balls only (ResCount)
-    unsigned char *scratch;  // global-adjacency class: per CTA adjacency, 1/d, nodes, local id per node
+    // global-adjacency class: per CTA adjacency, 1/d and nodes, and a local id per node of the graph
+    // (0xffff between launches: a CTA takes its ball's back)
+    unsigned char *scratch;
     size_t scratch_cta;
+    uint16_t *marks;
+    size_t marks_cta;
+    int32_t ctas;            // (host) its CTAs
 };
 
 template <typename Acc, int C>
@@ -115,7 +121,7 @@ __global__ void __launch_bounds__(1024) k_resident(const ResArgs a) {
         adj = reinterpret_cast<Adj *>(q);
         inv = reinterpret_cast<Acc *>(q + L::adj_bytes(N));
         nodes = reinterpret_cast<int32_t *>(q + L::adj_bytes(N) + L::inv_bytes(N));
-        hval = reinterpret_cast<uint16_t *>(q + L::adj_bytes(N) + L::inv_bytes(N) + L::up(static_cast<size_t>(N) * 4));
+        hval = a.marks + blockIdx.x * a.marks_cta;
     } else {
         adj = reinterpret_cast<Adj *>(p);
         inv = reinterpret_cast<Acc *>(p + L::adj_bytes(N));
@@ -519,6 +525,8 @@ static int32_t res_capacity(int cls) {
     return static_cast<int32_t>(BIP ? rows / 2 : rows);
 }
 
+static size_t marks_stride(int32_t n) { return (static_cast<size_t>(n) + 127) / 128 * 128; }
+
 template <typename Acc, int W, bool BIP, bool GADJ>
 static void res_launch(sc_graph *g, ResArgs a, int cls, cudaStream_t s) {
     constexpr int C = GADJ ? 1 : 16 / static_cast<int>(sizeof(Acc));
@@ -531,12 +539,16 @@ static void res_launch(sc_graph *g, ResArgs a, int cls, cudaStream_t s) {
     a.hash = GADJ ? 0 : std::min<int>(2 * N, static_cast<int>((L::x_bytes(N) - L::up(static_cast<size_t>(N) * 4)) / 6));
     int grid = a.ngroups;
     if (GADJ) {
-        grid = std::min(grid, (g->num_sms > 0 ? g->num_sms : 148) * k.per_sm);
-        a.scratch_cta = L::adj_bytes(N) + L::inv_bytes(N) + L::up(static_cast<size_t>(N) * 4) +
-                        (static_cast<size_t>(g->n) * 2 + 255) / 256 * 256;
-        g->res_scratch.reserve(a.scratch_cta * grid);
-        SC_CUDA(cudaMemsetAsync(g->res_scratch.get(), 0xff, a.scratch_cta * grid, s));
+        grid = std::min(grid, a.ctas);
+        a.scratch_cta = L::adj_bytes(N) + L::inv_bytes(N) + L::up(static_cast<size_t>(N) * 4);
+        g->res_scratch.reserve(a.scratch_cta * a.ctas);
         a.scratch = g->res_scratch.get();
+        a.marks_cta = marks_stride(g->n);
+        if (g->res_marks.count < a.marks_cta * a.ctas) {
+            g->res_marks.reserve(a.marks_cta * a.ctas);
+            SC_CUDA(cudaMemsetAsync(g->res_marks.get(), 0xff, g->res_marks.count * sizeof(uint16_t), s));
+        }
+        a.marks = g->res_marks.get();
     }
     auto *fn = k_resident<Acc, C, W, BIP, GADJ>;
     SC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(k.smem)));
@@ -813,6 +825,15 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
                 a.groups = nullptr;
                 a.ngroups = static_cast<int32_t>(single.size());
                 a.over = g->res_over.get();
+                size_t free_b = 0, total_b = 0;
+                SC_CUDA(cudaMemGetInfo(&free_b, &total_b));
+                a.ctas = global_class_ctas(marks_stride(n) * sizeof(uint16_t), single.size(), g->num_sms,
+                                           g->res_marks.count * sizeof(uint16_t), free_b);
+                if (a.ctas == 0) {  // (2 bytes a node and SM: 14 million nodes in 4 GB)
+                    left.insert(left.end(), single.begin(), single.end());
+                    list.clear();
+                    break;
+                }
                 const int32_t ns = kResSample;
                 if (choice.global < 0 && a.ngroups > ns) {  // fewer run in one wave, as soon as measured
                     std::vector<int32_t> pick;

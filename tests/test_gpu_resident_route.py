@@ -110,6 +110,38 @@ def test_balls_without_their_adjacency_by_cost(cuda_lib, maker, ell, precision, 
     assert np.array_equal(s, s0)
 
 
+def test_node_marks_are_taken_back(cuda_lib):
+    """The class without the adjacency marks a ball's nodes and takes the marks
+    back: calls of both precisions, of few sources and of many, and ones whose
+    balls do not fit, leave nothing behind for the next."""
+    from paper_2305_16086_gb300 import binding
+
+    g = gg.perturbed_grid(130, 131, 0.05, 5)
+    rng = np.random.default_rng(4)
+    with _graph(g) as G:
+        want = {}
+        for p in ("fp32", "fp64"):
+            want[p], _, _ = G.all_edges(policy="fixed", ell_fixed=141, precision=p, windows=False)
+        for precision, count in (("fp32", 5), ("fp64", 300), ("fp32", 120), ("fp64", 4), ("fp32", 2000)):
+            ent = rng.integers(0, g.nnz, count)
+            q, rep = binding.some_edges(G, ent, policy="fixed", ell_fixed=141, precision=precision)
+            nsrc = np.unique(np.concatenate([g.entry_rows()[ent], g.col_idx[ent]])).size
+            assert rep["resident_sources"] == nsrc
+            assert np.array_equal(q, want[precision][ent])
+    # 67,860 nodes: in mid-lattice balls past the class, marks up to where they overflow
+    g = gg.perturbed_grid(260, 261, 0.05, 5)
+    mid = 130 * 261 + 130
+    ent = g.row_ptr[mid:mid + 60].astype(np.int64)
+    with _graph(g) as G:
+        a, ra = binding.some_edges(G, ent, policy="fixed", ell_fixed=401, precision="fp32")
+        b, rb = binding.some_edges(G, ent, policy="fixed", ell_fixed=201, precision="fp32")
+        a0, _ = binding.some_edges(G, ent, policy="fixed", ell_fixed=401, precision="fp32", windows=False)
+        b0, _ = binding.some_edges(G, ent, policy="fixed", ell_fixed=201, precision="fp32", windows=False)
+    nsrc = np.unique(np.concatenate([g.entry_rows()[ent], g.col_idx[ent]])).size
+    assert 0 < ra["resident_sources"] < nsrc and rb["resident_sources"] == nsrc
+    assert np.array_equal(a, a0) and np.array_equal(b, b0)
+
+
 @pytest.mark.parametrize("maker,ell,precision", [
     (lambda: _regular(9000, 8, 1), 7, "fp32"),       # no ball fits
     (lambda: _bipartite(14000, 4, 2), 15, "fp32"),   # balls that fit at a cost
