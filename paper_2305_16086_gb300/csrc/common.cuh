@@ -169,6 +169,7 @@ struct sc_graph {
     sc::DevBuf<uint32_t> fr_pairs;
     sc::DevBuf<unsigned char> fr_part, fr_sec;
     int32_t front_hchunks = 0, front_hrows = 0, front_runs = 0;
+    int32_t front_pair_rows[3] = {0, 0, 0};  // rows of up to 1, 2 and 4 chunks
     bool front_ready = false;
     // row runs of about equal CSR entries, one per warp, for the TMA kernel
     sc::DevBuf<int32_t> part;

@@ -421,6 +421,7 @@ static void ensure_front(sc_graph *g) {
     if (g->front_ready) return;
     std::vector<int32_t> hi_row, hi_k0, hv_id, hv_first, run_lo, run_hi;
     int32_t lo = 0;  // first row of the open run
+    int32_t upto[3] = {0, 0, 0};
     auto close_run = [&](int32_t r) {
         if (r > lo) {
             run_lo.push_back(lo);
@@ -431,6 +432,7 @@ static void ensure_front(sc_graph *g) {
     for (int32_t r = 0; r < g->n; ++r) {
         const int32_t b = g->h_row_ptr[r], e = g->h_row_ptr[r + 1];
         if (r - lo == kFrontRunRows || e - g->h_row_ptr[lo] > kFrontRun || e - b > kFrontHeavy) close_run(r);
+        for (int k = 0; k < 3; ++k) upto[k] += e - b <= kChunk << k;
         if (e - b <= kFrontHeavy) continue;
         lo = r + 1;
         hv_first.push_back(static_cast<int32_t>(hi_row.size()));
@@ -457,6 +459,7 @@ static void ensure_front(sc_graph *g) {
     g->front_hchunks = static_cast<int32_t>(hi_row.size());
     g->front_hrows = static_cast<int32_t>(hv_id.size());
     g->front_runs = static_cast<int32_t>(run_lo.size());
+    std::copy(upto, upto + 3, g->front_pair_rows);
     g->front_ready = true;
 }
 
@@ -511,9 +514,10 @@ static void front_t(sc_graph *g, const FrontLaunch &h, cudaStream_t s) {
     g->fr_sec.reserve(nodes * sizeof(typename SectorMask<T, B>::Word));
     a.sectors = g->fr_sec.get();
     if (h.lists || h.which == 0) {
-        g->fr_pairs.reserve(4 * nodes * kBallSparseCols);
+        g->fr_pairs.reserve(nodes * kBallSparseCols);
         g->fr_rows.reserve(nodes);
         a.pairs = g->fr_pairs.get();
+        std::copy(g->front_pair_rows, g->front_pair_rows + 3, a.pair_rows);
         a.rows = g->fr_rows.get();
     }
     const int sms = g->num_sms > 0 ? g->num_sms : 148;

@@ -114,9 +114,12 @@ struct FrontArgs {
     int32_t nruns;
     Acc *part;             // slices x nhchunks x B chunk sums
     int32_t *arrived;      // slices x nhrows (zeroed before hop 2, one set a hop)
-    // work lists of hop L-1, per slice: pairs row * B + column by chunks of the row (capacity
-    // kBallSparseCols * n each), rows (capacity n); their lengths (zeroed before hop 2; nullable: none made)
-    uint32_t *pairs;       // 4 x slices x kBallSparseCols x n
+    // work lists of hop L-1, per slice: pairs row * B + column by chunks of the row, rows (capacity n);
+    // their lengths (zeroed before hop 2; nullable: none made). A row's kind is a matter of its degree, so
+    // the four lists of pairs lie end to end, kBallSparseCols times the rows of each: pair_rows[k], the
+    // rows of the kinds before k + 1
+    uint32_t *pairs;       // slices x kBallSparseCols x n
+    int32_t pair_rows[3];
     int32_t *rows;         // slices x n
     int32_t *lists;        // slices x kBallLists
     int32_t list_ctas;     // hop 3: CTAs that make them
@@ -129,6 +132,13 @@ struct FrontArgs {
     double *g, *t1, *t2;
     GatherRec rec;
 };
+
+// the list of pairs of one kind and slice
+template <typename T>
+__device__ __forceinline__ uint32_t *pair_list(const FrontArgs<T> &a, int kind, int64_t slice) {
+    const int32_t before = kind == 0 ? 0 : kind == 1 ? a.pair_rows[0] : kind == 2 ? a.pair_rows[1] : a.pair_rows[2];
+    return a.pairs + (slice * a.n + before) * kBallSparseCols;
+}
 
 // The chunk sums of a heavy row meet: the warp stores its E values per lane
 // (lanes past B / E hold none), and the last warp of the row to arrive adds all
@@ -415,7 +425,7 @@ __device__ __forceinline__ void list_row(const FrontArgs<T> &a, int64_t slice, i
         a.rows[slice * a.n + first] = row;
         return;
     }
-    uint32_t *out = a.pairs + (static_cast<int64_t>(kind) * gridDim.y + slice) * kBallSparseCols * a.n + first;
+    uint32_t *out = pair_list(a, kind, slice) + first;
 #pragma unroll
     for (int q = 0; q < W; ++q) {
         uint32_t bits = need[q];
@@ -693,7 +703,7 @@ __global__ void __launch_bounds__(kSpmmWarps * 32) k_ball(const FrontArgs<T> a) 
         int32_t r = 0, k0 = 0, cnt = 0;
         Acc sc = Acc(0);
         if (at < count) {
-            pr = a.pairs[(static_cast<int64_t>(kind) * gridDim.y + slice) * kBallSparseCols * a.n + at];
+            pr = pair_list(a, kind, slice)[at];
             r = static_cast<int32_t>(pr / B);
             k0 = row_ptr[r] + (lane & ((1 << kind) - 1)) * kChunk;
             cnt = min(kChunk, row_ptr[r + 1] - k0);
