@@ -84,6 +84,7 @@ constexpr int kDotBlocks = 256, kDotThreads = 256, kDotVectors = 2 * kDotThreads
 // blocks of a kernel whose per-block shares the next one sums in every block: eight per SM, so
 // that the sums stay a few loads per thread however many rows there are
 constexpr int kShareBlocks = 8 * 152;
+constexpr int kRunAhead = 32;  // Lanczos steps from which a check is read behind the next steps
 
 static dim3 dot_grid(int nvec) { return dim3(kDotBlocks, std::max(1, ceil_div(nvec, kDotVectors))); }
 
@@ -555,11 +556,12 @@ sc_status estimate_lambda_impl(sc_graph *g, const sc_lambda_opts *opts, sc_lambd
 
         // alpha_j and |w_j|^2 of every step stay on the device; the host reads
         // them only at the steps where it checks convergence (every 4th from
-        // step 8, and the last possible one). A check's copies go to page-locked
-        // memory, and the steps up to the next check are queued before the host
-        // waits for them, so that the GPU works on while the host solves the
-        // tridiagonal problem; steps past the one the check stops at are
-        // discarded. A breakdown (|w_j| <= 1e-12) between two checks is found at
+        // step 8, and the last possible one). From step kRunAhead on a check's
+        // copies go to page-locked memory, and the steps up to the next check are
+        // queued before the host waits for them, so that the GPU works on while the
+        // host solves the tridiagonal problem; steps past the one the check stops at
+        // are discarded. (Before that the host waits: page-locked memory costs a call
+        // 0.6 ms, which a short one does not earn back.) A breakdown (|w_j| <= 1e-12) between two checks is found at
         // the next one and the steps after it are discarded too, which gives the
         // same steps and result as stopping at the breakdown itself.
         DevBuf<double> ab;
@@ -567,18 +569,16 @@ sc_status estimate_lambda_impl(sc_graph *g, const sc_lambda_opts *opts, sc_lambd
         double *d_alpha = ab.get(), *d_nrm2 = d_alpha + max_iter, *d_one = d_nrm2 + max_iter;
         struct Check {  // a check's copies and the event behind them, two in turn
             double *h = nullptr;  // alpha, |w|^2, one sweep enough: max_iter values each
+            double *locked = nullptr;
             cudaEvent_t done = nullptr;
             int kk = 0;  // steps at the check (0: none queued)
             ~Check() {
                 if (done) cudaEventDestroy(done);
-                if (h) cudaFreeHost(h);
+                if (locked) cudaFreeHost(locked);
             }
         } check[2];
-        for (Check &c2 : check) {
-            SC_CUDA(cudaMallocHost(reinterpret_cast<void **>(&c2.h),
-                                   3 * static_cast<size_t>(max_iter) * sizeof(double)));
-            SC_CUDA(cudaEventCreateWithFlags(&c2.done, cudaEventDisableTiming));
-        }
+        const size_t check_bytes = 3 * static_cast<size_t>(max_iter) * sizeof(double);
+        std::vector<double> early(3 * static_cast<size_t>(max_iter));
         struct Drain {  // queued copies end before their buffers go
             cudaStream_t s;
             ~Drain() { cudaStreamSynchronize(s); }
@@ -591,7 +591,8 @@ sc_status estimate_lambda_impl(sc_graph *g, const sc_lambda_opts *opts, sc_lambd
         auto settle = [&](Check &c2) {  // the host side of a queued check
             const int kk = c2.kk;
             c2.kk = 0;
-            SC_CUDA(cudaEventSynchronize(c2.done));
+            if (c2.h == c2.locked) SC_CUDA(cudaEventSynchronize(c2.done));
+            else SC_CUDA(cudaStreamSynchronize(s));
             const double *h_alpha = c2.h, *h_nrm2 = c2.h + max_iter, *h_one = c2.h + 2 * static_cast<size_t>(max_iter);
             for (int q = static_cast<int>(alpha.size()); q < kk; ++q)
                 if (h_one[q] == 0.0) {
@@ -629,15 +630,19 @@ sc_status estimate_lambda_impl(sc_graph *g, const sc_lambda_opts *opts, sc_lambd
             if (kk == max_iter || kk == n - nlock || (kk >= 8 && kk % 4 == 0)) {
                 Check &now = check[turn], &before = check[turn ^ 1];
                 turn ^= 1;
-                SC_CUDA(cudaMemcpyAsync(now.h, d_alpha, kk * sizeof(double), cudaMemcpyDeviceToHost, s));
-                SC_CUDA(cudaMemcpyAsync(now.h + max_iter, d_nrm2, kk * sizeof(double), cudaMemcpyDeviceToHost, s));
-                SC_CUDA(cudaMemcpyAsync(now.h + 2 * static_cast<size_t>(max_iter), d_one, kk * sizeof(double),
-                                        cudaMemcpyDeviceToHost, s));
-                SC_CUDA(cudaEventRecord(now.done, s));
+                const bool ahead = kk >= kRunAhead;
+                if (ahead && !now.locked) {
+                    SC_CUDA(cudaMallocHost(reinterpret_cast<void **>(&now.locked), check_bytes));
+                    SC_CUDA(cudaEventCreateWithFlags(&now.done, cudaEventDisableTiming));
+                }
+                now.h = ahead ? now.locked : early.data();
+                SC_CUDA(cudaMemcpy2DAsync(now.h, max_iter * sizeof(double), d_alpha, max_iter * sizeof(double),
+                                          kk * sizeof(double), 3, cudaMemcpyDeviceToHost, s));
+                if (ahead) SC_CUDA(cudaEventRecord(now.done, s));
                 now.kk = kk;
                 if (before.kk) settle(before);
                 const bool last = kk == max_iter || kk == n - nlock;
-                if (!ended && redo < 0 && last) settle(now);  // nothing to queue behind it
+                if (!ended && redo < 0 && (last || !ahead)) settle(now);  // nothing to queue behind it
                 if (ended) break;
                 if (redo >= 0) {  // step `redo` again, carefully; what was queued after it is dropped
                     careful = true;
