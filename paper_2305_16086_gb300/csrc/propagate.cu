@@ -1580,8 +1580,8 @@ static void run_blocks_win(Run &R, std::vector<int32_t> sources, const std::vect
         }
     } cs;
     cudaStream_t is = s;
+    SC_CUDA(cudaStreamSynchronize(s));  // the copies of the lists, which go when this returns before the GPU is done
     if (R.capture) {
-        SC_CUDA(cudaStreamSynchronize(s));
         SC_CUDA(cudaStreamCreateWithFlags(&cs.c, cudaStreamNonBlocking));
         is = cs.c;
     }

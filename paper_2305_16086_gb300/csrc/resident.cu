@@ -713,7 +713,18 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
         g->res_list.reserve(list.size());
         g->res_over.reserve(list.size() + 1);
         g->res_count.reserve(kResCounts);
-        SC_CUDA(cudaMemcpyAsync(g->res_list.get(), list.data(), list.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+        // (a copy from host memory may still read it when the call returns)
+        bool copying = false;
+        auto put_list = [&] {
+            SC_CUDA(cudaMemcpyAsync(g->res_list.get(), list.data(), list.size() * sizeof(int32_t),
+                                    cudaMemcpyHostToDevice, s));
+            copying = true;
+        };
+        auto free_list = [&] {  // before `list` changes
+            if (copying) SC_CUDA(cudaStreamSynchronize(s));
+            copying = false;
+        };
+        put_list();
         ResArgs a{};
         a.row_ptr = g->row_ptr.get();
         a.ell = g->res_ell.get();
@@ -787,10 +798,10 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
                     const size_t i = std::upper_bound(seg_start.begin(), seg_start.end(), v) - seg_start.begin() - 1;
                     (seg_class[i] == lowest ? first : later[seg_class[i]]).push_back(q);
                 }
+                free_list();
                 list.swap(first);
                 cls = lowest;
-                SC_CUDA(cudaMemcpyAsync(g->res_list.get(), list.data(), list.size() * sizeof(int32_t),
-                                        cudaMemcpyHostToDevice, s));
+                put_list();
             }
         }
         auto more = [&](int c) {
@@ -800,10 +811,10 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
         };
         for (; cls < kResClasses && (!list.empty() || more(cls)); ++cls) {
             if (!later[cls].empty()) {  // with what earlier classes left over
+                free_list();
                 list.insert(list.end(), later[cls].begin(), later[cls].end());
                 later[cls].clear();
-                SC_CUDA(cudaMemcpyAsync(g->res_list.get(), list.data(), list.size() * sizeof(int32_t),
-                                        cudaMemcpyHostToDevice, s));
+                put_list();
             }
             if (list.empty()) continue;
             if (cls == kResClasses - 1) {
@@ -879,15 +890,17 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
             int32_t nover = 0;
             SC_CUDA(cudaMemcpyAsync(&nover, g->res_over.get(), sizeof(int32_t), cudaMemcpyDeviceToHost, s));
             SC_CUDA(cudaStreamSynchronize(s));
+            copying = false;
             list.resize(nover);
             if (nover > 0) {
                 SC_CUDA(cudaMemcpyAsync(list.data(), g->res_over.get() + 1, nover * sizeof(int32_t),
                                         cudaMemcpyDeviceToHost, s));
                 SC_CUDA(cudaStreamSynchronize(s));
                 std::sort(list.begin(), list.end());
-                SC_CUDA(cudaMemcpyAsync(g->res_list.get(), list.data(), nover * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+                put_list();
             }
         }
+        free_list();
         for (int32_t q : list)
             for (int c = 0; c < width; ++c) {
                 const int32_t v = order[static_cast<size_t>(q) * width + c];
