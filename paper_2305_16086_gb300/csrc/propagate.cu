@@ -2740,9 +2740,6 @@ static void batch_impl(sc_graph *const *graphs, int32_t count, const sc_options 
     seg_start[count] = N;
     // per graph: source-hops, sources run resident, shortest and longest source run
     std::vector<int64_t> g_hops(count, 0), g_resident(count, 0);
-    auto seg_at = [&](int32_t v) {
-        return static_cast<size_t>(std::upper_bound(seg_start.begin(), seg_start.end(), v) - seg_start.begin()) - 1;
-    };
     std::vector<int32_t> g_lmin(count, INT32_MAX), g_lmax(count, 0);
     auto book = [&](const std::vector<int32_t> &src) {
         int32_t i = 0;
@@ -2766,8 +2763,13 @@ static void batch_impl(sc_graph *const *graphs, int32_t count, const sc_options 
         }
         if (!res.empty()) {
             const std::vector<int32_t> left = resident_blocks(R, res, len, seg_start, seg_take, seg_bip, beta);
-            for (int32_t v : res) g_resident[seg_at(v)] += len[v] + extra > 0 ? 1 : 0;
-            for (int32_t v : left) --g_resident[seg_at(v)];
+            size_t q = 0;  // both lists are in id order
+            i = 0;
+            for (int32_t v : res) {
+                while (v >= n_off[i + 1]) ++i;
+                while (q < left.size() && left[q] < v) ++q;
+                if ((q == left.size() || left[q] != v) && len[v] + extra > 0) ++g_resident[i];
+            }
             rest.insert(rest.end(), left.begin(), left.end());
         }
         run_blocks_win(R, rest, len, seg_start, beta, seg_bip);
