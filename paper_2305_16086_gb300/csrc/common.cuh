@@ -8,6 +8,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <map>
+#include <set>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -236,6 +237,8 @@ struct sc_graph {
         int first = 0, global = -1;
     };
     std::map<std::tuple<bool, int32_t, int32_t>, ResChoice> res_choice;
+    // as a member of batches: (fp64, hops) of runs in which none of its sources ran resident
+    std::set<std::pair<bool, int32_t>> res_batch_none;
     sc::DevBuf<unsigned char> res_scratch;
     sc::DevBuf<uint16_t> res_marks;  // per CTA a local id per node, 0xffff between launches
     std::vector<cudaEvent_t> hop_events;  // pairs bracketing timed propagation launches

@@ -2687,12 +2687,17 @@ static void batch_impl(sc_graph *const *graphs, int32_t count, const sc_options 
     const int fixV = o.rows_split == 0 ? -1 : o.rows_split;
     const int32_t h0 = bf16_first_hop(o);
     const int tune_prec = (o.precision == SC_PREC_BF16 && h0 > 1) ? SC_PREC_FP32 : o.precision;
-    // graphs of small degree run resident; the block kernels take the others
+    // graphs of small degree run resident; the block kernels take the others, and those of which no
+    // source ran resident before (six random 8-regular graphs of 6,000 nodes at 9 hops: 0.8 of 10.7 ms)
+    const bool fp64 = o.precision == SC_PREC_FP64;
     std::vector<char> seg_take(count, 0);
     int32_t res_deg = 0;
     bool all_res = true;
     for (int32_t i = 0; i < count; ++i) {
-        seg_take[i] = resident_allowed(o) && resident_degree_ok(graphs[i]->max_degree) ? 1 : 0;
+        seg_take[i] = resident_allowed(o) && resident_degree_ok(graphs[i]->max_degree) &&
+                              (learned || !graphs[i]->res_batch_none.count({fp64, ell[i] + extra}))
+                          ? 1
+                          : 0;
         if (seg_take[i]) res_deg = std::max(res_deg, graphs[i]->max_degree);
         else all_res = false;
     }
@@ -2776,6 +2781,9 @@ static void batch_impl(sc_graph *const *graphs, int32_t count, const sc_options 
         book(src);
     };
     run(all);
+    if (!learned)
+        for (int32_t i = 0; i < count; ++i)
+            if (seg_take[i] && g_resident[i] == 0) graphs[i]->res_batch_none.insert({fp64, ell[i] + extra});
 
     // ---- combine (and for the learned lengths the check / extension loop), Foster sums, outputs
     DevBuf<double> d_s, seg_sum;

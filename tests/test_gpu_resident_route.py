@@ -211,3 +211,24 @@ def test_left_over_sources_take_the_better_blocks(cuda_lib, maker, ell, precisio
     assert np.array_equal(s, s0) and np.array_equal(q, s0[ent])
     if b is not None:
         assert np.array_equal(b, b0)
+
+
+def test_batches_of_graphs_that_do_not_run_resident(cuda_lib):
+    """A member of which no source ran resident is left to the blocks in later
+    batches of the same length and precision; others are tried again."""
+    from paper_2305_16086_gb300 import Graph, binding
+
+    gs = [_regular(6000, 8, 1), gg.perturbed_grid(20, 31, 0.05, 1), _regular(6000, 8, 2)]
+    Gs = [Graph(g.row_ptr, g.col_idx) for g in gs]
+    try:
+        seen = []
+        for ells, precision in (([9, 45, 9], "fp32"), ([9, 45, 9], "fp32"), ([3, 45, 9], "fp32"), ([9, 45, 9], "fp64")):
+            out, reps = binding.batch_all_edges(Gs, ells, policy="fixed", precision=precision)
+            for G, e, s in zip(Gs, ells, out):
+                s0, _, _ = G.all_edges(policy="fixed", ell_fixed=e, precision=precision, windows=False)
+                assert np.array_equal(s, s0)
+            seen.append([r["resident_sources"] for r in reps])
+    finally:
+        for G in Gs:
+            G.close()
+    assert seen == [[0, 620, 0], [0, 620, 0], [6000, 620, 0], [0, 620, 0]]
