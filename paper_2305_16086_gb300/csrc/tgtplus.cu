@@ -72,7 +72,6 @@ static void walks_t(sc_graph *g, const void *x, const int32_t *src, int nsrc, co
     a.nsrc = nsrc;
     a.tt = tt;
     a.walk_count = g->tp_walks.get();
-    a.g = nullptr;
     a.key0 = static_cast<uint32_t>(seed);
     a.key1 = static_cast<uint32_t>(seed >> 32);
     k_walk_chunks<T, B><<<ceil_div(max_chunks, 8), 256, 0, s>>>(static_cast<const T *>(x), a, c);

@@ -760,7 +760,6 @@ struct WalkArgs {
     const int32_t *row_ptr, *col, *src, *tau;
     int32_t n, nsrc, tt;
     const long long *walk_count;
-    double *g;             // unscaled half sums; the walk mean of X d_i is added
     uint32_t key0, key1;
 };
 
