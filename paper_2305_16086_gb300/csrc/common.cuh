@@ -231,12 +231,9 @@ struct sc_graph {
     int res_order_width[2] = {0, 0};
     int res_width = 0;
     bool res_ready = false;
-    // what a sample of its balls said, by (fp64, longest and mean run): the first class, and whether
-    // the class without the adjacency pays (-1: not asked)
-    struct ResChoice {
-        int first = 0, global = -1;
-    };
-    std::map<std::tuple<bool, int32_t, int32_t>, ResChoice> res_choice;
+    // what samples of its balls said, by (fp64, longest and mean run): the first class, and whether
+    // the class without the adjacency pays
+    std::map<std::tuple<bool, int32_t, int32_t>, int> res_first, res_global;
     // as a member of batches: (fp64, hops) of runs in which none of its sources ran resident
     std::set<std::pair<bool, int32_t>> res_batch_none;
     sc::DevBuf<unsigned char> res_scratch;

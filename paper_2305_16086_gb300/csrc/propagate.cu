@@ -1053,6 +1053,7 @@ struct Run {
     // statistics
     int64_t launches = 0, hops = 0, source_hops = 0, hop_launches = 0, walks = 0, graph_launches = 0, walk_steps = 0;
     int64_t resident_sources = 0;
+    int resident_global = -1;
     // per kernel class (SC_KC_*): event pairs (index into the graph's pool) and algorithmic bytes
     std::vector<std::pair<int, int64_t>> timed;
     int64_t event_pairs = 0;
@@ -1755,7 +1756,8 @@ static std::vector<int32_t> resident_blocks(Run &R, const std::vector<int32_t> &
                        const auto hi = std::upper_bound(seg_start.begin(), seg_start.end(), v);
                        const double share = beta < 0 ? 1.0 : window_share(*hi - *(hi - 1), beta, L, R.B);
                        return block_share_ns(g, *(hi - 1), *hi, L, R.prec == SC_PREC_FP64, share);
-                   }};
+                   },
+                   &R.resident_global};
     ResidentStats st;
     std::vector<int32_t> left = run_resident(rr, sources, len, seg_start, seg_take, seg_bip, &st);
     R.launches += st.launches;

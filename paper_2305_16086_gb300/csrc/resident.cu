@@ -649,25 +649,27 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
     const int32_t n = g->n;
     const bool fp64 = r.prec == SC_PREC_FP64;
     const int W = g->res_width;
-    std::vector<int32_t> left;
+    std::vector<int32_t> h_len(n, 0), left;
     int32_t longest = 0;
     int64_t total = 0, count = 0;
     for (int32_t v : sources) {
         const int32_t l = std::max(len[v] + r.extra, 0);
+        h_len[v] = l;
         longest = std::max(longest, l);
         total += l;
         count += l > 0;
     }
     const std::tuple<bool, int32_t, int32_t> key(fp64, longest, static_cast<int32_t>(total / std::max<int64_t>(count, 1)));
-    const auto known = g->res_choice.find(key);
-    if (known != g->res_choice.end() && known->second.first == kResClasses - 1 &&
-        (!seg_bip[0] || known->second.global == 0)) {  // none runs
+    auto kept = [&](const std::map<std::tuple<bool, int32_t, int32_t>, int> &m) {  // a graph's own, -1: not asked
+        const auto it = seg_start.size() == 2 ? m.find(key) : m.end();
+        return it == m.end() ? -1 : it->second;
+    };
+    const int kept_first = kept(g->res_first), kept_global = kept(g->res_global);
+    if (kept_first == kResClasses - 1 && (!seg_bip[0] || kept_global == 0)) {  // none runs
         for (int32_t v : sources)
-            if (len[v] + r.extra > 0) left.push_back(v);
+            if (h_len[v] > 0) left.push_back(v);
         return left;
     }
-    std::vector<int32_t> h_len(n, 0);
-    for (int32_t v : sources) h_len[v] = len[v] + r.extra;
     g->res_len.reserve(n);
     SC_CUDA(cudaMemcpyAsync(g->res_len.get(), h_len.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, s));
     if (!g->res_ready) {
@@ -745,9 +747,6 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
         // third of a short one (random 8-regular, 5,000 nodes, 7 hops: 0.84 ms, 0.60 without)
         int cls = 0;
         const bool keep = seg_start.size() == 2 && static_cast<int32_t>(list.size()) == ngroups;
-        sc_graph::ResChoice choice;
-        const bool kept = known != g->res_choice.end();
-        if (kept) choice = known->second;
         auto measure = [&](ResArgs m, int c, unsigned long long *h) {  // the balls of m's groups
             SC_CUDA(cudaMemsetAsync(g->res_count.get(), 0, kResCounts * sizeof(unsigned long long), s));
             m.count = g->res_count.get();
@@ -761,8 +760,8 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
         int32_t seg_max = 0;
         for (size_t i = 0; i + 1 < seg_start.size(); ++i)
             if (seg_take[i] && (seg_bip[i] != 0) == bip) seg_max = std::max(seg_max, seg_start[i + 1] - seg_start[i]);
-        if (kept) {
-            cls = choice.first;
+        if (kept_first >= 0) {
+            cls = kept_first;
         } else if (seg_max + width > cap_of(0)) {
             std::vector<int32_t> pick;
             const int32_t ns = std::min<int32_t>(kResSample, a.ngroups);
@@ -777,8 +776,7 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
             // no ball of the sample fits with its adjacency
             if (h[kResOver] == static_cast<unsigned long long>(ns)) cls = kResClasses - 1;
         }
-        choice.first = cls;
-        if (keep) g->res_choice[key] = choice;
+        if (keep) g->res_first[key] = cls;
         // groups of small segments need no more than the class that holds the segment, which leaves
         // room for more CTAs per SM: `list` starts with the smallest class in use, later classes get
         // their own groups and the ones that did not fit
@@ -836,17 +834,23 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
                 a.groups = nullptr;
                 a.ngroups = static_cast<int32_t>(single.size());
                 a.over = g->res_over.get();
-                size_t free_b = 0, total_b = 0;
-                SC_CUDA(cudaMemGetInfo(&free_b, &total_b));
-                a.ctas = global_class_ctas(marks_stride(n) * sizeof(uint16_t), single.size(), g->num_sms,
-                                           g->res_marks.count * sizeof(uint16_t), free_b);
+                const size_t marks = marks_stride(n) * sizeof(uint16_t), held = g->res_marks.count * sizeof(uint16_t);
+                a.ctas = global_class_ctas(marks, single.size(), g->num_sms, held, 0);
+                if (a.ctas == 0) {
+                    size_t free_b = 0, total_b = 0;
+                    SC_CUDA(cudaMemGetInfo(&free_b, &total_b));
+                    a.ctas = global_class_ctas(marks, single.size(), g->num_sms, held, free_b);
+                }
                 if (a.ctas == 0) {  // (2 bytes a node and SM: 14 million nodes in 4 GB)
                     left.insert(left.end(), single.begin(), single.end());
                     list.clear();
                     break;
                 }
                 const int32_t ns = kResSample;
-                if (choice.global < 0 && a.ngroups > ns) {  // fewer run in one wave, as soon as measured
+                // few sources run about as soon as measured, and a call's later runs (the same sources at
+                // longer lengths, in which this class does better) take the first one's answer
+                int pays = kept_global >= 0 ? kept_global : *r.global;
+                if (pays < 0 && a.ngroups > 4 * ns) {
                     std::vector<int32_t> pick;
                     double blocks_ns = 0.0, hops = 0.0;
                     for (int32_t q = 0; q < ns; ++q) {
@@ -862,11 +866,12 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
                     unsigned long long h[kResCounts];
                     measure(m, cls, h);
                     const int32_t cap_rows = fp64 ? res_global_rows<double>(W) : res_global_rows<float>(W);
-                    choice.global = global_class_pays(h, ns, hops, blocks_ns, W, static_cast<double>(g->nnz) / n,
-                                                      cap_rows, g->num_sms > 0 ? g->num_sms : 148);
-                    if (keep) g->res_choice[key] = choice;
+                    pays = global_class_pays(h, ns, hops, blocks_ns, W, static_cast<double>(g->nnz) / n, cap_rows,
+                                             g->num_sms > 0 ? g->num_sms : 148);
+                    if (seg_start.size() == 2) g->res_global[key] = pays;
+                    *r.global = pays;
                 }
-                if (choice.global == 0) {
+                if (pays == 0) {
                     left.insert(left.end(), single.begin(), single.end());
                     list.clear();
                     break;

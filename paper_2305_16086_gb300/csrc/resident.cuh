@@ -17,6 +17,7 @@ struct ResidentRun {
     GatherRec rec;
     std::function<void(const std::function<void()> &)> timed;  // runs one traversal launch, with its events
     std::function<double(int32_t, int32_t)> block_ns;  // source, hops: its share of the blocks' time, estimated
+    int *global;  // whether the class without the adjacency pays, from one run of a call to the next (-1: not asked)
 };
 
 struct ResidentStats {
