@@ -30,8 +30,10 @@
 // load and a table insert, then a barrier) and of a hop (one barrier), which is
 // why several CTAs share an SM when the ball is small. Whole calls, windowed
 // blocks against this: 150 x 613 strip at 67 + 2 hops 94 -> 8.4 ms, 400 x 400
-// lattice at learned lengths (37 to 353 hops) 625 -> 29.6 ms, 24 mixed graphs with
-// lattices of 1,000 to 5,000 nodes at 1,003 hops 223 -> 73 ms.
+// lattice at learned lengths (37 to 353 hops) 625 -> 30 ms, 24 mixed graphs with
+// lattices of 1,000 to 5,000 nodes at 1,003 hops 223 -> 85 ms. On graphs whose balls
+// grow fast (expanders, trees) nothing fits within a few hops; what a sample of the
+// balls says decides which class, if any, runs (res_first, global_class_pays).
 #include <algorithm>
 #include <numeric>
 
@@ -817,7 +819,8 @@ std::vector<int32_t> run_resident(const ResidentRun &r, const std::vector<int32_
             if (list.empty()) continue;
             if (cls == kResClasses - 1) {
                 // one source to a group, adjacency in global memory: bipartite graphs only (one
-                // buffer, half the rows a hop; without that the block kernels are as fast)
+                // buffer, half the rows a hop; without that the block kernels are as fast), and only
+                // where it pays
                 if (!bip) break;
                 std::vector<int32_t> single;
                 for (int32_t q : list)
