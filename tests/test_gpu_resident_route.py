@@ -232,3 +232,27 @@ def test_batches_of_graphs_that_do_not_run_resident(cuda_lib):
         for G in Gs:
             G.close()
     assert seen == [[0, 620, 0], [0, 620, 0], [6000, 620, 0], [0, 620, 0]]
+
+
+@pytest.mark.parametrize("maker", [lambda: _regular(9000, 8, 1), lambda: _regular(6000, 4, 4)])
+@pytest.mark.parametrize("policy", ["learned", "per_edge", "global"])
+def test_lengths_by_policy(cuda_lib, maker, policy):
+    """Lengths that differ by source, the learned length's records and its
+    extension rounds through the resident form and its left-overs."""
+    from paper_2305_16086_gb300 import binding
+
+    g, t = maker(), gg.barabasi_albert(2500, 5, 21)
+    init = np.random.default_rng(3).normal(0, 0.2, binding.MLP_PARAMS).astype(np.float32)
+    with _graph(t) as Gt:
+        Gt.estimate_lambda()
+        model, _ = binding.mlp_train([Gt], init, epochs=60, lr=1e-2, eps=1e-3, precision="fp32")
+    with _graph(g) as G:
+        G.estimate_lambda()
+        binding.mlp_load(G, model)
+        for precision in ("fp32", "fp64"):
+            kw = dict(policy=policy, eps=1e-3, precision=precision)
+            s, b, rep = G.all_edges(record_tail=policy != "learned", **kw)
+            s0, b0, rep0 = G.all_edges(record_tail=policy != "learned", windows=False, **kw)
+            assert rep["extension_rounds"] == rep0["extension_rounds"]
+            assert rep["edges_extended"] == rep0["edges_extended"]
+            assert np.array_equal(s, s0) and (b is None or np.array_equal(b, b0))
