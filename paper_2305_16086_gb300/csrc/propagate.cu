@@ -1459,9 +1459,13 @@ static void run_blocks_win(Run &R, std::vector<int32_t> sources, const std::vect
     sources.erase(std::remove_if(sources.begin(), sources.end(), [&](int32_t v) { return len[v] + R.extra <= 0; }),
                   sources.end());
     if (sources.empty()) return;
-    auto seg_of = [&](int32_t v) {
-        return static_cast<int32_t>(std::upper_bound(seg_start.begin(), seg_start.end(), v) - seg_start.begin()) - 1;
-    };
+    // the segment of every source, looked up once: as a binary search within the comparisons of the sort
+    // below it took 8 to 9.4 ms for 80,000 sources of 24 graphs, by how the compiler laid it out (whole
+    // calls 72.7 to 74 ms, 66.5 so)
+    std::vector<int32_t> segment(g->n);
+    for (int32_t v : sources)
+        segment[v] = static_cast<int32_t>(std::upper_bound(seg_start.begin(), seg_start.end(), v) - seg_start.begin()) - 1;
+    auto seg_of = [&](int32_t v) { return segment[v]; };
     // colour (BFS depth parity) of the sources of bipartite segments, -1 elsewhere: blocks of one
     // colour compute half the rows per hop (SliceWin::parity)
     const bool any_bip = std::any_of(seg_bipartite.begin(), seg_bipartite.end(), [](char c) { return c != 0; });
